@@ -96,6 +96,8 @@ __global__ void __launch_bounds__(kBlkThreads) k_block_pi(BlockArgs a, GridSync 
     __shared__ double s_sum[PMAX];                // reduced sums of the current block
     __shared__ double s_A[KM * KM], s_Ri[KM * KM], s_mu[KM];
     __shared__ int s_flag[2];
+    __shared__ GridBar s_bar;
+    if (threadIdx.x == 0) grid_bar_init(&s_bar, gs);
     // dynamic: per warp the y_new and x_cur of 32 rows ([NW][32][2k]), then
     // the per-warp partial sums ([NW][P])
     extern __shared__ __align__(16) double s_dyn[];
@@ -153,7 +155,7 @@ __global__ void __launch_bounds__(kBlkThreads) k_block_pi(BlockArgs a, GridSync 
         }
     };
     publish(0);
-    if (!grid_sync(gs)) return;
+    if (!grid_sync(&s_bar)) return;
 
     for (int t = 0;; t++) {
         // ---- sums of Y_t over all CTAs (same order in every CTA)
@@ -282,7 +284,7 @@ __global__ void __launch_bounds__(kBlkThreads) k_block_pi(BlockArgs a, GridSync 
         }
         __syncthreads();
         publish((t + 1) & 1);
-        if (!grid_sync(gs)) return;
+        if (!grid_sync(&s_bar)) return;
     }
 }
 

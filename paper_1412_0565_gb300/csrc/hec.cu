@@ -235,6 +235,8 @@ __device__ __forceinline__ bool is_creator(const HecArgs &a, int u) {
 __global__ void k_hec_resolve(HecArgs a, GridSync *gs) {
     __shared__ int sm_scan[32];
     __shared__ int sm_red[32];
+    __shared__ GridBar s_bar;
+    if (threadIdx.x == 0) grid_bar_init(&s_bar, gs);
     const int n = a.n;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int nth = gridDim.x * blockDim.x;
@@ -244,7 +246,7 @@ __global__ void k_hec_resolve(HecArgs a, GridSync *gs) {
         a.minA[v] = kInf;
         a.minU[v] = kInf;
     }
-    if (!grid_sync(gs)) return;
+    if (!grid_sync(&s_bar)) return;
 
     int rounds = 0;
     for (int round = 0; round < a.max_rounds; round++) {
@@ -259,7 +261,7 @@ __global__ void k_hec_resolve(HecArgs a, GridSync *gs) {
             if (s == kActive) atomicMin(&a.minA[mv], a.r[v]);
             else if (s == kUndecided) atomicMin(&a.minU[mv], a.r[v]);
         }
-        if (!grid_sync(gs)) return;
+        if (!grid_sync(&s_bar)) return;
         // decide
         int und = 0;
         for (int v = tid; v < n; v += nth) {
@@ -280,21 +282,21 @@ __global__ void k_hec_resolve(HecArgs a, GridSync *gs) {
             for (int i = 0; i < (int)(blockDim.x + 31) / 32; i++) t += sm_red[i];
             if (t) atomicAdd(&a.undecided[round % 3], t);
         }
-        if (!grid_sync(gs)) return;
+        if (!grid_sync(&s_bar)) return;
         if (*((volatile int *)&a.undecided[round % 3]) == 0) break;
     }
 
     // minA over all active in-neighbours
     for (int v = tid; v < n; v += nth) a.minA[v] = kInf;
-    if (!grid_sync(gs)) return;
+    if (!grid_sync(&s_bar)) return;
     for (int v = tid; v < n; v += nth) {
         const int mv = a.m[v];
         if (mv >= 0 && a.state[v] == kActive) atomicMin(&a.minA[mv], a.r[v]);
     }
-    if (!grid_sync(gs)) return;
+    if (!grid_sync(&s_bar)) return;
     // creator flags, indexed by rank
     for (int v = tid; v < n; v += nth) a.ids[a.r[v]] = is_creator(a, v) ? 1 : 0;
-    if (!grid_sync(gs)) return;
+    if (!grid_sync(&s_bar)) return;
 
     // exclusive scan of the flags in rank order: contiguous chunk per CTA
     const int chunk = (n + gridDim.x - 1) / gridDim.x;
@@ -309,7 +311,7 @@ __global__ void k_hec_resolve(HecArgs a, GridSync *gs) {
         for (int i = 0; i < (int)(blockDim.x + 31) / 32; i++) t += sm_red[i];
         a.cta_tot[blockIdx.x] = t;
     }
-    if (!grid_sync(gs)) return;
+    if (!grid_sync(&s_bar)) return;
     __shared__ int s_base;
     if (threadIdx.x == 0) {
         int b = 0;
@@ -330,7 +332,7 @@ __global__ void k_hec_resolve(HecArgs a, GridSync *gs) {
         if (i < hi) a.ids[i] = run + ex;
         run += tot;
     }
-    if (!grid_sync(gs)) return;
+    if (!grid_sync(&s_bar)) return;
 
     // labels
     for (int v = tid; v < n; v += nth) {

@@ -93,6 +93,14 @@ constexpr int kTileCost = 3840;                   // entries + 4 * rows per tile
 constexpr int kSmallMaxThreads = 1024;
 constexpr int kFinThreads = 256;
 
+// Stop sums of one CTA as stored for the other CTAs' control warps: two
+// 16-byte words, so that a lane fetches a record with two loads.
+struct __align__(16) PartRec {
+    float4 ab;   // A.hi, A.lo, B.hi, B.lo
+    float4 c;    // C.hi, C.lo
+};
+constexpr int kPartDoubles = (int)(sizeof(PartRec) / sizeof(double));
+
 struct PiArgs {
     int n;
     const int *rp;
@@ -116,7 +124,7 @@ struct PiArgs {
     void *buf[3];           // iterate ring
     double *gd;             // FP64 form: g - d_i
     PiResult *res;
-    ff *partials;           // [2][gridDim.x][3] (tiled kernel)
+    PartRec *partials;      // [2][gridDim.x]: the CTAs' stop sums, by sweep parity
     float zero_tol2;        // (64 eps)^2 of the sweep precision
     long long sell_nnz;     // SELL-32 size of the level (0: unknown)
     const int *cinvp;       // coarse level's layout order (start = 1), or nullptr
@@ -144,6 +152,42 @@ struct PiArgs {
     int cl_emax;            // cluster kernel: SELL-32 entries each CTA holds (at most)
 };
 
+
+__device__ __forceinline__ void store_part(PartRec *dst, const Part &q) {
+    dst->ab = make_float4(q.A.hi, q.A.lo, q.B.hi, q.B.lo);
+    dst->c = make_float4(q.C.hi, q.C.lo, 0.f, 0.f);
+}
+
+// Sum of the gridDim.x records at src by one warp: lane l takes records l,
+// l + 32, ... in order, then the lanes' tree.  Five records per lane are
+// fetched before the first is added: what bounds the control warp on levels
+// whose rows take less than it is the number of dependent trips to L2 (two
+// here for 304 CTAs; ten with a fetch per addition, 3.7 us).
+__device__ __forceinline__ Part grid_part(const PartRec *src, int lane) {
+    Part q = part_zero();
+    const int nb = (int)gridDim.x;
+    for (int b0 = lane; b0 < nb; b0 += 32 * 5) {
+        float4 ab[5], c[5];
+#pragma unroll
+        for (int u = 0; u < 5; u++) {
+            ab[u] = c[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (b0 + 32 * u < nb) {
+                ab[u] = __ldcg(&src[b0 + 32 * u].ab);
+                c[u] = __ldcg(&src[b0 + 32 * u].c);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 5; u++) {
+            if (b0 + 32 * u >= nb) continue;
+            Part t;
+            t.A = ff_make(ab[u].x, ab[u].y);
+            t.B = ff_make(ab[u].z, ab[u].w);
+            t.C = ff_make(c[u].x, c[u].y);
+            q = part_add(q, t);
+        }
+    }
+    return warp_sum_part(q);
+}
 
 // Start value of row i: Gaussian (Alg. 1 Step 2), prolongation (I^T y of
 // Alg. 1 Step 3) of the coarse result, or an explicit vector.
@@ -181,8 +225,11 @@ struct Slot {
     int pad;
 };
 
-// fp64: also form the doubles (the FP32 kernels leave them unused)
-__device__ __forceinline__ Slot slot_make(ff m, int e, double g, bool fp64) {
+// fp64: also form the doubles (the FP32 kernels leave them unused); inv_g is
+// 1 / g, divided once per launch (an FP64 division is a chain of about ten
+// dependent FP64 instructions, and the scaling exponent is 0 in nearly every
+// sweep)
+__device__ __forceinline__ Slot slot_make(ff m, int e, double g, double inv_g, bool fp64) {
     Slot sl;
     sl.m = m;
     sl.e = e;
@@ -192,7 +239,7 @@ __device__ __forceinline__ Slot slot_make(ff m, int e, double g, bool fp64) {
     sl.m_d = sl.sig_d = sl.gm_d = 0.0;
     if (fp64) {
         sl.m_d = ff_to_double(m);
-        sl.sig_d = ldexp(1.0 / g, e);
+        sl.sig_d = e ? ldexp(inv_g, e) : inv_g;
         sl.gm_d = g * sl.m_d;
     }
     return sl;
@@ -205,6 +252,7 @@ struct Ctl {
     ff m_cur;              // m_s: used by sweep s+1
     ff inv_n, omt2;        // 1/n and (1 - tol)^2
     int e_cur, e_prev;     // e_s, e_{s-1}
+    double inv_g;          // 1/g
     // result of the decision (valid once `stopped`)
     int stopped, zero, res_sweep, capped;
     double mu_res, ss_res, mu_res_prev, ss_res_prev, cos_res;
@@ -223,7 +271,7 @@ __device__ __forceinline__ void ctrl_step(const PiArgs &a, int s, const Part &P,
     const ff ss = ff_add_f(P.B, -nf * mu.hi * mu.hi);
     const ff cs = ff_add_f(P.C, -nf * mu.hi * c.mu_prev.hi);
     // annihilated: ||proj y_s|| <= 64 eps 2^{e_{s-1}} ||proj y_{s-1}||
-    const bool zero = ss.hi <= a.zero_tol2 * ldexpf(c.ss_prev.hi, 2 * c.e_prev);
+    const bool zero = ss.hi <= a.zero_tol2 * (c.e_prev ? ldexpf(c.ss_prev.hi, 2 * c.e_prev) : c.ss_prev.hi);
     // cos_s >= 1 - tol  <=>  cs > 0 and cs^2 >= (1 - tol)^2 ss_s ss_{s-1}
     const bool conv = cs.hi > 0.f && !ff_lt(ff_mul(cs, cs), ff_mul(ff_mul(ss, c.ss_prev), c.omt2));
     bool stop = zero;
@@ -249,15 +297,16 @@ __device__ __forceinline__ void ctrl_step(const PiArgs &a, int s, const Part &P,
     }
     // parameters of sweep s+2 (exact power-of-two scaling of mu_s - m_s)
     const ff dm = ff_sub(mu, c.m_cur);
-    const ff m_next = ff_make(ldexpf(dm.hi, c.e_cur), ldexpf(dm.lo, c.e_cur));
+    const ff m_next = c.e_cur ? ff_make(ldexpf(dm.hi, c.e_cur), ldexpf(dm.lo, c.e_cur)) : dm;
     int e_next = 0;
-    {
+    // (1e-14 is above 2^-48: without a pending rescale no new one is due)
+    if (c.e_cur != 0 || ss.hi <= 1e-14f) {
         // predicted log2 ||y_{s+1}|| <= log2 ||y_s|| + e_s; lift it back to ~1
         const float l2 = 0.5f * log2f(fmaxf(ss.hi, 1e-37f)) + (float)c.e_cur;
         if (l2 < -24.f) e_next = (int)(-l2);
     }
     if (next) {
-        *next = slot_make(m_next, e_next, a.g, fp64);
+        *next = slot_make(m_next, e_next, a.g, c.inv_g, fp64);
         next->stop = stop ? 1 : 0;
         next->zero = zero ? 1 : 0;
     }
@@ -273,6 +322,7 @@ __device__ __forceinline__ void ctl_init(Ctl &c, const PiArgs &a, double mu0, do
     c.ss_prev = ff_from_double(ss0);
     c.m_cur = ff_zero();   // m_1: the start was projected exactly
     c.inv_n = ff_from_double(1.0 / (double)a.n);
+    c.inv_g = 1.0 / a.g;
     const double omt = 1.0 - a.tol;
     c.omt2 = ff_from_double(omt * omt);
     c.e_cur = 0;
@@ -346,6 +396,8 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_power_tiled(PiArgs a, GridS
     unsigned short *s_row = reinterpret_cast<unsigned short *>(s_rp + kTileRows + 4);  // kChunk
     __shared__ Part s_pw[kTileThreads / 32];
     __shared__ Slot s_slot[2];
+    __shared__ GridBar s_bar;
+    if (threadIdx.x == 0) grid_bar_init(&s_bar, gs);
 
     const int n = a.n;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -390,34 +442,22 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_power_tiled(PiArgs a, GridS
             Part q = (lane < (int)(blockDim.x >> 5)) ? s_pw[lane] : part_zero();
             q = warp_sum_part(q);
             if (lane == 0) {
-                ff *dst = a.partials + (size_t)blockIdx.x * 3;
-                dst[0] = q.A;
-                dst[1] = q.B;
-                dst[2] = q.C;
+                store_part(a.partials + blockIdx.x, q);
             }
         }
     }
-    if (!grid_sync(gs)) return;
-    Ctl c;
+    if (!grid_sync(&s_bar)) return;
+    __shared__ Ctl c;   // used by lane 0 of the control warp (in registers it would take every row thread's)
     if (warp == 0) {
-        Part q = part_zero();
-        for (int b = lane; b < (int)gridDim.x; b += 32) {
-            const ff *src = a.partials + (size_t)b * 3;
-            Part t;
-            t.A = ff_make(LDX(&src[0].hi), LDX(&src[0].lo));
-            t.B = ff_make(LDX(&src[1].hi), LDX(&src[1].lo));
-            t.C = ff_zero();
-            q = part_add(q, t);
-        }
-        q = warp_sum_part(q);
+        const Part q = grid_part(a.partials, lane);
         const double mu0 = to_d(q.A) / (double)n;
         double ss0 = to_d(q.B) - (double)n * mu0 * mu0;
         if (ss0 < 0.0) ss0 = 0.0;
         const int e0 = start_exponent(ss0);
-        ctl_init(c, a, mu0, ss0, e0);
         if (lane == 0) {
-            s_slot[1] = slot_make(ff_from_double(mu0), e0, a.g, fp64);  // sweep 1: exact mean of y_0
-            s_slot[0] = slot_make(ff_zero(), 0, a.g, fp64);             // sweep 2: m_1 = 0
+            ctl_init(c, a, mu0, ss0, e0);
+            s_slot[1] = slot_make(ff_from_double(mu0), e0, a.g, c.inv_g, fp64);  // sweep 1: exact mean of y_0
+            s_slot[0] = slot_make(ff_zero(), 0, a.g, c.inv_g, fp64);             // sweep 2: m_1 = 0
         }
     }
     __syncthreads();
@@ -440,20 +480,8 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_power_tiled(PiArgs a, GridS
         if (warp == 0) {
             // ---- control: reduce sweep s over all CTAs, decide, plan sweep s+2
             if (s >= 1) {
-                Part q = part_zero();
-                const ff *base = a.partials + (size_t)(s & 1) * gridDim.x * 3;
-                for (int b = lane; b < (int)gridDim.x; b += 32) {
-                    const ff *src = base + (size_t)b * 3;
-                    Part t;
-                    t.A = ff_make(LDX(&src[0].hi), LDX(&src[0].lo));
-                    t.B = ff_make(LDX(&src[1].hi), LDX(&src[1].lo));
-                    t.C = ff_make(LDX(&src[2].hi), LDX(&src[2].lo));
-                    q = part_add(q, t);
-                }
-                q = warp_sum_part(q);
-                Slot nx;
-                ctrl_step(a, s, q, c, &nx, false, fp64);
-                if (lane == 0) s_slot[s & 1] = nx;
+                const Part q = grid_part(a.partials + (size_t)(s & 1) * gridDim.x, lane);
+                if (lane == 0) ctrl_step(a, s, q, c, &s_slot[s & 1], false, fp64);
             }
         } else {
             // ---- rows of sweep s+1
@@ -556,31 +584,22 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_power_tiled(PiArgs a, GridS
             Part q = (lane >= 1 && lane < (int)(blockDim.x >> 5)) ? s_pw[lane] : part_zero();
             q = warp_sum_part(q);
             if (lane == 0) {
-                ff *dst = a.partials + ((size_t)((s + 1) & 1) * gridDim.x + blockIdx.x) * 3;
-                dst[0] = q.A;
-                dst[1] = q.B;
-                dst[2] = q.C;
+                // the CTA's rows were stored before the CTA barrier above, so
+                // thread 0 can arrive for the CTA at once
+                store_part(a.partials + (size_t)((s + 1) & 1) * gridDim.x + blockIdx.x, q);
+                s_bar.ok = grid_arrive_wait(&s_bar);
             }
         }
-        if (!grid_sync(gs)) return;
+        __syncthreads();
+        if (!s_bar.ok) return;
         s++;
     }
     // ---------------------------------------------------------- result
     if (warp == 0) {
         if (exit_kind == 2 && !no_sweeps) {
             // the last sweep s ended the loop by count: reduce it now
-            Part q = part_zero();
-            const ff *base = a.partials + (size_t)(s & 1) * gridDim.x * 3;
-            for (int b = lane; b < (int)gridDim.x; b += 32) {
-                const ff *src = base + (size_t)b * 3;
-                Part t;
-                t.A = ff_make(LDX(&src[0].hi), LDX(&src[0].lo));
-                t.B = ff_make(LDX(&src[1].hi), LDX(&src[1].lo));
-                t.C = ff_make(LDX(&src[2].hi), LDX(&src[2].lo));
-                q = part_add(q, t);
-            }
-            q = warp_sum_part(q);
-            ctrl_step(a, s, q, c, nullptr, true, fp64);
+            const Part q = grid_part(a.partials + (size_t)(s & 1) * gridDim.x, lane);
+            if (lane == 0) ctrl_step(a, s, q, c, nullptr, true, fp64);
         }
         if (blockIdx.x == 0 && lane == 0) {
             const int rs = c.res_sweep;
@@ -612,6 +631,8 @@ __global__ void __launch_bounds__(STAGE ? kStageThreads : kTileThreads, STAGE ? 
     T *const s_x = reinterpret_cast<T *>(smem_raw);
     __shared__ Part s_pw[kStageThreads / 32];
     __shared__ Slot s_slot[2];
+    __shared__ GridBar s_bar;
+    if (threadIdx.x == 0) grid_bar_init(&s_bar, gs);
     const int n = a.n;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     T *const ring0 = (T *)a.buf[0], *const ring1 = (T *)a.buf[1], *const ring2 = (T *)a.buf[2];
@@ -674,34 +695,22 @@ __global__ void __launch_bounds__(STAGE ? kStageThreads : kTileThreads, STAGE ? 
             Part q = (lane < (int)(blockDim.x >> 5)) ? s_pw[lane] : part_zero();
             q = warp_sum_part(q);
             if (lane == 0) {
-                ff *dst = a.partials + (size_t)blockIdx.x * 3;
-                dst[0] = q.A;
-                dst[1] = q.B;
-                dst[2] = q.C;
+                store_part(a.partials + blockIdx.x, q);
             }
         }
     }
-    if (!grid_sync(gs)) return;
-    Ctl c;
+    if (!grid_sync(&s_bar)) return;
+    __shared__ Ctl c;   // used by lane 0 of the control warp (in registers it would take every row thread's)
     if (warp == 0) {
-        Part q = part_zero();
-        for (int b = lane; b < (int)gridDim.x; b += 32) {
-            const ff *src = a.partials + (size_t)b * 3;
-            Part t;
-            t.A = ff_make(LDX(&src[0].hi), LDX(&src[0].lo));
-            t.B = ff_make(LDX(&src[1].hi), LDX(&src[1].lo));
-            t.C = ff_zero();
-            q = part_add(q, t);
-        }
-        q = warp_sum_part(q);
+        const Part q = grid_part(a.partials, lane);
         const double mu0 = to_d(q.A) / (double)n;
         double ss0 = to_d(q.B) - (double)n * mu0 * mu0;
         if (ss0 < 0.0) ss0 = 0.0;
         const int e0 = start_exponent(ss0);
-        ctl_init(c, a, mu0, ss0, e0);
         if (lane == 0) {
-            s_slot[1] = slot_make(ff_from_double(mu0), e0, a.g, fp64);
-            s_slot[0] = slot_make(ff_zero(), 0, a.g, fp64);
+            ctl_init(c, a, mu0, ss0, e0);
+            s_slot[1] = slot_make(ff_from_double(mu0), e0, a.g, c.inv_g, fp64);
+            s_slot[0] = slot_make(ff_zero(), 0, a.g, c.inv_g, fp64);
         }
     }
     __syncthreads();
@@ -727,20 +736,8 @@ __global__ void __launch_bounds__(STAGE ? kStageThreads : kTileThreads, STAGE ? 
         T *y = pick3<T *>(ring0, ring1, ring2, (s + 1) % 3);
         if (warp == 0) {
             if (s >= 1) {
-                Part q = part_zero();
-                const ff *base = a.partials + (size_t)(s & 1) * gridDim.x * 3;
-                for (int b = lane; b < (int)gridDim.x; b += 32) {
-                    const ff *src = base + (size_t)b * 3;
-                    Part t;
-                    t.A = ff_make(LDX(&src[0].hi), LDX(&src[0].lo));
-                    t.B = ff_make(LDX(&src[1].hi), LDX(&src[1].lo));
-                    t.C = ff_make(LDX(&src[2].hi), LDX(&src[2].lo));
-                    q = part_add(q, t);
-                }
-                q = warp_sum_part(q);
-                Slot nx;
-                ctrl_step(a, s, q, c, &nx, false, fp64);
-                if (lane == 0) s_slot[s & 1] = nx;
+                const Part q = grid_part(a.partials + (size_t)(s & 1) * gridDim.x, lane);
+                if (lane == 0) ctrl_step(a, s, q, c, &s_slot[s & 1], false, fp64);
             }
         } else {
             const T m = fp64 ? (T)sl.m_d : (T)sl.m.hi;
@@ -809,6 +806,7 @@ __global__ void __launch_bounds__(STAGE ? kStageThreads : kTileThreads, STAGE ? 
                                     t0 = t;
                                 } else if (t - t0 > kBarrierTimeoutNs || ld_relaxed_gpu(&gs->err)) {
                                     atomicExch(&gs->err, 1u);
+                                    s_bar.err = 1;   // the CTA leaves at its next barrier
                                     break;
                                 }
                             }
@@ -836,30 +834,21 @@ __global__ void __launch_bounds__(STAGE ? kStageThreads : kTileThreads, STAGE ? 
             Part q = (lane >= 1 && lane < (int)(blockDim.x >> 5)) ? s_pw[lane] : part_zero();
             q = warp_sum_part(q);
             if (lane == 0) {
-                ff *dst = a.partials + ((size_t)((s + 1) & 1) * gridDim.x + blockIdx.x) * 3;
-                dst[0] = q.A;
-                dst[1] = q.B;
-                dst[2] = q.C;
+                // the CTA's rows were stored before the CTA barrier above, so
+                // thread 0 can arrive for the CTA at once
+                store_part(a.partials + (size_t)((s + 1) & 1) * gridDim.x + blockIdx.x, q);
+                s_bar.ok = grid_arrive_wait(&s_bar);
             }
         }
-        if (!grid_sync(gs)) return;
+        __syncthreads();
+        if (!s_bar.ok) return;
         s++;
     }
     // ---------------------------------------------------------- result
     if (warp == 0) {
         if (exit_kind == 2 && !no_sweeps) {
-            Part q = part_zero();
-            const ff *base = a.partials + (size_t)(s & 1) * gridDim.x * 3;
-            for (int b = lane; b < (int)gridDim.x; b += 32) {
-                const ff *src = base + (size_t)b * 3;
-                Part t;
-                t.A = ff_make(LDX(&src[0].hi), LDX(&src[0].lo));
-                t.B = ff_make(LDX(&src[1].hi), LDX(&src[1].lo));
-                t.C = ff_make(LDX(&src[2].hi), LDX(&src[2].lo));
-                q = part_add(q, t);
-            }
-            q = warp_sum_part(q);
-            ctrl_step(a, s, q, c, nullptr, true, fp64);
+            const Part q = grid_part(a.partials + (size_t)(s & 1) * gridDim.x, lane);
+            if (lane == 0) ctrl_step(a, s, q, c, nullptr, true, fp64);
         }
         if (blockIdx.x == 0 && lane == 0) {
             const int rs = c.res_sweep;
@@ -922,6 +911,8 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_power_2p(PiArgs a, GridSyn
     __shared__ Part s_pw[kStageThreads / 32];
     __shared__ double s_mx[kStageThreads / 32];
     __shared__ Slot s_slot[2];
+    __shared__ GridBar s_bar;
+    if (threadIdx.x == 0) grid_bar_init(&s_bar, gs);
     __shared__ int s_sc;
     __shared__ Ctl s_ctl;   // the control warp's state (kept out of every thread's registers)
     const int n = a.n;
@@ -986,26 +977,14 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_power_2p(PiArgs a, GridSyn
             Part q = (lane < (int)(blockDim.x >> 5)) ? s_pw[lane] : part_zero();
             q = warp_sum_part(q);
             if (lane == 0) {
-                ff *dst = a.partials + (size_t)blockIdx.x * 3;
-                dst[0] = q.A;
-                dst[1] = q.B;
-                dst[2] = q.C;
+                store_part(a.partials + blockIdx.x, q);
             }
         }
     }
-    if (!grid_sync(gs)) return;
+    if (!grid_sync(&s_bar)) return;
     if (warp == 0) {
         Ctl c;
-        Part q = part_zero();
-        for (int k = lane; k < P; k += 32) {
-            const ff *src = a.partials + (size_t)k * 3;
-            Part t;
-            t.A = ff_make(LDX(&src[0].hi), LDX(&src[0].lo));
-            t.B = ff_make(LDX(&src[1].hi), LDX(&src[1].lo));
-            t.C = ff_zero();
-            q = part_add(q, t);
-        }
-        q = warp_sum_part(q);
+        const Part q = grid_part(a.partials, lane);
         const double xmax = grid_max(a.x_pmax);
         const double mu0 = to_d(q.A) / (double)n;
         double ss0 = to_d(q.B) - (double)n * mu0 * mu0;
@@ -1014,8 +993,8 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_power_2p(PiArgs a, GridSyn
         ctl_init(c, a, mu0, ss0, e0);
         if (lane == 0) {
             s_ctl = c;
-            s_slot[1] = slot_make(ff_from_double(mu0), e0, a.g, fp64);
-            s_slot[0] = slot_make(ff_zero(), 0, a.g, fp64);
+            s_slot[1] = slot_make(ff_from_double(mu0), e0, a.g, c.inv_g, fp64);
+            s_slot[0] = slot_make(ff_zero(), 0, a.g, c.inv_g, fp64);
             s_sc = fix_scale(a.g, xmax);
         }
     }
@@ -1039,17 +1018,7 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_power_2p(PiArgs a, GridSyn
         if (warp == 0 && s >= 1) {
             // decisions of sweep s-1 and the fixed-point scale of sweep s,
             // overlapped with phase 1 of pass 0 (published by its barrier)
-            Part q = part_zero();
-            const ff *base = a.partials + (size_t)(s & 1) * P * 3;
-            for (int k = lane; k < P; k += 32) {
-                const ff *src = base + (size_t)k * 3;
-                Part t;
-                t.A = ff_make(LDX(&src[0].hi), LDX(&src[0].lo));
-                t.B = ff_make(LDX(&src[1].hi), LDX(&src[1].lo));
-                t.C = ff_make(LDX(&src[2].hi), LDX(&src[2].lo));
-                q = part_add(q, t);
-            }
-            q = warp_sum_part(q);
+            const Part q = grid_part(a.partials + (size_t)(s & 1) * P, lane);
             Slot nx;
             Ctl c = s_ctl;
             ctrl_step(a, s, q, c, &nx, false, fp64);
@@ -1142,7 +1111,7 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_power_2p(PiArgs a, GridSyn
                 }
             }
             X2T(s, t, 2);
-            if (!grid_sync(gs)) return;
+            if (!grid_sync(&s_bar)) return;
             X2T(s, t, 3);
             if (warp > 0) {
                 // ------------------------------------------------ phase 2
@@ -1234,31 +1203,18 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_power_2p(PiArgs a, GridSyn
             Part q = (lane >= 1 && lane < (int)(blockDim.x >> 5)) ? s_pw[lane] : part_zero();
             q = warp_sum_part(q);
             if (lane == 0) {
-                ff *dst = a.partials + ((size_t)((s + 1) & 1) * P + blockIdx.x) * 3;
-                dst[0] = q.A;
-                dst[1] = q.B;
-                dst[2] = q.C;
+                store_part(a.partials + (size_t)((s + 1) & 1) * P + blockIdx.x, q);
             }
         }
-        if (!grid_sync(gs)) return;
+        if (!grid_sync(&s_bar)) return;
         s++;
     }
     // ---------------------------------------------------------- result
     if (warp == 0) {
         Ctl c = s_ctl;
         if (exit_kind == 2 && !no_sweeps) {
-            Part q = part_zero();
-            const ff *base = a.partials + (size_t)(s & 1) * P * 3;
-            for (int k = lane; k < P; k += 32) {
-                const ff *src = base + (size_t)k * 3;
-                Part t;
-                t.A = ff_make(LDX(&src[0].hi), LDX(&src[0].lo));
-                t.B = ff_make(LDX(&src[1].hi), LDX(&src[1].lo));
-                t.C = ff_make(LDX(&src[2].hi), LDX(&src[2].lo));
-                q = part_add(q, t);
-            }
-            q = warp_sum_part(q);
-            ctrl_step(a, s, q, c, nullptr, true, fp64);
+            const Part q = grid_part(a.partials + (size_t)(s & 1) * P, lane);
+            if (lane == 0) ctrl_step(a, s, q, c, nullptr, true, fp64);
         }
         if (blockIdx.x == 0 && lane == 0) {
             const int rs = c.res_sweep;
@@ -1549,7 +1505,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_power_small(PiArgs a, Grid
         if (lane == 0) s_pw[0][warp] = p;
     }
     __syncthreads();
-    Ctl c;
+    __shared__ Ctl c;   // used by lane 0 of the control warp (in registers it would take every row thread's)
     if (warp == 0) {
         Part q = (lane < nw) ? s_pw[0][lane] : part_zero();
         q = warp_sum_part(q);
@@ -1557,10 +1513,10 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_power_small(PiArgs a, Grid
         double ss0 = to_d(q.B) - (double)n * mu0 * mu0;
         if (ss0 < 0.0) ss0 = 0.0;
         const int e0 = start_exponent(ss0);
-        ctl_init(c, a, mu0, ss0, e0);
         if (lane == 0) {
-            s_slot[1] = slot_make(ff_from_double(mu0), e0, a.g, fp64);
-            s_slot[0] = slot_make(ff_zero(), 0, a.g, fp64);
+            ctl_init(c, a, mu0, ss0, e0);
+            s_slot[1] = slot_make(ff_from_double(mu0), e0, a.g, c.inv_g, fp64);
+            s_slot[0] = slot_make(ff_zero(), 0, a.g, c.inv_g, fp64);
         }
     }
     __syncthreads();
@@ -1587,9 +1543,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_power_small(PiArgs a, Grid
             if (lane == 0) TRACE(s, 0);
             if (s >= 1) {
                 const Part q = ctl_part(s & 1);
-                Slot nx;
-                ctrl_step(a, s, q, c, &nx, false, fp64);
-                if (lane == 0) s_slot[s & 1] = nx;
+                if (lane == 0) ctrl_step(a, s, q, c, &s_slot[s & 1], false, fp64);
             }
             if (lane == 0) TRACE(s, 1);
         } else {
@@ -1690,7 +1644,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_power_small(PiArgs a, Grid
     if (warp == 0) {
         if (exit_kind == 2 && !no_sweeps) {
             const Part q = ctl_part(s & 1);
-            ctrl_step(a, s, q, c, nullptr, true, fp64);
+            if (lane == 0) ctrl_step(a, s, q, c, nullptr, true, fp64);
         }
         if (lane == 0) {
             const int rs = c.res_sweep;
@@ -1862,7 +1816,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_power_cluster(PiArgs a, Gr
         if (lane == 0) s_pw[warp] = p;
     }
     __syncthreads();
-    Ctl c;
+    __shared__ Ctl c;   // used by lane 0 of the control warp (in registers it would take every row thread's)
     if (warp == 0) {
         Part q = (lane < nw) ? s_pw[lane] : part_zero();
         q = warp_sum_part(q);
@@ -1870,10 +1824,10 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_power_cluster(PiArgs a, Gr
         double ss0 = to_d(q.B) - (double)n * mu0 * mu0;
         if (ss0 < 0.0) ss0 = 0.0;
         const int e0 = start_exponent(ss0);
-        ctl_init(c, a, mu0, ss0, e0);
         if (lane == 0) {
-            s_slot[1] = slot_make(ff_from_double(mu0), e0, a.g, true);
-            s_slot[0] = slot_make(ff_zero(), 0, a.g, true);
+            ctl_init(c, a, mu0, ss0, e0);
+            s_slot[1] = slot_make(ff_from_double(mu0), e0, a.g, c.inv_g, true);
+            s_slot[0] = slot_make(ff_zero(), 0, a.g, c.inv_g, true);
         }
     }
     __syncthreads();
@@ -1908,9 +1862,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_power_cluster(PiArgs a, Gr
         if (warp == 0) {
             if (s >= 1) {
                 const Part q = cluster_part((s - 1) & 1);
-                Slot nx;
-                ctrl_step(a, s, q, c, &nx, false, true);
-                if (lane == 0) s_slot[s & 1] = nx;
+                if (lane == 0) ctrl_step(a, s, q, c, &s_slot[s & 1], false, true);
             }
         } else {
             const double mT = sl.m_d, sig = sl.sig_d, gm = sl.gm_d;
@@ -1970,7 +1922,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_power_cluster(PiArgs a, Gr
     if (warp == 0) {
         if (exit_kind == 2 && !no_sweeps) {
             const Part q = cluster_part((s - 1) & 1);
-            ctrl_step(a, s, q, c, nullptr, true, true);
+            if (lane == 0) ctrl_step(a, s, q, c, nullptr, true, true);
         }
         if (lane == 0) {
             const int rs = c.res_sweep;
@@ -2326,12 +2278,12 @@ cmg_status_t power_iteration(const PiRun &run, GridSync *gs, cudaStream_t s, con
         if (maxb < X.P) return CMG_ERR_TOO_LARGE;
         double *partials;
         if (ws) {
-            if (2 * X.P * 3 > ws->partials_cap) return CMG_ERR_TOO_LARGE;
+            if (2 * X.P * kPartDoubles > ws->partials_cap) return CMG_ERR_TOO_LARGE;
             partials = ws->partials;
         } else {
-            CMG_TRY(scr.get(&partials, (size_t)2 * X.P * 3));
+            CMG_TRY(scr.get(&partials, (size_t)2 * X.P * kPartDoubles));
         }
-        a.partials = reinterpret_cast<ff *>(partials);
+        a.partials = reinterpret_cast<PartRec *>(partials);
         return coop_launch(kern, X.P, kStageThreads, X.smem, s, args, gs);
     }
     if (lv.lay) {
@@ -2374,12 +2326,12 @@ cmg_status_t power_iteration(const PiRun &run, GridSync *gs, cudaStream_t s, con
         const int blocks = (int)std::max<long long>(1, std::min<long long>(maxb, (tasks + row_warps - 1) / row_warps));
         double *partials;
         if (ws) {
-            if (2 * blocks * 3 > ws->partials_cap) return CMG_ERR_TOO_LARGE;
+            if (2 * blocks * kPartDoubles > ws->partials_cap) return CMG_ERR_TOO_LARGE;
             partials = ws->partials;
         } else {
-            CMG_TRY(scr.get(&partials, (size_t)2 * blocks * 3));
+            CMG_TRY(scr.get(&partials, (size_t)2 * blocks * kPartDoubles));
         }
-        a.partials = reinterpret_cast<ff *>(partials);
+        a.partials = reinterpret_cast<PartRec *>(partials);
         return coop_launch(kern, blocks, threads, smem, s, args, gs);
     }
     if (!a.tile_row) {
@@ -2402,15 +2354,14 @@ cmg_status_t power_iteration(const PiRun &run, GridSync *gs, cudaStream_t s, con
     // one tile per CTA where possible (each tile's phases are latency-bound),
     // never more CTAs than co-resident
     const int blocks = std::max(1, std::min(maxb, a.ntiles));
-    // partial sums: [2][blocks][3] float-float values (6 floats = 3 doubles each)
     double *partials;
     if (ws) {
-        if (2 * blocks * 3 > ws->partials_cap) return CMG_ERR_TOO_LARGE;
+        if (2 * blocks * kPartDoubles > ws->partials_cap) return CMG_ERR_TOO_LARGE;
         partials = ws->partials;
     } else {
-        CMG_TRY(scr.get(&partials, (size_t)2 * blocks * 3));
+        CMG_TRY(scr.get(&partials, (size_t)2 * blocks * kPartDoubles));
     }
-    a.partials = reinterpret_cast<ff *>(partials);
+    a.partials = reinterpret_cast<PartRec *>(partials);
     return coop_launch(kern, blocks, kTileThreads, smem, s, args, gs);
 }
 
@@ -2438,7 +2389,7 @@ __device__ __forceinline__ void block_allsum(double (&v)[K], double *sm, double 
 // Grid-wide sum of K doubles per thread, result in out[] of every thread.
 template <int K>
 __device__ __forceinline__ bool grid_allsum(double (&v)[K], double *sm, double *part,
-                                            double (&out)[K], GridSync *gs) {
+                                            double (&out)[K], GridBar *bar) {
     double tot[K];
     block_allsum<K>(v, sm, tot);
     if (gridDim.x == 1) {
@@ -2449,7 +2400,7 @@ __device__ __forceinline__ bool grid_allsum(double (&v)[K], double *sm, double *
     if (threadIdx.x == 0)
 #pragma unroll
         for (int k = 0; k < K; k++) part[blockIdx.x * K + k] = tot[k];
-    if (!grid_sync(gs)) return false;
+    if (!grid_sync(bar)) return false;
     const int lane = threadIdx.x & 31;
     double s[K];
 #pragma unroll
@@ -2507,6 +2458,8 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(FinArgs a, GridSync *g
     __shared__ double sm[32 * 4];
     __shared__ double s_best[32], s_bval[32];
     __shared__ int s_bidx[32];
+    __shared__ GridBar s_bar;
+    if (threadIdx.x == 0) grid_bar_init(&s_bar, gs);
     const int n = a.n;
     int r0, r1;
     cta_rows(a.rp, n, blockIdx.x, gridDim.x, &r0, &r1);
@@ -2544,7 +2497,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(FinArgs a, GridSync *g
                     p[1] += yv * yv;
                 }
             }
-            if (!grid_allsum<4>(p, sm, part0, S, gs)) return;
+            if (!grid_allsum<4>(p, sm, part0, S, &s_bar)) return;
             const double mu = S[0] / (double)n;
             const double ss = S[1] - (double)n * mu * mu;
             const double inv = ss > 0.0 ? 1.0 / sqrt(ss) : 0.0;
@@ -2601,7 +2554,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(FinArgs a, GridSync *g
             part1[blockIdx.x * 4 + 1] = (double)bidx;
             part1[blockIdx.x * 4 + 2] = bval;
         }
-        if (!grid_sync(gs)) return;
+        if (!grid_sync(&s_bar)) return;
         __syncthreads();
         if (threadIdx.x == 0) {
             double bb = -1.0, bv = 0.0;
@@ -2620,9 +2573,9 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(FinArgs a, GridSync *g
         __syncthreads();
         if (s_bval[0] < 0.0)
             for (int i = r0 + threadIdx.x; i < r1; i += blockDim.x) a.u[i] = -a.u[i];
-        if (!grid_sync(gs)) return;
+        if (!grid_sync(&s_bar)) return;
     } else if (!a.fresh) {
-        if (!grid_sync(gs)) return;
+        if (!grid_sync(&s_bar)) return;
     }
     // ---- Rayleigh quotient: lambda = (1/2) sum_i sum_j w_ij (u_i - u_j)^2 / ||u||^2
     p[0] = p[1] = p[2] = p[3] = 0.0;
@@ -2644,7 +2597,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(FinArgs a, GridSync *g
             p[1] += ui * ui;
         }
     }
-    if (!grid_allsum<4>(p, sm, part2, S, gs)) return;
+    if (!grid_allsum<4>(p, sm, part2, S, &s_bar)) return;
     const double uu = S[1];
     const double lam = 0.5 * S[0] / uu;
     // ---- residual ||(L - lambda I) u|| / ||u||, (L u)_i = sum_j w_ij (u_i - u_j)
@@ -2665,7 +2618,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(FinArgs a, GridSync *g
             p[0] += rr * rr;
         }
     }
-    if (!grid_allsum<4>(p, sm, part0, S, gs)) return;
+    if (!grid_allsum<4>(p, sm, part0, S, &s_bar)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         a.out[0] = lam;
         a.out[1] = sqrt(S[0] / uu);
