@@ -95,6 +95,8 @@ struct LevelData {
     SweepLayout lay;
     bool has_xl = false;    // ... or its two-phase layout (lay then holds only the row order)
     XLayout xl;
+    bool has_rows = false;  // ... or the row kernel's plan
+    RowPlan rows;
     int cl_ctas = 0, cl_threads = 0, cl_emax = 0;   // FP64 sweeps in one cluster (cluster_plan)
     size_t cl_smem = 0;
     int fp32 = 0;           // this level's sweeps run in FP32
@@ -124,6 +126,7 @@ static void free_level(LevelData &L, cudaStream_t s) {
     dev_free(L.tiles, s);
     free_sweep_layout(L.lay, s);
     free_xlayout(L.xl, s);
+    free_row_plan(L.rows, s);
     L = LevelData();
 }
 
@@ -243,6 +246,7 @@ static PiLevel level_view(const LevelData &L) {
     v.sell_nnz = L.sell_nnz;
     v.lay = L.has_lay ? &L.lay : nullptr;
     v.xl = L.has_xl ? &L.xl : nullptr;
+    v.rows = L.has_rows ? &L.rows : nullptr;
     v.cl_ctas = L.cl_ctas;
     v.cl_threads = L.cl_threads;
     v.cl_emax = L.cl_emax;
@@ -433,9 +437,38 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
                 free_sweep_layout(L.lay, s);
                 if (st != CMG_ERR_TOO_LARGE) return st;
             }
+            // FP64 levels: the row kernel, resident or streaming; FP32 levels:
+            // resident where the layout fits the SMs' shared memory, else the
+            // slice kernel.  CMG_STAGE (either value) keeps the slice kernel.
+            const bool try_rows = getenv("CMG_STAGE") == nullptr;
+            if (try_rows && !L.fp32) {
+                size_t lb = 0, rb = 0;
+                CMG_TRY(build_sweep_layout(1, voff1, std::vector<int>{0, L.n}, L.n, L.rp, L.col, L.w, 0, &L.lay, &lb, s,
+                                           true));
+                const cmg_status_t st = build_row_plan(L.n, L.nnz, L.rp, L.col, L.w, L.lay, 0, &L.rows, &rb, s);
+                if (st == CMG_OK) {
+                    L.has_lay = L.has_rows = true;
+                    lay_bytes += lb + rb;
+                    continue;
+                }
+                free_row_plan(L.rows, s);
+                free_sweep_layout(L.lay, s);
+                if (st != CMG_ERR_TOO_LARGE) return st;
+            }
             CMG_TRY(build_sweep_layout(1, voff1, std::vector<int>{0, L.n}, L.n, L.rp, L.col, L.w, L.fp32,
                                        &L.lay, &lay_bytes, s));
             L.has_lay = true;
+            if (try_rows && L.fp32) {
+                size_t rb = 0;
+                const cmg_status_t st = build_row_plan(L.n, L.nnz, L.rp, L.col, L.w, L.lay, 1, &L.rows, &rb, s);
+                if (st == CMG_OK) {
+                    L.has_rows = true;
+                    lay_bytes += rb;
+                    continue;
+                }
+                free_row_plan(L.rows, s);
+                if (st != CMG_ERR_TOO_LARGE) return st;
+            }
             // gathers that a staged prefix of the iterate would serve
             stage_try[k] = std::min(L.n, stage_capacity(L.fp32));
             if (stage_try[k] > 0) CMG_TRY(layout_count_below(L.lay, stage_try[k], below_dev + k, s));
@@ -506,6 +539,7 @@ cmg_status_t cmg::hierarchy_view(cmg_hierarchy_t h, HierarchyView *out) {
         v.w32 = nullptr;
         v.lay = nullptr;
         v.xl = nullptr;
+        v.rows = nullptr;
         v.cl_ctas = 0;
         out->lv.push_back(v);
     }

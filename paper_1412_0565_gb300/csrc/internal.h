@@ -178,6 +178,34 @@ inline bool partial_stage_pays(unsigned long long below, long long entries, int 
            (double)below * (double)n >= 3.0 * (double)kPartialStage * (double)entries;
 }
 
+// Plan of the row kernel (resident.cu) for a single-graph level whose rows are
+// in the sweep layout's order: items (a warp's unit of work) dealt to P CTAs
+// in contiguous ranges, and for FP64 sweeps the items' own entry arrays.
+struct RowPlan {
+    int P = 0;                  // CTAs of the launch
+    int ni = 0;                 // items
+    int fp32 = 0, col16 = 1;
+    int resident = 0;           // the matrix stays in shared memory for the launch
+    int stage = 0;              // ... and the iterate is copied there every sweep
+    int stream = 0;             // streaming form: read evict-first
+    size_t smem = 0;
+    int res_e = 0, res_i = 0, res_r = 0;   // most entries, items, rows of a CTA
+    long long entries = 0;
+    int4 *item = nullptr;       // [ni + 1] first row, first entry, steps, log2 lanes | rows << 3
+    int *range = nullptr;       // [P + 1] first item of each CTA
+    void *ucol = nullptr;       // FP64: columns (uint16 or int32) and weights by item
+    double *uw = nullptr;
+};
+// Builds it from the level's CSR and the row order (FP64: L.perm / L.inv) or
+// the whole sweep layout (FP32).  CMG_ERR_TOO_LARGE: the level is left to the
+// slice kernel (an FP64 row of more than 4,096 entries, which one warp would
+// hold up, or an FP32 level beyond shared memory).  Adds its bytes to *bytes.
+cmg_status_t build_row_plan(int n, long long nnz, const int *rp, const int *col, const double *w,
+                            const SweepLayout &L, int fp32, RowPlan *R, size_t *bytes, cudaStream_t s);
+void free_row_plan(RowPlan &R, cudaStream_t s);
+struct PiArgs;
+cmg_status_t launch_power_rows(const RowPlan &R, const SweepLayout &L, PiArgs &a, GridSync *gs, cudaStream_t s);
+
 // Bits needed for the ids 0..c-1 (at least 1).
 inline int bits_for(int c) {
     int b = 1;
@@ -241,6 +269,8 @@ struct PiLevel {
     const SweepLayout *lay;
     // two-phase layout (same row order as lay), or nullptr
     const XLayout *xl;
+    // row kernel plan (same row order as lay), or nullptr
+    const RowPlan *rows;
     // FP64 sweeps in one thread-block cluster (cluster_plan): CTAs (0: not
     // planned), threads per CTA, dynamic shared memory per CTA, and the
     // largest SELL-32 entry count a CTA holds
