@@ -89,7 +89,6 @@ struct LevelData {
     int *agg = nullptr;  // onto the next level
     int *tiles = nullptr;
     int ntiles = 0;
-    long long sell_nnz = 0;
     double g = 0.0;
     bool has_lay = false;   // large level: sweeps read the sweep layout
     SweepLayout lay;
@@ -97,8 +96,8 @@ struct LevelData {
     XLayout xl;
     bool has_rows = false;  // ... or the row kernel's plan
     RowPlan rows;
-    int cl_ctas = 0, cl_threads = 0, cl_emax = 0;   // FP64 sweeps in one cluster (cluster_plan)
-    size_t cl_smem = 0;
+    bool has_fix = false;   // small FP64 level: fixed-point sweeps in shared memory
+    FixPlan fix;
     int fp32 = 0;           // this level's sweeps run in FP32
 };
 
@@ -115,6 +114,7 @@ struct cmg_hierarchy_s {
     double *out2 = nullptr;
     double *u_dev = nullptr;
     size_t bytes = 0;
+    int cluster_min = 512;   // rows from which a clustered level is reported as one
 };
 
 static void free_level(LevelData &L, cudaStream_t s) {
@@ -127,6 +127,7 @@ static void free_level(LevelData &L, cudaStream_t s) {
     free_sweep_layout(L.lay, s);
     free_xlayout(L.xl, s);
     free_row_plan(L.rows, s);
+    free_fix_plan(L.fix, s);
     L = LevelData();
 }
 
@@ -243,14 +244,10 @@ static PiLevel level_view(const LevelData &L) {
     v.agg = L.agg;
     v.tile_row = L.tiles;
     v.ntiles = L.ntiles;
-    v.sell_nnz = L.sell_nnz;
     v.lay = L.has_lay ? &L.lay : nullptr;
     v.xl = L.has_xl ? &L.xl : nullptr;
     v.rows = L.has_rows ? &L.rows : nullptr;
-    v.cl_ctas = L.cl_ctas;
-    v.cl_threads = L.cl_threads;
-    v.cl_emax = L.cl_emax;
-    v.cl_smem = L.cl_smem;
+    v.fix = L.has_fix ? &L.fix : nullptr;
     return v;
 }
 
@@ -324,7 +321,6 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
             st = galerkin_async(F.n, F.nnz, F.rp, F.col, F.w, agg, bits_for(F.n), cnt_dev, rp_t,
                                 col_t, w_t, s);
             if (st != CMG_OK) break;
-            if ((st = sell_size_async(&cnt_dev->c, F.n, rp_t, &cnt_dev->sell, s)) != CMG_OK) break;
             st = from_cuda(cudaMemcpyAsync(&hc, cnt_dev, sizeof(hc), cudaMemcpyDeviceToHost, s));
             if (st != CMG_OK) break;
             if ((st = from_cuda(cudaStreamSynchronize(s))) != CMG_OK) break;
@@ -339,7 +335,6 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
         C.n = hc.c;
         C.nnz = hc.nseg;
         memcpy(&C.g, &hc.gbits, sizeof(double));
-        C.sell_nnz = (C.n <= 65536) ? (long long)hc.sell : 0;
         st = dev_alloc_n(&C.rp, (size_t)C.n + 1, s);
         if (st == CMG_OK) st = dev_alloc_n(&C.col, (size_t)std::max<long long>(C.nnz, 1), s);
         if (st == CMG_OK) st = dev_alloc_n(&C.w, (size_t)std::max<long long>(C.nnz, 1), s);
@@ -370,42 +365,49 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
     // attachment graphs whose coarse levels ran in FP32).
     const int form32 = o.precision == CMG_PRECISION_FP32_SWEEP;
     const int nlev = (int)h->lv.size();
-    {
-        unsigned long long *cnt;
-        CMG_TRY(scr.get(&cnt, 1));
-        for (int k = 0; k < nlev; k++) {
-            LevelData &L = h->lv[k];
-            if (k == 0 && L.n <= 65536) CMG_TRY(sell_size(L.n, L.rp, cnt, &L.sell_nnz, s));
-            L.fp32 = (form32 && L.nnz >= kFp32MinEntries) ? 1 : 0;
-        }
-    }
+    for (auto &L : h->lv) L.fp32 = (form32 && L.nnz >= kFp32MinEntries) ? 1 : 0;
     for (auto &L : h->lv) {
         if (!L.fp32) continue;
         CMG_TRY(dev_alloc_n(&L.w32, (size_t)std::max<long long>(L.nnz, 1), s));
         CMG_TRY(launch_to_float(L.nnz, L.w, L.w32, s));
     }
-    // ---- FP64 levels of 512 to a few thousand rows: sweeps in one thread-
-    // block cluster (every CTA holds the iterate; rows split over the SMs)
-    // (CMG_CLUSTER=0: never; CMG_CLUSTER=<rows>: from that many rows on)
+    // ---- FP64 levels of up to a few thousand rows: fixed-point sweeps in the
+    // shared memory of one CTA or one thread-block cluster (CMG_CLUSTER=0: one
+    // CTA only; CMG_CLUSTER=<rows>: what cmg_level_kernels calls a cluster level)
+    size_t lay_bytes = 0;
     const char *cl_env = getenv("CMG_CLUSTER");
-    if (!cl_env || cl_env[0] != '0') {
-        const int cl_min = cl_env ? std::max(128, atoi(cl_env)) : 512;
-        std::vector<int> rph;
-        for (auto &L : h->lv) {
-            if (L.fp32 || L.n < cl_min || !cluster_may_hold(L.n)) continue;
-            rph.resize((size_t)L.n + 1);
-            CMG_CUDA(cudaMemcpyAsync(rph.data(), L.rp, sizeof(int) * ((size_t)L.n + 1), cudaMemcpyDeviceToHost, s));
-            CMG_CUDA(cudaStreamSynchronize(s));
-            PiLevel v = level_view(L);
-            cluster_plan(&v, rph.data());
-            L.cl_ctas = v.cl_ctas;
-            L.cl_threads = v.cl_threads;
-            L.cl_emax = v.cl_emax;
-            L.cl_smem = v.cl_smem;
+    h->cluster_min = cl_env ? std::max(128, atoi(cl_env)) : 512;
+    {
+        std::vector<FixLevel> small;
+        std::vector<int> who;
+        for (int k = 0; k < nlev; k++) {
+            const LevelData &L = h->lv[k];
+            if (L.fp32 || !fix_may_hold(L.n, L.nnz)) continue;
+            FixLevel f = {};
+            f.n = L.n;
+            f.nnz = L.nnz;
+            f.rp = L.rp;
+            f.col = L.col;
+            f.w = L.w;
+            f.g = L.g;
+            f.max_ctas = cl_env && cl_env[0] == '0' ? 1 : 8;
+            small.push_back(f);
+            who.push_back(k);
         }
+        const cmg_status_t st = build_fix_plans(small, s);
+        for (size_t q = 0; q < small.size(); q++) {
+            LevelData &L = h->lv[who[q]];
+            if (st == CMG_OK && small[q].ok) {
+                L.has_fix = true;
+                L.fix = small[q].plan;
+                lay_bytes += L.fix.bytes;
+            } else {
+                free_fix_plan(small[q].plan, s);
+            }
+        }
+        if (st != CMG_OK) return st;
     }
     // ---- sweep layouts for the levels the shared-memory kernels cannot hold
-    size_t lay_bytes = 0;
     std::vector<int> stage_try(nlev, 0), partial_try(nlev, 0);
     std::vector<unsigned long long> below(2 * (size_t)nlev, 0);
     unsigned long long *below_dev = nullptr;
@@ -415,7 +417,7 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
         CMG_TRY(scr.get(&below_dev, 2 * (size_t)nlev));
         for (int k = 0; k < nlev; k++) {
             LevelData &L = h->lv[k];
-            if (L.cl_ctas > 0 || small_level_fits(level_view(L), L.fp32)) continue;
+            if (L.has_fix || small_level_fits(level_view(L), L.fp32)) continue;
             const int hv[2] = {0, L.n};
             CMG_CUDA(cudaMemcpyAsync(voff1, hv, sizeof(hv), cudaMemcpyHostToDevice, s));
             bool x2 = false;
@@ -540,7 +542,7 @@ cmg_status_t cmg::hierarchy_view(cmg_hierarchy_t h, HierarchyView *out) {
         v.lay = nullptr;
         v.xl = nullptr;
         v.rows = nullptr;
-        v.cl_ctas = 0;
+        v.fix = nullptr;
         out->lv.push_back(v);
     }
     out->device = h->device;
@@ -786,7 +788,7 @@ cmg_status_t cmg_level_kernels(cmg_hierarchy_t h, int32_t *kind_out, int32_t *st
         const LevelData &L = h->lv[j];
         const int staged = L.has_lay ? L.lay.stage_n : 0;
         int kind = 0;
-        if (L.cl_ctas > 0) kind = 5;
+        if (L.has_fix) kind = (L.fix.C > 1 && L.n >= h->cluster_min) ? 5 : 0;
         else if (L.has_xl) kind = 4;
         else if (L.has_lay) kind = staged > 0 ? 2 : 1;
         else if (!small_level_fits(level_view(L), L.fp32)) kind = 3;

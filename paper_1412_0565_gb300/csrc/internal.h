@@ -203,7 +203,37 @@ struct RowPlan {
 cmg_status_t build_row_plan(int n, long long nnz, const int *rp, const int *col, const double *w,
                             const SweepLayout &L, int fp32, RowPlan *R, size_t *bytes, cudaStream_t s);
 void free_row_plan(RowPlan &R, cudaStream_t s);
+// Plan of the fixed-point kernel for small FP64 levels (fixed.cu): one CTA, or one
+// cluster of up to 8, holds the level in shared memory.
+struct FixPlan {
+    int C = 0, threads = 0;
+    int ni = 0, by_warp = 0;               // one item of that many steps per row warp (0: by entries)
+    int res_e = 0, res_i = 0, res_r = 0;   // most entries, items, rows of a CTA
+    size_t smem = 0, bytes = 0;
+    void *arena = nullptr;                 // the arrays below, one allocation
+    int4 *item = nullptr;
+    int *range = nullptr, *perm = nullptr;
+    uint16_t *ucol = nullptr;
+    int2 *uc = nullptr, *ud = nullptr;
+};
+// A level offered to build_fix_plans; ok: planned.
+struct FixLevel {
+    int n;
+    long long nnz;
+    const int *rp, *col;
+    const double *w;
+    double g;
+    int max_ctas;      // 1: no cluster
+    FixPlan plan;
+    int ok;
+};
+// Plans every level that fits (one launch, one host synchronisation).
+cmg_status_t build_fix_plans(std::vector<FixLevel> &lv, cudaStream_t s);
+// Whether a level of this size is worth offering.
+bool fix_may_hold(int n, long long nnz);
+void free_fix_plan(FixPlan &F, cudaStream_t s);
 struct PiArgs;
+cmg_status_t launch_power_fix(const FixPlan &F, PiArgs &a, cudaStream_t s);
 cmg_status_t launch_power_rows(const RowPlan &R, const SweepLayout &L, PiArgs &a, GridSync *gs, cudaStream_t s);
 
 // Bits needed for the ids 0..c-1 (at least 1).
@@ -220,7 +250,6 @@ struct LevelCounts {
     int nseg;                   // coarse stored entries
     int pad;
     unsigned long long gbits;   // coarse Gershgorin shift (bits of a double)
-    unsigned long long sell;    // SELL-32 size of the coarse level
     GridSync gs;                // barrier state of the coarsening kernel
 };
 
@@ -263,7 +292,6 @@ struct PiLevel {
     const int *agg;      // this level -> next coarser level (nullptr at the coarsest)
     const int *tile_row; // row tiles of the sweep kernel (nullptr: built on demand)
     int ntiles;
-    long long sell_nnz;  // SELL-32 size for the shared-memory kernel (0: unknown)
     // sweep layout (one graph) for the slice kernel, or nullptr; with a layout
     // the level's iterates are stored in the layout's row order
     const SweepLayout *lay;
@@ -271,32 +299,9 @@ struct PiLevel {
     const XLayout *xl;
     // row kernel plan (same row order as lay), or nullptr
     const RowPlan *rows;
-    // FP64 sweeps in one thread-block cluster (cluster_plan): CTAs (0: not
-    // planned), threads per CTA, dynamic shared memory per CTA, and the
-    // largest SELL-32 entry count a CTA holds
-    int cl_ctas, cl_threads, cl_emax;
-    size_t cl_smem;
+    // fixed-point kernel plan (natural row order on the outside), or nullptr
+    const FixPlan *fix;
 };
-
-// Plans a level's FP64 sweeps in one thread-block cluster of 2..8 CTAs,
-// each holding the whole iterate ring and the SELL-32 slices of its share
-// of the rows, from the level's row pointers (host copy, n + 1).  Leaves
-// lv->cl_ctas at 0 when the level is outside the plan's range or no cluster
-// of that size can be resident.
-void cluster_plan(PiLevel *lv, const int *rp_host);
-// Whether a cluster CTA could hold an n-row level's iterate ring (3 x n
-// values), g - d_i and slot order at all: the check before cluster_plan,
-// which needs the level's row pointers on the host.
-bool cluster_may_hold(int n);
-
-// SELL-32 size of a CSR level (sum over 32-row slices of 32 x longest row);
-// dev_counter: one device unsigned long long of scratch.  Synchronises s.
-cmg_status_t sell_size(int n, const int *rp, unsigned long long *dev_counter, long long *out,
-                       cudaStream_t s);
-// The same for a level whose row count is in device memory (at most n_cap),
-// without host synchronisation (the caller reads *dev_counter later).
-cmg_status_t sell_size_async(const int *n_dev, int n_cap, const int *rp,
-                             unsigned long long *dev_counter, cudaStream_t s);
 
 // Row tiles of a level for the tiled sweep kernel (tile_count + 1 entries).
 int tile_count(int n, long long nnz);

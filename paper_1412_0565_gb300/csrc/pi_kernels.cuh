@@ -58,7 +58,6 @@ struct PiArgs {
     PiResult *res;
     PartRec *partials;      // [2][gridDim.x]: the CTAs' stop sums, by sweep parity
     float zero_tol2;        // (64 eps)^2 of the sweep precision
-    long long sell_nnz;     // SELL-32 size of the level (0: unknown)
     const int *cinvp;       // coarse level's layout order (start = 1), or nullptr
     // slice kernel: the level's sweep layout (rows in layout order)
     const int *perm;
@@ -85,7 +84,8 @@ struct PiArgs {
     const int4 *items;
     const int *item_range;
     int res_entries, res_items, res_rows;
-    int cl_emax;            // cluster kernel: SELL-32 entries each CTA holds (at most)
+    int nitems;             // fixed-point sweeps: items of the level
+    const int2 *fix_d;      // fixed-point sweeps: diagonal D_i by row in layout order
 };
 
 
@@ -195,6 +195,26 @@ struct Ctl {
 };
 
 
+// Records the decision to stop after sweep s.
+__device__ __forceinline__ void ctl_stop(const PiArgs &a, int s, ff mu, ff ss, ff cs, bool zero, bool conv, Ctl &c) {
+    c.stopped = 1;
+    c.zero = zero;
+    c.res_sweep = s;
+    if (zero) {
+        c.mu_res = to_d(c.mu_prev);
+        c.ss_res = to_d(c.ss_prev);
+        c.cos_res = 1.0;
+    } else {
+        c.mu_res = to_d(mu);
+        c.ss_res = to_d(ss);
+        c.mu_res_prev = to_d(c.mu_prev);
+        c.ss_res_prev = to_d(c.ss_prev);
+        const double den = sqrt(c.ss_res * c.ss_res_prev);
+        c.cos_res = den > 0.0 ? to_d(cs) / den : 1.0;
+    }
+    c.capped = (a.mode == 0 && !zero && !conv) ? 1 : 0;
+}
+
 // One control step for sweep s (s >= 1) with its reduced sums P.  Decides,
 // and fills the slot for sweep s+2 (m_{s+1}, e_{s+1}).  `count_exit`: the
 // loop ends after sweep s regardless (fixed count or sweep cap reached).
@@ -213,24 +233,7 @@ __device__ __forceinline__ void ctrl_step(const PiArgs &a, int s, const Part &P,
     bool stop = zero;
     if (a.mode == 0) stop = stop || conv || count_exit;
     else stop = stop || count_exit;
-    if (stop && !c.stopped) {
-        c.stopped = 1;
-        c.zero = zero;
-        c.res_sweep = s;
-        if (zero) {
-            c.mu_res = to_d(c.mu_prev);
-            c.ss_res = to_d(c.ss_prev);
-            c.cos_res = 1.0;
-        } else {
-            c.mu_res = to_d(mu);
-            c.ss_res = to_d(ss);
-            c.mu_res_prev = to_d(c.mu_prev);
-            c.ss_res_prev = to_d(c.ss_prev);
-            const double den = sqrt(c.ss_res * c.ss_res_prev);
-            c.cos_res = den > 0.0 ? to_d(cs) / den : 1.0;
-        }
-        c.capped = (a.mode == 0 && !zero && !conv) ? 1 : 0;
-    }
+    if (stop && !c.stopped) ctl_stop(a, s, mu, ss, cs, zero, conv, c);
     // parameters of sweep s+2 (exact power-of-two scaling of mu_s - m_s)
     const ff dm = ff_sub(mu, c.m_cur);
     const ff m_next = c.e_cur ? ff_make(ldexpf(dm.hi, c.e_cur), ldexpf(dm.lo, c.e_cur)) : dm;

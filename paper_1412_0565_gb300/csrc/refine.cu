@@ -22,7 +22,7 @@
 // Sums and scalars are float-float (ffloat.cuh) on the FP32 pipe; FP64 is
 // used where the FP64 form computes its sweeps, and for the final scalars.
 //
-// Two kernels:
+// Kernels here (fixed.cu and resident.cu hold the others):
 //   k_power_tiled  large levels: cooperative persistent kernel, one grid
 //                  barrier per sweep.  Rows are cut into tiles (at most
 //                  kTileRows rows, about kChunk entries); a tile's column
@@ -40,10 +40,6 @@
 namespace cmg {
 
 #ifdef CMG_TRACE
-// cycle stamps of the first sweeps of the last small-kernel launch:
-// [sweep][0] loop top, [1] control done, [2] first row warp done, [3] last row warp done
-__device__ long long g_trace[256][8];
-#define TRACE(s, k) do { if ((s) < 256) g_trace[(s)][(k)] = clock64(); } while (0)
 // cycle stamps of the phases of the two-phase kernel's third sweep, per CTA
 // and pass: [b][t][0] pass top, [2] phase 1 done, [3] after the barrier,
 // [5] the last dest block's list summed, [6] its rows completed
@@ -52,17 +48,8 @@ __device__ long long g_x2t[160][32][8];
 extern "C" int cmg_debug_x2_trace(long long *host, int count) {
     return (int)cudaMemcpyFromSymbol(host, g_x2t, sizeof(long long) * (size_t)count);
 }
-// cycle stamps of the cluster kernel's first sweeps (rank 0, thread 0):
-// [s][0] loop top, [1] rows done, [2] sums stored, [3] after the barrier
-__device__ long long g_clt[256][4];
-#define CLT(s, k) do { if ((s) < 256 && threadIdx.x == 0 && cluster_rank() == 0) g_clt[(s)][(k)] = clock64(); } while (0)
-extern "C" int cmg_debug_cluster_trace(long long *host, int count) {
-    return (int)cudaMemcpyFromSymbol(host, g_clt, sizeof(long long) * (size_t)count);
-}
 #else
-#define TRACE(s, k) do { } while (0)
 #define X2T(s, t, k) do { } while (0)
-#define CLT(s, k) do { } while (0)
 #endif
 
 constexpr int kTileThreads = 512;                 // warp 0: control, 15 row warps
@@ -932,259 +919,49 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_power_2p(PiArgs a, GridSyn
 }
 
 // ================================================================== small kernel
-// Shared memory: ring[3][n] T, gd[n] (FP64 form), w[E] T, rp[n+1] int,
-// col[E] int, slice offsets[n/32 + 2] int.  E = nnz (CSR) or the SELL-32
-// size (one lane per row: each 32-row slice stores entry k of its rows
-// contiguously, rows padded to the slice's longest with zero weights, so the
-// lanes of a warp read consecutive words -- no bank conflicts).
-// ================================================================== slot order
-// The one-CTA and cluster kernels hold a level's rows in "slot" order: rows by
-// decreasing degree, ties by row number, so that the 32 rows of a SELL-32
-// slice have about the same length and the slices carry little padding (a
-// padded entry costs an FP64 FMA like a stored one).  The iterate, g - d_i
-// and the columns are renumbered to slots; rows are mapped back on output.
-// The order is taken when it shrinks the SELL-32 size by at least 1/16 and
-// every row holds fewer than n entries; otherwise slots are rows.  Sorted
-// order never needs more entries than row order: in any order, at least k+1
-// slices hold a row at least as long as the sorted row at position 32k, so
-// the k-th widest slice is at least as wide as the sorted order's k-th slice,
-// and a buffer sized for row order holds either.
-__host__ __device__ __forceinline__ bool slot_order_pays(long long natural, long long sorted) {
-    return sorted * 16 <= natural * 15;
-}
-
-// perm[p] = row of slot p and inv[i] = slot of row i (n ints each, shared
-// memory); hist: n ints of shared scratch.  A stable counting sort: bucket
-// maxdeg - d_i, bucket starts by one warp's scan, rows placed by one warp in
-// row order (rows of equal degree keep their order).  Every thread of the CTA
-// calls it; the CTA is synchronised on return.
-__device__ __noinline__ void slot_order(int n, const int *rp, int *perm, int *inv, int *hist) {
-    __shared__ int s_maxd, s_sorted;
-    __shared__ unsigned long long s_nat;
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
-    if (tid == 0) {
-        s_maxd = 0;
-        s_sorted = 0;
-        s_nat = 0;
-    }
-    __syncthreads();
-    int md = 0;
-    unsigned long long nat = 0;
-    for (int i = tid; i < n; i += nt) md = max(md, rp[i + 1] - rp[i]);
-    for (int q = tid; q < (n + 31) / 32; q += nt) {
-        int L = 0;
-        for (int r = 32 * q; r < min(n, 32 * q + 32); r++) L = max(L, rp[r + 1] - rp[r]);
-        nat += 32ull * (unsigned long long)L;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        md = max(md, __shfl_xor_sync(0xffffffffu, md, o));
-        nat += __shfl_xor_sync(0xffffffffu, nat, o);
-    }
-    if (lane == 0) {
-        atomicMax(&s_maxd, md);
-        atomicAdd(&s_nat, nat);
-    }
-    __syncthreads();
-    const int D = s_maxd;
-    if (D < n) {
-        for (int b = tid; b <= D; b += nt) hist[b] = 0;
-        __syncthreads();
-        for (int i = tid; i < n; i += nt) {
-            const int b = D - (rp[i + 1] - rp[i]);
-            inv[i] = b;   // the row's bucket, read back by the placing warp
-            atomicAdd(&hist[b], 1);
-        }
-        __syncthreads();
-        if (tid < 32) {
-            // bucket starts (exclusive scan) and the SELL-32 size in slot
-            // order: a slice is as wide as the degree of its first slot
-            int carry = 0;
-            unsigned long long tot = 0;
-            for (int b0 = 0; b0 <= D; b0 += 32) {
-                const int b = b0 + lane;
-                const int c = (b <= D) ? hist[b] : 0;
-                int incl = c;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int t = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += t;
-                }
-                const int st = carry + incl - c;
-                if (b <= D) {
-                    hist[b] = st;
-                    const int starts = (st + c + 31) / 32 - (st + 31) / 32;
-                    tot += 32ull * (unsigned long long)(D - b) * (unsigned long long)starts;
-                }
-                carry += __shfl_sync(0xffffffffu, incl, 31);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-            if (lane == 0) s_sorted = slot_order_pays((long long)s_nat, (long long)tot) ? 1 : 0;
-        }
-        __syncthreads();
-    }
-    if (s_sorted) {
-        if (tid < 32) {
-            for (int i0 = 0; i0 < n; i0 += 32) {
-                const int i = i0 + lane;
-                const unsigned act = __ballot_sync(0xffffffffu, i < n);
-                if (i < n) {
-                    const int b = inv[i];
-                    const unsigned peers = __match_any_sync(act, b);
-                    const int r = __popc(peers & ((1u << lane) - 1u));
-                    const int base = hist[b];
-                    perm[base + r] = i;
-                    __syncwarp(act);
-                    if (r == 0) hist[b] = base + __popc(peers);
-                }
-                __syncwarp();
-            }
-        }
-    } else {
-        for (int p = tid; p < n; p += nt) perm[p] = p;
-    }
-    __syncthreads();
-    for (int p = tid; p < n; p += nt) inv[perm[p]] = p;
-    __syncthreads();
-}
-
-// Prefix sums pre[0..nsl] of the SELL-32 slice sizes in the order slot_order
-// takes, from the host copy of the row pointers (the same arithmetic; the
-// sorted widths come from the degree counts: slice q of the sorted rows is as
-// wide as the degree at sorted position 32q).
-static void slot_sell_prefix(int n, const int *rph, std::vector<int> &pre) {
-    const int nsl = (n + 31) / 32;
-    std::vector<int> wid(nsl, 0);
-    int D = 0;
-    long long nat = 0;
-    for (int q = 0; q < nsl; q++) {
-        for (int r = 32 * q; r < std::min(n, 32 * q + 32); r++) wid[q] = std::max(wid[q], rph[r + 1] - rph[r]);
-        nat += 32ll * wid[q];
-        D = std::max(D, wid[q]);
-    }
-    if (D < n) {
-        std::vector<int> cnt((size_t)D + 1, 0), sw(nsl, 0);
-        for (int i = 0; i < n; i++) cnt[rph[i + 1] - rph[i]]++;
-        long long tot = 0;
-        int pos = 0;   // sorted position of the first row of degree d
-        for (int d = D; d >= 0; d--) {
-            for (int q = (pos + 31) / 32; 32 * q < pos + cnt[d]; q++) {
-                sw[q] = d;
-                tot += 32ll * d;
-            }
-            pos += cnt[d];
-        }
-        if (slot_order_pays(nat, tot)) wid.swap(sw);
-    }
-    pre.assign(nsl + 1, 0);
-    for (int q = 0; q < nsl; q++) pre[q + 1] = pre[q] + 32 * wid[q];
-}
-
-template <typename T>
-constexpr size_t small_smem_bytes(long long n, long long e) {
-    return (size_t)(sizeof(T) * (3 * n + e) + (sizeof(T) == 8 ? 8 * n : 0) + 4 * (n + 1) + 4 * e +
-                    4 * (n / 32 + 2) + 4 * n + 64);
-}
-
-template <typename T, int G>
+// Levels one CTA can hold that have no fixed-point plan (step entry points,
+// geometric levels): shared memory holds ring[3][n], g - d_i [n], w[nnz],
+// rp[n + 1], col[nnz].
+template <int G>
 __global__ void __launch_bounds__(kSmallMaxThreads) k_power_small(PiArgs a, GridSync *) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n = a.n;
     const int m = a.rp[n];
-    const bool sell = (G == 1) && a.sell_nnz > 0;
-    const int E = sell ? (int)a.sell_nnz : m;
-    const bool fp64 = sizeof(T) == 8;
-    T *ring0 = reinterpret_cast<T *>(smem_raw);
-    double *s_gd = reinterpret_cast<double *>(ring0 + 3 * n);
-    T *s_w = fp64 ? reinterpret_cast<T *>(s_gd + n) : ring0 + 3 * n;
-    int *s_rp = reinterpret_cast<int *>(s_w + E);
+    double *ring0 = reinterpret_cast<double *>(smem_raw);
+    double *s_gd = ring0 + 3 * (size_t)n;
+    double *s_w = s_gd + n;
+    // every row thread's stop sums (A, B, C), by sweep parity; the control warp
+    // reduces them (one float-float conversion per control lane, instead of
+    // one per row thread)
+    double *s_dacc = s_w + m;
+    int *s_rp = reinterpret_cast<int *>(s_dacc + 6 * (size_t)blockDim.x);
     int *s_col = s_rp + n + 1;
-    int *s_soff = s_col + E;
-    // SELL-32 form: the row of each slot (the iterate, g - d_i and the
-    // columns are held by slot)
-    int *s_perm = s_soff + (n / 32 + 2);
-    // FP64 form: every row thread's stop sums (A, B, C as doubles), by sweep
-    // parity; the control warp reduces them (one float-float conversion per
-    // control lane, instead of one per row thread: conversions issue on the
-    // FP64 pipe)
-    double *s_dacc = reinterpret_cast<double *>(
-        (reinterpret_cast<uintptr_t>(s_perm + n) + 7) & ~(uintptr_t)7);
-    __shared__ Part s_pw[2][32];
+    __shared__ Part s_pw[32];
     __shared__ Slot s_slot[2];
+    __shared__ Ctl c;   // used by lane 0 of the control warp (in registers it would take every row thread's)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nw = blockDim.x >> 5;
     // the control warp's sums of the row warps' partials of parity `par`, in
     // a fixed order (rows warps in order per lane, then the lanes' xor tree)
     auto ctl_part = [&](int par) -> Part {
-        if constexpr (sizeof(T) == 8) {
-            double A = 0.0, B = 0.0, C = 0.0;
-            for (int w = 1; w < nw; w++) {
-                const double *src = s_dacc + ((size_t)par * blockDim.x + 32 * w + lane) * 3;
-                A += src[0];
-                B += src[1];
-                C += src[2];
-            }
-            Part p;
-            p.A = ff_from_double(A);
-            p.B = ff_from_double(B);
-            p.C = ff_from_double(C);
-            return warp_sum_part(p);
-        } else {
-            const Part q = (lane >= 1 && lane < nw) ? s_pw[par][lane] : part_zero();
-            return warp_sum_part(q, 1, pow2_at_least(nw));
+        double A = 0.0, B = 0.0, C = 0.0;
+        for (int w = 1; w < nw; w++) {
+            const double *src = s_dacc + ((size_t)par * blockDim.x + 32 * w + lane) * 3;
+            A += src[0];
+            B += src[1];
+            C += src[2];
         }
+        Part p;
+        p.A = ff_from_double(A);
+        p.B = ff_from_double(B);
+        p.C = ff_from_double(C);
+        return warp_sum_part(p);
     };
-    const T *__restrict__ wv = wsel<T>(a);
-    const T g = (T)a.g;
-    const float inv_gf = 1.0f / (float)a.g;
-    const double inv_gd = 1.0 / a.g;
 
     for (int i = tid; i <= n; i += blockDim.x) s_rp[i] = a.rp[i];
-    const int nsl = (n + 31) / 32;
-    if (sell) {
-        __syncthreads();
-        // slot order; inv and the sort's scratch borrow ring slots 1 and 2
-        // (n values each), which the first sweep overwrites
-        int *s_inv = reinterpret_cast<int *>(ring0 + n);
-        slot_order(n, s_rp, s_perm, s_inv, reinterpret_cast<int *>(ring0 + 2 * (size_t)n));
-        for (int q = tid; q < nsl; q += blockDim.x) {
-            int L = 0;
-            for (int p = 32 * q; p < min(n, 32 * q + 32); p++) {
-                const int r = s_perm[p];
-                L = max(L, s_rp[r + 1] - s_rp[r]);
-            }
-            s_soff[q + 1] = 32 * L;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            s_soff[0] = 0;
-            for (int q = 0; q < nsl; q++) s_soff[q + 1] += s_soff[q];
-        }
-        __syncthreads();
-        for (int p = tid; p < 32 * nsl; p += blockDim.x) {
-            const int q = p >> 5, l = p & 31;
-            const int L = (s_soff[q + 1] - s_soff[q]) >> 5;
-            const int r = (p < n) ? s_perm[p] : 0;
-            const int e0 = (p < n) ? s_rp[r] : 0;
-            const int len = (p < n) ? s_rp[r + 1] - e0 : 0;
-            for (int k = 0; k < L; k++) {
-                const int idx = s_soff[q] + 32 * k + l;
-                if (k < len) {
-                    s_col[idx] = s_inv[a.col[e0 + k]];
-                    s_w[idx] = wv[e0 + k];
-                } else {
-                    s_col[idx] = (p < n) ? p : 0;   // zero weight: no contribution
-                    s_w[idx] = (T)0;
-                }
-            }
-        }
-        __syncthreads();
-    } else {
-        for (int e = tid; e < m; e += blockDim.x) {
-            s_col[e] = a.col[e];
-            s_w[e] = wv[e];
-        }
+    for (int e = tid; e < m; e += blockDim.x) {
+        s_col[e] = a.col[e];
+        s_w[e] = a.w[e];
     }
     {
         const void *cb = nullptr;
@@ -1196,25 +973,21 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_power_small(PiArgs a, Grid
         }
         Part acc = part_zero();
         for (int i = tid; i < n; i += blockDim.x) {
-            const int r = sell ? s_perm[i] : i;
-            const T xt = (T)start_value(a, r, cb, cmu, cinv);
+            const double xt = start_value(a, i, cb, cmu, cinv);
             ring0[i] = xt;
-            if (fp64) {
-                double d = 0.0;
-                for (int e = a.rp[r], e1 = a.rp[r + 1]; e < e1; e++) d += a.w[e];
-                s_gd[i] = a.g - d;
-            }
-            const ff v = fp64 ? ff_from_double((double)xt) : ff_make((float)xt, 0.f);
+            double d = 0.0;
+            for (int e = a.rp[i], e1 = a.rp[i + 1]; e < e1; e++) d += a.w[e];
+            s_gd[i] = a.g - d;
+            const ff v = ff_from_double(xt);
             acc.A = ff_add(acc.A, v);
             acc.B = ff_add(acc.B, ff_mul(v, v));
         }
         Part p = warp_sum_part(acc);
-        if (lane == 0) s_pw[0][warp] = p;
+        if (lane == 0) s_pw[warp] = p;
     }
     __syncthreads();
-    __shared__ Ctl c;   // used by lane 0 of the control warp (in registers it would take every row thread's)
     if (warp == 0) {
-        Part q = (lane < nw) ? s_pw[0][lane] : part_zero();
+        Part q = (lane < nw) ? s_pw[lane] : part_zero();
         q = warp_sum_part(q);
         const double mu0 = to_d(q.A) / (double)n;
         double ss0 = to_d(q.B) - (double)n * mu0 * mu0;
@@ -1222,8 +995,8 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_power_small(PiArgs a, Grid
         const int e0 = start_exponent(ss0);
         if (lane == 0) {
             ctl_init(c, a, mu0, ss0, e0);
-            s_slot[1] = slot_make(ff_from_double(mu0), e0, a.g, c.inv_g, fp64);
-            s_slot[0] = slot_make(ff_zero(), 0, a.g, c.inv_g, fp64);
+            s_slot[1] = slot_make(ff_from_double(mu0), e0, a.g, c.inv_g, true);
+            s_slot[0] = slot_make(ff_zero(), 0, a.g, c.inv_g, true);
         }
     }
     __syncthreads();
@@ -1244,105 +1017,50 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_power_small(PiArgs a, Grid
             exit_kind = 2;
             break;
         }
-        const T *x = ring0 + (size_t)(s % 3) * n;
-        T *y = ring0 + (size_t)((s + 1) % 3) * n;
+        const double *x = ring0 + (size_t)(s % 3) * n;
+        double *y = ring0 + (size_t)((s + 1) % 3) * n;
         if (warp == 0) {
-            if (lane == 0) TRACE(s, 0);
             if (s >= 1) {
                 const Part q = ctl_part(s & 1);
-                if (lane == 0) ctrl_step(a, s, q, c, &s_slot[s & 1], false, fp64);
+                if (lane == 0) ctrl_step(a, s, q, c, &s_slot[s & 1], false, true);
             }
-            if (lane == 0) TRACE(s, 1);
         } else {
-            if (lane == 0 && warp == 1) TRACE(s, 4);
-            const T mT = fp64 ? (T)sl.m_d : (T)sl.m.hi;
-            const T sig = fp64 ? (T)sl.sig_d : (T)scale2f(inv_gf, sl.e);
-            const T gm = fp64 ? (T)sl.gm_d : g * mT;
-            Acc<T> acc;
+            Acc<double> acc;
             acc.reset();
             for (int base = rt / G;; base += groups) {
                 if (__shfl_sync(0xffffffffu, base, 0) >= n) break;
                 const int i = base;
-                T ac = (T)0, xi = (T)0;
-                if (sell) {
-                    // one lane per row, 32 rows per warp = one slice; padded
-                    // entries have zero weight
-                    const int q = base >> 5;
-                    const int off = s_soff[q] + (base & 31);
-                    const int L = (s_soff[q + 1] - s_soff[q]) >> 5;
-                    xi = (i < n) ? x[i] : (T)0;
-                    T a0 = (T)0, a1 = (T)0;
-                    int k = 0;
-                    for (; k + 1 < L; k += 2) {
-                        const int c0 = s_col[off + 32 * k], c1 = s_col[off + 32 * k + 32];
-                        const T w0 = s_w[off + 32 * k], w1 = s_w[off + 32 * k + 32];
-                        const T x0 = x[c0], x1 = x[c1];
-                        if (fp64) {
-                            a0 = fma(w0, x0, a0);
-                            a1 = fma(w1, x1, a1);
-                        } else {
-                            a0 += w0 * (xi - x0);
-                            a1 += w1 * (xi - x1);
-                        }
-                    }
-                    if (k < L) {
-                        const T w0 = s_w[off + 32 * k], x0 = x[s_col[off + 32 * k]];
-                        if (fp64) a0 = fma(w0, x0, a0);
-                        else a0 += w0 * (xi - x0);
-                    }
-                    ac = a0 + a1;
-                } else if (i < n) {
+                double ac = 0.0, xi = 0.0;
+                if (i < n) {
                     xi = x[i];
                     // four independent accumulators: the loads of four entries
                     // are in flight together
-                    T a0 = (T)0, a1 = (T)0, a2 = (T)0, a3 = (T)0;
+                    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
                     int e = s_rp[i] + rlane;
                     const int e1 = s_rp[i + 1];
                     for (; e + 3 * G < e1; e += 4 * G) {
                         const int c0 = s_col[e], c1 = s_col[e + G], c2 = s_col[e + 2 * G], c3 = s_col[e + 3 * G];
-                        const T w0 = s_w[e], w1 = s_w[e + G], w2 = s_w[e + 2 * G], w3 = s_w[e + 3 * G];
-                        const T x0 = x[c0], x1 = x[c1], x2 = x[c2], x3 = x[c3];
-                        if (fp64) {
-                            a0 = fma(w0, x0, a0);
-                            a1 = fma(w1, x1, a1);
-                            a2 = fma(w2, x2, a2);
-                            a3 = fma(w3, x3, a3);
-                        } else {
-                            a0 += w0 * (xi - x0);
-                            a1 += w1 * (xi - x1);
-                            a2 += w2 * (xi - x2);
-                            a3 += w3 * (xi - x3);
-                        }
+                        const double w0 = s_w[e], w1 = s_w[e + G], w2 = s_w[e + 2 * G], w3 = s_w[e + 3 * G];
+                        a0 = fma(w0, x[c0], a0);
+                        a1 = fma(w1, x[c1], a1);
+                        a2 = fma(w2, x[c2], a2);
+                        a3 = fma(w3, x[c3], a3);
                     }
-                    for (; e < e1; e += G) {
-                        if (fp64) a0 = fma(s_w[e], x[s_col[e]], a0);
-                        else a0 += s_w[e] * (xi - x[s_col[e]]);
-                    }
+                    for (; e < e1; e += G) a0 = fma(s_w[e], x[s_col[e]], a0);
                     ac = (a0 + a1) + (a2 + a3);
                 }
                 ac = group_sum<G>(ac);
-                if (lane == 0 && warp == 1) TRACE(s, 5);
+                // only the lanes leading a row group hold sums
                 if (i < n && rlane == 0) {
-                    T yv;
-                    if (fp64) yv = (T)((fma(s_gd[i], (double)xi, (double)ac) - (double)gm) * (double)sig);
-                    else yv = (g * (xi - mT) - ac) * sig;
+                    const double yv = (fma(s_gd[i], xi, ac) - sl.gm_d) * sl.sig_d;
                     y[i] = yv;
                     acc.add(yv, xi);
                 }
-                if (lane == 0 && warp == 1) TRACE(s, 6);
             }
-            // only the lanes leading a row group hold sums
-            if constexpr (sizeof(T) == 8) {
-                double *dst = s_dacc + ((size_t)((s + 1) & 1) * blockDim.x + tid) * 3;
-                dst[0] = acc.A;
-                dst[1] = acc.B;
-                dst[2] = acc.C;
-            } else {
-                const Part p = warp_sum_part(acc.get(), G);
-                if (lane == 0) s_pw[(s + 1) & 1][warp] = p;
-            }
-            if (lane == 0 && warp == 1) TRACE(s, 2);
-            if (lane == 0 && warp == nw - 1) TRACE(s, 3);
+            double *dst = s_dacc + ((size_t)((s + 1) & 1) * blockDim.x + tid) * 3;
+            dst[0] = acc.A;
+            dst[1] = acc.B;
+            dst[2] = acc.C;
         }
         __syncthreads();
         s++;
@@ -1351,7 +1069,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_power_small(PiArgs a, Grid
     if (warp == 0) {
         if (exit_kind == 2 && !no_sweeps) {
             const Part q = ctl_part(s & 1);
-            if (lane == 0) ctrl_step(a, s, q, c, nullptr, true, fp64);
+            if (lane == 0) ctrl_step(a, s, q, c, nullptr, true, true);
         }
         if (lane == 0) {
             const int rs = c.res_sweep;
@@ -1362,354 +1080,11 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_power_small(PiArgs a, Grid
     }
     __syncthreads();
     // result -> buf[0], previous iterate -> buf[1]
-    T *o0 = (T *)a.buf[0], *o1 = (T *)a.buf[1];
-    const T *rr = ring0 + (size_t)s_rb * n, *rp = ring0 + (size_t)s_rbp * n;
+    double *o0 = (double *)a.buf[0], *o1 = (double *)a.buf[1];
+    const double *rr = ring0 + (size_t)s_rb * n, *rp = ring0 + (size_t)s_rbp * n;
     for (int i = tid; i < n; i += blockDim.x) {
-        const int r = sell ? s_perm[i] : i;
-        o0[r] = rr[i];
-        o1[r] = rp[i];
-    }
-}
-
-// ================================================================== cluster kernel
-// FP64 sweeps of a level spread over one thread-block cluster of C CTAs
-// (2..8, one per SM).  Every CTA holds the whole iterate ring (3 x n rows
-// rounded up to whole slices) and g - d_i of every row, and the SELL-32
-// slices of its share of the rows (rows in slot order, slices split into C
-// ranges of about equal SELL size).  A sweep: the row warps compute their rows from the
-// local iterate (each warp's stop sums summed over its lanes as float-
-// float); then all threads copy the CTA's row block, in 16-byte pieces, into
-// every other CTA's ring (distributed shared memory) while the control warp
-// sums the warps' stop sums and stores the total into every CTA's slot
-// [sweep parity][rank]; then the cluster meets at its barrier.  Every
-// CTA's control warp sums the C slots in rank order and takes the same
-// decisions, so all CTAs run the same sweeps and reach the same barriers.
-// A CTA is at most one sweep ahead of another (one barrier per sweep), so
-// two slot parities and the ring of three keep stores and reads apart.
-constexpr int kClusterMax = 8;
-
-__device__ __forceinline__ unsigned cluster_rank() {
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ unsigned cluster_ctas() {
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
-// every thread of every CTA of the cluster; orders the distributed
-// shared-memory stores before it with the reads after it
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ unsigned cluster_addr(const void *local, unsigned cta) {
-    const unsigned la = (unsigned)__cvta_generic_to_shared(local);
-    unsigned ra;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(cta));
-    return ra;
-}
-__device__ __forceinline__ void st_cluster_f32(float *local, unsigned cta, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(local, cta)), "f"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster_v2f64(double2 *local, unsigned cta, double2 v) {
-    asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(cluster_addr(local, cta)), "d"(v.x), "d"(v.y)
-                 : "memory");
-}
-
-// First slice of each of C ranges of about equal SELL-32 size, from the
-// prefix sums pre[0..nsl] of the slices' sizes (the host plans with the same
-// arithmetic).
-__host__ __device__ __forceinline__ int cluster_split(const int *pre, int nsl, int C, int r) {
-    if (r <= 0) return 0;
-    if (r >= C) return nsl;
-    const long long target = (long long)pre[nsl] * r / C;
-    int lo = 0, hi = nsl;   // first q with pre[q] >= target
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if ((long long)pre[mid] < target) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
-
-__global__ void __launch_bounds__(kSmallMaxThreads) k_power_cluster(PiArgs a, GridSync *) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int n = a.n, nsl = (n + 31) / 32, nr = 32 * nsl;   // ring slots hold whole slices
-    const int C = (int)cluster_ctas();
-    const unsigned rank = cluster_rank();
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int nw = blockDim.x >> 5, nrw = nw - 1, rw = warp - 1;
-    double *ring0 = reinterpret_cast<double *>(smem_raw);      // [3][nr]
-    double *s_gd = ring0 + 3 * (size_t)nr;                      // [nr]
-    Part *s_cpart = reinterpret_cast<Part *>(s_gd + nr);        // [2][kClusterMax]: CTAs' stop sums
-    double *s_w = reinterpret_cast<double *>(s_cpart + 2 * kClusterMax);   // [emax]
-    int *s_col = reinterpret_cast<int *>(s_w + a.cl_emax);
-    int *s_pre = s_col + a.cl_emax;                             // [nsl + 1]
-    int *s_perm = s_pre + nsl + 1;                              // [n]: row of each slot
-    __shared__ Part s_pw[32];
-    __shared__ Slot s_slot[2];
-    __shared__ int s_q[2];
-    const double g = a.g;
-
-    // ---- slot order (the same in every CTA); inv and the sort's scratch
-    // borrow ring slots 1 and 2, cleared below
-    const int *s_inv = reinterpret_cast<const int *>(ring0 + nr);
-    slot_order(n, a.rp, s_perm, reinterpret_cast<int *>(ring0 + nr), reinterpret_cast<int *>(ring0 + 2 * (size_t)nr));
-    // ---- the slices' SELL-32 sizes, this CTA's range and its entries
-    for (int q = tid; q < nsl; q += blockDim.x) {
-        int L = 0;
-        for (int p = 32 * q; p < min(n, 32 * q + 32); p++) {
-            const int r = s_perm[p];
-            L = max(L, a.rp[r + 1] - a.rp[r]);
-        }
-        s_pre[q + 1] = 32 * L;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        s_pre[0] = 0;
-        for (int q = 0; q < nsl; q++) s_pre[q + 1] += s_pre[q];
-        s_q[0] = cluster_split(s_pre, nsl, C, (int)rank);
-        s_q[1] = cluster_split(s_pre, nsl, C, (int)rank + 1);
-    }
-    __syncthreads();
-    const int q0 = s_q[0], q1 = s_q[1], e_base = s_pre[q0];
-    for (int p = 32 * q0 + tid; p < 32 * q1; p += blockDim.x) {
-        const int q = p >> 5, l = p & 31;
-        const int L = (s_pre[q + 1] - s_pre[q]) >> 5;
-        const int r = (p < n) ? s_perm[p] : 0;
-        const int e0 = (p < n) ? a.rp[r] : 0;
-        const int len = (p < n) ? a.rp[r + 1] - e0 : 0;
-        for (int k = 0; k < L; k++) {
-            const int idx = s_pre[q] - e_base + 32 * k + l;
-            if (k < len) {
-                s_col[idx] = s_inv[a.col[e0 + k]];
-                s_w[idx] = a.w[e0 + k];
-            } else {
-                s_col[idx] = (p < n) ? p : 0;   // zero weight: no contribution
-                s_w[idx] = 0.0;
-            }
-        }
-    }
-    __syncthreads();   // inv read before ring slots 1 and 2 are cleared
-    // ---- start vector and g - d_i of every slot (the same in every CTA)
-    {
-        const void *cb = nullptr;
-        double cmu = 0.0, cinv = 0.0;
-        if (a.start == 1) {
-            cb = a.cbuf[a.cres->buf];
-            cmu = a.cres->mu;
-            cinv = a.cres->inv_s;
-        }
-        Part acc = part_zero();
-        for (int i = tid; i < nr; i += blockDim.x) {
-            double xt = 0.0, gd = 0.0;
-            if (i < n) {
-                const int r = s_perm[i];
-                xt = start_value(a, r, cb, cmu, cinv);
-                double d = 0.0;
-                for (int e = a.rp[r], e1 = a.rp[r + 1]; e < e1; e++) d += a.w[e];
-                gd = g - d;
-                const ff v = ff_from_double(xt);
-                acc.A = ff_add(acc.A, v);
-                acc.B = ff_add(acc.B, ff_mul(v, v));
-            }
-            ring0[i] = xt;
-            ring0[nr + i] = 0.0;
-            ring0[2 * (size_t)nr + i] = 0.0;
-            s_gd[i] = gd;
-        }
-        Part p = warp_sum_part(acc);
-        if (lane == 0) s_pw[warp] = p;
-    }
-    __syncthreads();
-    __shared__ Ctl c;   // used by lane 0 of the control warp (in registers it would take every row thread's)
-    if (warp == 0) {
-        Part q = (lane < nw) ? s_pw[lane] : part_zero();
-        q = warp_sum_part(q);
-        const double mu0 = to_d(q.A) / (double)n;
-        double ss0 = to_d(q.B) - (double)n * mu0 * mu0;
-        if (ss0 < 0.0) ss0 = 0.0;
-        const int e0 = start_exponent(ss0);
-        if (lane == 0) {
-            ctl_init(c, a, mu0, ss0, e0);
-            s_slot[1] = slot_make(ff_from_double(mu0), e0, a.g, c.inv_g, true);
-            s_slot[0] = slot_make(ff_zero(), 0, a.g, c.inv_g, true);
-        }
-    }
-    __syncthreads();
-    // every CTA's shared memory is set up before any CTA stores into it
-    cluster_barrier();
-
-    // the C CTAs' stop sums of parity par, in rank order (every lane)
-    auto cluster_part = [&](int par) -> Part {
-        Part q = part_zero();
-        for (int r = 0; r < C; r++) q = part_add(q, s_cpart[par * kClusterMax + r]);
-        return q;
-    };
-    // this CTA's row block, in 16-byte pieces, into every other CTA's ring
-    const int rb0 = 32 * q0, rb_pairs = 16 * (q1 - q0);
-
-    const bool no_sweeps = (a.mode == 1 && a.k_fixed <= 0);
-    int s = 0;
-    int exit_kind = no_sweeps ? 2 : 0;
-    while (!no_sweeps) {
-        const Slot sl = s_slot[(s + 1) & 1];
-        if (sl.stop) {
-            exit_kind = 1;
-            break;
-        }
-        if ((a.mode == 1 && s >= a.k_fixed) || (a.mode == 0 && s >= a.max_sweeps)) {
-            exit_kind = 2;
-            break;
-        }
-        const double *x = ring0 + (size_t)(s % 3) * nr;
-        double *y = ring0 + (size_t)((s + 1) % 3) * nr;
-        CLT(s, 0);
-        if (warp == 0) {
-            if (s >= 1) {
-                const Part q = cluster_part((s - 1) & 1);
-                if (lane == 0) ctrl_step(a, s, q, c, &s_slot[s & 1], false, true);
-            }
-        } else {
-            const double mT = sl.m_d, sig = sl.sig_d, gm = sl.gm_d;
-            Acc<double> acc;
-            acc.reset();
-            for (int q = q0 + rw; q < q1; q += nrw) {
-                const int i = 32 * q + lane;
-                const int off = s_pre[q] - e_base + lane;
-                const int L = (s_pre[q + 1] - s_pre[q]) >> 5;
-                const double xi = x[i];
-                double a0 = 0.0, a1 = 0.0;
-                int k = 0;
-                for (; k + 1 < L; k += 2) {
-                    a0 = fma(s_w[off + 32 * k], x[s_col[off + 32 * k]], a0);
-                    a1 = fma(s_w[off + 32 * k + 32], x[s_col[off + 32 * k + 32]], a1);
-                }
-                if (k < L) a0 = fma(s_w[off + 32 * k], x[s_col[off + 32 * k]], a0);
-                if (i < n) {
-                    const double yv = (fma(s_gd[i], xi, a0 + a1) - gm) * sig;
-                    y[i] = yv;
-                    acc.add(yv, xi);
-                }
-            }
-            // the warp's stop sums as float-float, summed over its lanes
-            const Part p = warp_sum_part(acc.get());
-            if (lane == 0) s_pw[warp] = p;
-        }
-        __syncthreads();
-        CLT(s, 1);
-        if (warp == 0) {
-            // this CTA's stop sums (row warps in order) into every CTA's slot
-            Part q = (lane >= 1 && lane < nw) ? s_pw[lane] : part_zero();
-            q = warp_sum_part(q);
-            if (lane < C) {
-                Part *slot = s_cpart + (s & 1) * kClusterMax + rank;
-                if (lane == (int)rank) {
-                    *slot = q;
-                } else {
-                    const float *src = reinterpret_cast<const float *>(&q);
-                    float *dst = reinterpret_cast<float *>(slot);
-                    for (int k = 0; k < 6; k++) st_cluster_f32(dst + k, (unsigned)lane, src[k]);
-                }
-            }
-        }
-        for (int k = tid; k < (C - 1) * rb_pairs; k += blockDim.x) {
-            const int pr = k / rb_pairs, j = k - pr * rb_pairs;
-            const unsigned peer = (unsigned)(pr < (int)rank ? pr : pr + 1);
-            const double2 v = reinterpret_cast<const double2 *>(y + rb0)[j];
-            st_cluster_v2f64(reinterpret_cast<double2 *>(y + rb0) + j, peer, v);
-        }
-        CLT(s, 2);
-        cluster_barrier();
-        CLT(s, 3);
-        s++;
-    }
-    __shared__ int s_rb, s_rbp;
-    if (warp == 0) {
-        if (exit_kind == 2 && !no_sweeps) {
-            const Part q = cluster_part((s - 1) & 1);
-            if (lane == 0) ctrl_step(a, s, q, c, nullptr, true, true);
-        }
-        if (lane == 0) {
-            const int rs = c.res_sweep;
-            s_rb = c.zero ? (rs + 2) % 3 : rs % 3;
-            s_rbp = (rs + 2) % 3;
-            if (rank == 0) write_result(a, c, 0, 1);
-        }
-    }
-    __syncthreads();
-    if (rank == 0) {
-        // result -> buf[0], previous iterate -> buf[1]
-        double *o0 = (double *)a.buf[0], *o1 = (double *)a.buf[1];
-        const double *rr = ring0 + (size_t)s_rb * nr, *rp = ring0 + (size_t)s_rbp * nr;
-        for (int i = tid; i < n; i += blockDim.x) {
-            o0[s_perm[i]] = rr[i];
-            o1[s_perm[i]] = rp[i];
-        }
-    }
-}
-
-static size_t cluster_smem(int n, int, int emax) {
-    const int nsl = (n + 31) / 32, nr = 32 * nsl;
-    return 8 * (4 * (size_t)nr + (size_t)emax) + sizeof(Part) * 2 * kClusterMax +
-           4 * ((size_t)emax + nsl + 1 + (size_t)n) + 16;
-}
-
-// Shared memory a cluster CTA may take (0: unknown).
-static long long cluster_room() {
-    DeviceInfo d;
-    if (device_info(&d) != CMG_OK) return 0;
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, (const void *)k_power_cluster) != cudaSuccess) return 0;
-    return (long long)d.max_smem_optin - (long long)fa.sharedSizeBytes - 1024;
-}
-
-bool cluster_may_hold(int n) {
-    return n >= 128 && n <= 65536 && (long long)cluster_smem(n, 0, 0) <= cluster_room();
-}
-
-void cluster_plan(PiLevel *lv, const int *rph) {
-    lv->cl_ctas = 0;
-    const int n = lv->n;
-    if (!cluster_may_hold(n)) return;
-    const long long room = cluster_room();
-    const int nsl = (n + 31) / 32;
-    std::vector<int> pre;
-    slot_sell_prefix(n, rph, pre);
-    // about 96 rows per CTA: enough FP64 work per SM to repay the barrier
-    for (int C = std::max(2, std::min(kClusterMax, (n + 95) / 96)); C <= kClusterMax; C++) {
-        int emax = 0, smax = 0;
-        for (int r = 0; r < C; r++) {
-            const int a0 = cluster_split(pre.data(), nsl, C, r), a1 = cluster_split(pre.data(), nsl, C, r + 1);
-            emax = std::max(emax, pre[a1] - pre[a0]);
-            smax = std::max(smax, a1 - a0);
-        }
-        const int threads = 32 * (1 + std::max(1, std::min(31, smax)));
-        const size_t smem = cluster_smem(n, threads, emax);
-        if ((long long)smem > room) continue;
-        if (allow_max_dynamic_smem((const void *)k_power_cluster) != CMG_OK) return;
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)C;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.gridDim = dim3((unsigned)C);
-        cfg.blockDim = dim3((unsigned)threads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        int ncl = 0;
-        if (cudaOccupancyMaxActiveClusters(&ncl, (const void *)k_power_cluster, &cfg) != cudaSuccess || ncl < 1) {
-            cudaGetLastError();
-            return;
-        }
-        lv->cl_ctas = C;
-        lv->cl_threads = threads;
-        lv->cl_emax = emax;
-        lv->cl_smem = smem;
-        return;
+        o0[i] = rr[i];
+        o1[i] = rp[i];
     }
 }
 
@@ -1767,33 +1142,23 @@ static const void *sell_kernel(int fp32, int col16, bool chunks, bool stream, bo
                  : sell_kernel_ti<double, int>(chunks, stream, stage);
 }
 
-template <typename T>
 static const void *small_kernel(int G) {
     switch (G) {
-        case 1: return (const void *)k_power_small<T, 1>;
-        case 2: return (const void *)k_power_small<T, 2>;
-        case 4: return (const void *)k_power_small<T, 4>;
-        case 8: return (const void *)k_power_small<T, 8>;
-        case 16: return (const void *)k_power_small<T, 16>;
-        default: return (const void *)k_power_small<T, 32>;
+        case 1: return (const void *)k_power_small<1>;
+        case 2: return (const void *)k_power_small<2>;
+        case 4: return (const void *)k_power_small<4>;
+        case 8: return (const void *)k_power_small<8>;
+        case 16: return (const void *)k_power_small<16>;
+        default: return (const void *)k_power_small<32>;
     }
 }
 
-// Lanes per row in the small kernel: about 4 entries per lane, fewer lanes
-// when that leaves more row groups than rows would need.
-static int small_lanes(int n, long long nnz, int fp32) {
+// Lanes per row in the small kernel: every lane-operation costs FP64 issue
+// slots, so the fewest lanes that keep each lane's dependent FMA chain short.
+static int small_lanes(int n, long long nnz) {
     const double avg = (double)nnz / (double)std::max(1, n);
     int g = 1;
-    if (fp32) {
-        // a row per lane while a lane's (unrolled) entry loop stays short:
-        // every lane that holds a row pays its share of the per-sweep
-        // float-float reduction
-        while (g < 32 && g * 32 < avg) g <<= 1;
-    } else {
-        // FP64: every lane-operation costs FP64 issue slots, so use the fewest
-        // lanes that keep each lane's dependent FMA chain short
-        while (g < 32 && g * 16 < avg) g <<= 1;
-    }
+    while (g < 32 && g * 16 < avg) g <<= 1;
     return g;
 }
 
@@ -1805,17 +1170,9 @@ static int small_threads(int n, int G) {
     return 32 * (w + 1);
 }
 
-// Entries the small kernel stores: the SELL-32 size with one lane per row
-// (when known), else the CSR size.
-static long long small_entries(const PiLevel &lv, int G) {
-    return (G == 1 && lv.sell_nnz > 0) ? lv.sell_nnz : lv.nnz;
-}
-
-static size_t small_bytes(const PiLevel &lv, int G, int fp32) {
-    const long long e = small_entries(lv, G);
-    if (fp32) return small_smem_bytes<float>(lv.n, e);
-    // plus the row threads' FP64 stop sums: 2 parities x 3 doubles per thread
-    return small_smem_bytes<double>(lv.n, e) + 8 + 48 * (size_t)small_threads(lv.n, G);
+static size_t small_bytes(const PiLevel &lv, int G) {
+    return 8 * (4 * (size_t)lv.n + (size_t)lv.nnz + 6 * (size_t)small_threads(lv.n, G)) +
+           4 * ((size_t)lv.n + 1 + (size_t)lv.nnz) + 16;
 }
 
 size_t xsweep_smem(int fp32) {
@@ -1845,44 +1202,14 @@ int stage_capacity(int fp32) {
 }
 
 // Lanes per row with which the small kernel holds the level (0: it cannot).
-static int small_config(const PiLevel &lv, int fp32) {
+static int small_config(const PiLevel &lv) {
     DeviceInfo d;
     if (device_info(&d) != CMG_OK) return 0;
-    const int G = small_lanes(lv.n, lv.nnz, fp32);
-    return small_bytes(lv, G, fp32) + 4096 <= (size_t)d.max_smem_optin ? G : 0;
+    const int G = small_lanes(lv.n, lv.nnz);
+    return small_bytes(lv, G) + 4096 <= (size_t)d.max_smem_optin ? G : 0;
 }
 
-bool small_level_fits(const PiLevel &lv, int fp32) { return small_config(lv, fp32) > 0; }
-
-__global__ void k_sell_size(int n_static, const int *__restrict__ n_dev, const int *__restrict__ rp,
-                            unsigned long long *out) {
-    const int n = n_dev ? *n_dev : n_static;
-    const int nsl = (n + 31) / 32;
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nsl; q += gridDim.x * blockDim.x) {
-        int L = 0;
-        for (int r = 32 * q; r < min(n, 32 * q + 32); r++) L = max(L, rp[r + 1] - rp[r]);
-        atomicAdd(out, (unsigned long long)(32 * L));
-    }
-}
-
-cmg_status_t sell_size(int n, const int *rp, unsigned long long *dev_counter, long long *out,
-                       cudaStream_t s) {
-    CMG_CUDA(cudaMemsetAsync(dev_counter, 0, sizeof(unsigned long long), s));
-    k_sell_size<<<grid_for((n + 31) / 32, 256), 256, 0, s>>>(n, nullptr, rp, dev_counter);
-    CMG_TRY(launch_status());
-    unsigned long long v = 0;
-    CMG_CUDA(cudaMemcpyAsync(&v, dev_counter, sizeof(v), cudaMemcpyDeviceToHost, s));
-    CMG_CUDA(cudaStreamSynchronize(s));
-    *out = (long long)v;
-    return CMG_OK;
-}
-
-cmg_status_t sell_size_async(const int *n_dev, int n_cap, const int *rp,
-                             unsigned long long *dev_counter, cudaStream_t s) {
-    CMG_CUDA(cudaMemsetAsync(dev_counter, 0, sizeof(unsigned long long), s));
-    k_sell_size<<<grid_for((n_cap + 31) / 32, 256), 256, 0, s>>>(n_cap, n_dev, rp, dev_counter);
-    return launch_status();
-}
+bool small_level_fits(const PiLevel &lv, int fp32) { return !fp32 && small_config(lv) > 0; }
 
 cmg_status_t power_iteration(const PiRun &run, GridSync *gs, cudaStream_t s, const PiWorkspace *ws) {
     const PiLevel &lv = *run.lv;
@@ -1914,7 +1241,6 @@ cmg_status_t power_iteration(const PiRun &run, GridSync *gs, cudaStream_t s, con
     a.res = run.res;
     a.partials = nullptr;
     a.zero_tol2 = run.fp32 ? kZeroTol2_32 : kZeroTol2_64;
-    a.sell_nnz = lv.sell_nnz;
     a.cinvp = run.coarse_inv;
     a.perm = nullptr;
     a.lay_h = a.lay_nsl = 0;
@@ -1928,29 +1254,11 @@ cmg_status_t power_iteration(const PiRun &run, GridSync *gs, cudaStream_t s, con
     a.stream_hint = 0;
     a.stage_n = 0;
     void *args[] = {&a, &gs};
-    if (lv.cl_ctas > 0 && !run.fp32 && !lv.lay) {
-        // FP64 sweeps in one thread-block cluster
-        a.cl_emax = lv.cl_emax;
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)lv.cl_ctas;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.gridDim = dim3((unsigned)lv.cl_ctas);
-        cfg.blockDim = dim3((unsigned)lv.cl_threads);
-        cfg.dynamicSmemBytes = lv.cl_smem;
-        cfg.stream = s;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        CMG_TRY(allow_max_dynamic_smem((const void *)k_power_cluster));
-        CMG_CUDA(cudaLaunchKernelExC(&cfg, (const void *)k_power_cluster, args));
-        return launch_status();
-    }
+    if (lv.fix && !run.fp32) return launch_power_fix(*lv.fix, a, s);
     if (small_level_fits(lv, run.fp32)) {
-        const int G = small_config(lv, run.fp32);
-        const void *kern = run.fp32 ? small_kernel<float>(G) : small_kernel<double>(G);
-        const size_t smem = small_bytes(lv, G, run.fp32);
+        const int G = small_config(lv);
+        const void *kern = small_kernel(G);
+        const size_t smem = small_bytes(lv, G);
         CMG_TRY(allow_max_dynamic_smem(kern));
         return coop_launch(kern, 1, small_threads(lv.n, G), smem, s, args, gs);
     }
@@ -2385,9 +1693,3 @@ cmg_status_t finalize(const PiLevel &lv, int fp32, void *const bufs[3], const Pi
 }
 
 }  // namespace cmg
-
-#ifdef CMG_TRACE
-extern "C" int cmg_debug_trace(long long *out) {
-    return (int)cudaMemcpyFromSymbol(out, cmg::g_trace, sizeof(cmg::g_trace));
-}
-#endif

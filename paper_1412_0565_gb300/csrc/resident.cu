@@ -4,7 +4,7 @@
 // rows to the CTAs.
 #include <algorithm>
 
-#include "pi_kernels.cuh"
+#include "fixed.cuh"
 
 namespace cmg {
 
@@ -22,14 +22,6 @@ constexpr int kItemCost = 256;     // per item, in entries: the rows' finish and
 constexpr int kCtaWork = 2048;
 constexpr int kPlanThreads = 1024;
 constexpr int kRowsMaxRow = 4096;  // longest row the FP64 items take (one warp each)
-
-struct PlanOut {
-    int P;                     // CTAs (at most the number asked for)
-    int ni;
-    int max_e, max_i, max_r;   // most entries, items and rows of one CTA
-    long long entries;
-    int maxdeg;
-};
 
 __device__ __forceinline__ int plan_deg(const int *rp, const uint32_t *perm, int p) {
     const int v = (int)perm[p];
@@ -64,12 +56,13 @@ __device__ __forceinline__ int plan_scan(int v, int *sm, int *total) {
 
 // P is cut to one CTA per kCtaWork; CTA p takes the items from the first whose entries before it, at kItemCost
 // more per item, reach p / P of the total.
-__device__ __forceinline__ void plan_ranges(int P, int ni, const int4 *item, int *range, PlanOut *out) {
+// (cut: false takes P as it is)
+__device__ __forceinline__ void plan_ranges(int P, bool cut, int ni, const int4 *item, int *range, PlanOut *out) {
     const int tid = threadIdx.x;
     __shared__ int s_max[3];
     if (tid < 3) s_max[tid] = 0;
     const long long total = (long long)item[ni].y + (long long)kItemCost * ni;
-    P = (int)min((long long)P, total / kCtaWork + 1);
+    if (cut) P = (int)min((long long)P, total / kCtaWork + 1);
     for (int p = tid; p <= P; p += blockDim.x) {
         const long long target = total * p / P;
         int lo = 0, hi = ni;
@@ -98,14 +91,13 @@ __device__ __forceinline__ void plan_ranges(int P, int ni, const int4 *item, int
     }
 }
 
-// FP64 items of the rows in degree order (perm), one CTA: rows longer than 16 S
-// take 32 lanes each, rows longer than 8 S 16 lanes, ... rows of at most S
-// one lane; an item is 32 lanes (32 / G rows), as many steps as its first
-// (longest) row needs.
-__global__ void __launch_bounds__(kPlanThreads) k_plan_units(int n, const int *__restrict__ rp,
-                                                             const uint32_t *__restrict__ perm, int S, int P,
-                                                             int4 *__restrict__ item, int *__restrict__ range,
-                                                             PlanOut *__restrict__ out) {
+// Items of n rows in degree order, one CTA: rows longer than 16 S entries take 32
+// lanes each, rows longer than 8 S 16 lanes, ... rows of at most S one lane; an
+// item is 32 lanes (32 / G rows) and as many steps as its first (longest) row
+// needs.  deg(p): length of the row at position p.  At most cap items are
+// written; returns their number.
+template <typename DEG>
+__device__ __forceinline__ int plan_units(int n, int S, DEG deg, int cap, int4 *item) {
     __shared__ int s_row[7], s_unit[7], s_sm[32];
     const int tid = threadIdx.x;
     if (tid < 7) {
@@ -114,7 +106,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_units(int n, const int *_
         int lo = 0, hi = n;
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;
-            if (plan_deg(rp, perm, mid) > thr) lo = mid + 1;
+            if (deg(mid) > thr) lo = mid + 1;
             else hi = mid;
         }
         s_row[tid] = lo;
@@ -143,7 +135,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_units(int n, const int *_
                 r0[k] = s_row[c] + ((u - s_unit[c]) << c);
                 const int rows = min(1 << c, s_row[c + 1] - r0[k]);
                 lw[k] = (5 - c) | (rows << 3);
-                st[k] = (plan_deg(rp, perm, r0[k]) + (32 >> c) - 1) >> (5 - c);
+                st[k] = (deg(r0[k]) + (32 >> c) - 1) >> (5 - c);
             }
             sum += st[k];
         }
@@ -152,18 +144,136 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_units(int n, const int *_
 #pragma unroll
         for (int k = 0; k < K; k++) {
             const int u = u0 + tid * K + k;
-            if (u < nu) item[u] = make_int4(r0[k], (int)(32 * off), st[k], lw[k]);
+            if (u < nu && u < cap) item[u] = make_int4(r0[k], (int)(32 * off), st[k], lw[k]);
             off += st[k];
         }
         run += tot;
     }
+    // beyond 32-bit offsets: the caller sees the entry count
+    if (tid == 0) item[min(nu, cap)] = make_int4(n, run > 0x3ffffff ? 0x7fffffff : (int)(32 * run), 0, 0);
+    __syncthreads();
+    return nu;
+}
+
+__global__ void __launch_bounds__(kPlanThreads) k_plan_units(int n, const int *__restrict__ rp,
+                                                             const uint32_t *__restrict__ perm, int S, int P, int cap,
+                                                             int4 *__restrict__ item, int *__restrict__ range,
+                                                             PlanOut *__restrict__ out) {
+    const int nu = plan_units(n, S, [&](int p) { return plan_deg(rp, perm, p); }, cap, item);
+    if (threadIdx.x == 0) out->maxdeg = plan_deg(rp, perm, 0);
+    plan_ranges(P, true, min(nu, cap), item, range, out);
+}
+
+// Everything k_power_fix needs of a level of at most kFixMaxN rows, one CTA per
+// level and one launch for all of them: degree order (a stable counting sort),
+// items and ranges, entries and diagonal in fixed point.  (The one-CTA and
+// cluster kernels sorted and laid out their level in the sweep launch itself,
+// and the cluster's plan read its row pointers back to the host.)
+__global__ void __launch_bounds__(kPlanThreads) k_plan_small(const SmallJob *__restrict__ jobs) {
+    __shared__ SmallJob J;
+    __shared__ unsigned short s_perm[kFixMaxN], s_inv[kFixMaxN];
+    __shared__ int s_hist[kFixMaxN + 1];
+    __shared__ int s_md;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
-        // beyond 32-bit offsets: the caller sees the entry count
-        item[nu] = make_int4(n, run > 0x3ffffff ? 0x7fffffff : (int)(32 * run), 0, 0);
-        out->maxdeg = n > 0 ? plan_deg(rp, perm, 0) : 0;
+        J = jobs[blockIdx.x];
+        s_md = 0;
     }
     __syncthreads();
-    plan_ranges(P, nu, item, range, out);
+    const int n = J.n;
+    // the sort's bucket (degrees of valid rows are below n)
+    auto len = [&](int i) { return J.rp[i + 1] - J.rp[i]; };
+    for (int i = tid; i < n; i += kPlanThreads) atomicMax(&s_md, min(len(i), kFixMaxN - 1));
+    __syncthreads();
+    const int D = s_md;
+    for (int b = tid; b <= D; b += kPlanThreads) s_hist[b] = 0;
+    __syncthreads();
+    for (int i = tid; i < n; i += kPlanThreads) {
+        const int b = D - min(len(i), kFixMaxN - 1);
+        s_inv[i] = (unsigned short)b;
+        atomicAdd(&s_hist[b], 1);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        int carry = 0;
+        for (int b0 = 0; b0 <= D; b0 += 32) {
+            const int b = b0 + lane;
+            const int c = b <= D ? s_hist[b] : 0;
+            int incl = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            if (b <= D) s_hist[b] = carry + incl - c;
+            carry += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        __syncwarp();
+        for (int i0 = 0; i0 < n; i0 += 32) {
+            const int i = i0 + lane;
+            const unsigned act = __ballot_sync(0xffffffffu, i < n);
+            if (i < n) {
+                const int b = s_inv[i];
+                const unsigned peers = __match_any_sync(act, b);
+                const int r = __popc(peers & ((1u << lane) - 1u));
+                const int base = s_hist[b];
+                s_perm[base + r] = (unsigned short)i;
+                __syncwarp(act);
+                if (r == 0) s_hist[b] = base + __popc(peers);
+            }
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    for (int p = tid; p < n; p += kPlanThreads) {
+        s_inv[s_perm[p]] = (unsigned short)p;
+        J.perm[p] = s_perm[p];
+    }
+    __syncthreads();
+    // one item per row warp: of at most 8 steps where one CTA holds them all, else
+    // of 16; beyond the warps, items of up to J.S steps dealt by their entries
+    auto deg = [&](int p) { return len(s_perm[p]); };
+    int nu = plan_units(n, 8, deg, J.cap_items, J.item);
+    int steps = D <= 256 && nu <= J.one_cta ? 8 : 0;
+    if (!steps) {
+        nu = plan_units(n, 16, deg, J.cap_items, J.item);
+        if (D <= 512 && nu <= J.cap_warps) steps = 16;
+        else if (J.S != 16) nu = plan_units(n, J.S, deg, J.cap_items, J.item);
+    }
+    plan_ranges(J.C, false, min(nu, J.cap_items), J.item, J.range, J.out);
+    const bool fits = nu <= J.cap_items && J.item[nu].y <= J.cap_entries;
+    if (tid == 0) {
+        J.out->by_warp = steps;
+        J.out->maxdeg = fits ? 0 : -1;   // -1: beyond the capacities, not filled
+        if (!fits) J.out->ni = 0;
+    }
+    if (!fits) return;
+    for (int u = warp; u < nu; u += kPlanThreads / 32) {
+        const int4 it = J.item[u];
+        const int lg = it.w & 7, rows = it.w >> 3, r = lane >> lg, g = lane & ((1 << lg) - 1);
+        const int p = it.x + (r < rows ? r : 0);
+        int e0 = 0, deg = 0;
+        if (r < rows) {
+            e0 = J.rp[s_perm[p]];
+            deg = len(s_perm[p]);
+        }
+        long long sum = 0;
+        for (int t = 0; t < it.z; t++) {
+            const int k = (t << lg) + g;
+            const int d = it.y + 32 * t + lane;
+            long long Cij = 0;
+            int cl = p;
+            if (k < deg) {
+                Cij = fix_weight(J.w[e0 + k], J.ginv, J.ge);
+                cl = s_inv[J.col[e0 + k]];
+            }
+            J.ucol[d] = (uint16_t)cl;
+            J.uc[d] = fix_split(Cij);
+            sum += Cij;
+        }
+        for (int o = (1 << lg) >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (r < rows && g == 0) J.ud[p] = fix_split(sum);
+    }
 }
 
 // FP32 items are those of the sweep layout: its heavy rows (lw = -1, z their
@@ -182,7 +292,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_slices(int n, int h, int 
         out->maxdeg = 0;
     }
     __syncthreads();
-    plan_ranges(P, ni, item, range, out);
+    plan_ranges(P, true, ni, item, range, out);
 }
 
 // Entries of the FP64 items, a warp per item; short rows and missing rows are
@@ -478,6 +588,11 @@ static const void *rows_kernel(const RowPlan &R) {
     return R.col16 ? rows_kernel_t<double, uint16_t>(R) : rows_kernel_t<double, int>(R);
 }
 
+cmg_status_t launch_plan_small(const SmallJob *jobs_dev, int count, cudaStream_t s) {
+    k_plan_small<<<count, kPlanThreads, 0, s>>>(jobs_dev);
+    return launch_status();
+}
+
 int rows_threads(const RowPlan &R) { return R.resident ? 1024 : 512; }
 
 static size_t rows_smem(int n, int fp32, int col16, int stage, const PlanOut &o) {
@@ -541,7 +656,7 @@ cmg_status_t build_row_plan(int n, long long nnz, const int *rp, const int *col,
             const int h = L.hheavy[0];
             k_plan_slices<<<1, kPlanThreads, 0, s>>>(n, h, (n - h + 31) / 32, L.meta, P, item, R->range, out_dev);
         } else {
-            k_plan_units<<<1, kPlanThreads, 0, s>>>(n, rp, L.perm, S, P, item, R->range, out_dev);
+            k_plan_units<<<1, kPlanThreads, 0, s>>>(n, rp, L.perm, S, P, (int)cap, item, R->range, out_dev);
         }
         CMG_TRY(launch_status());
         CMG_CUDA(cudaMemcpyAsync(&o, out_dev, sizeof(o), cudaMemcpyDeviceToHost, s));
