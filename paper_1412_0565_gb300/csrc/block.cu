@@ -56,32 +56,48 @@ struct BlockArgs {
 // normalised rows).
 __host__ __device__ constexpr int blk_parts(int k) { return k + 2 * k * k; }
 
-// Cholesky factor R (upper triangular, R^T R = A) and R^{-1} of a k x k SPD
-// matrix, in place in shared memory; returns false when a pivot is not
-// positive (the block has lost rank).
-__device__ bool chol_inv(int k, double *A, double *Ri) {
+// R^{-1} (upper triangular) of the Cholesky factor R (R^T R = A) of a k x k SPD
+// matrix A in shared memory (overwritten by R above its diagonal), by one warp:
+// lane i holds column i.  A warp issues an FP64 instruction every 64 cycles and
+// a division or square root is a dozen of them, so one thread's k (k + 1) / 2
+// divisions were the longest part of a sweep (about 10 us at k = 4): here each
+// pivot takes one reciprocal square root and the columns' sums run side by side
+// (with the partial sums and the rows' loads grouped: k = 4 on an 8K-vertex
+// random geometric graph 93.4 to 70.8 ms).  Returns false
+// (all lanes) when a pivot is not positive (the block has lost rank).
+__device__ bool chol_inv(int k, double *A, double *Ri, int lane) {
+    const bool mine = lane < k;
+    double rinv = 0.0;   // lane j: 1 / R_jj
     for (int j = 0; j < k; j++) {
-        double s = A[j * k + j];
-        for (int p = 0; p < j; p++) s -= A[p * k + j] * A[p * k + j];
+        // row j of R: t_i = A_ji - sum_p R_pj R_pi
+        double t = 0.0;
+        if (mine && lane >= j) {
+            t = A[j * k + lane];
+            for (int p = 0; p < j; p++) t = fma(-A[p * k + j], A[p * k + lane], t);
+        }
+        const double s = __shfl_sync(0xffffffffu, t, j);
         if (!(s > 0.0)) return false;
-        const double r = sqrt(s);
-        A[j * k + j] = r;
-        for (int i = j + 1; i < k; i++) {
-            double t = A[j * k + i];
-            for (int p = 0; p < j; p++) t -= A[p * k + j] * A[p * k + i];
-            A[j * k + i] = t / r;
-        }
+        const double ri = rsqrt(s);
+        if (lane == j) rinv = ri;
+        __syncwarp();
+        if (mine && lane > j) A[j * k + lane] = t * ri;
+        __syncwarp();
     }
-    // R^{-1} (upper triangular) by back substitution, column by column
-    for (int i = 0; i < k; i++)
-        for (int j = 0; j < k; j++) Ri[j * k + i] = 0.0;
-    for (int c = 0; c < k; c++) {
-        Ri[c * k + c] = 1.0 / A[c * k + c];
-        for (int r = c - 1; r >= 0; r--) {
-            double t = 0.0;
-            for (int p = r + 1; p <= c; p++) t += A[r * k + p] * Ri[p * k + c];
-            Ri[r * k + c] = -t / A[r * k + r];
+    // column c of R^{-1} (lane c), from its diagonal up
+    for (int r = k - 1; r >= 0; r--) {
+        const double rr = __shfl_sync(0xffffffffu, rinv, r);
+        if (mine) {
+            double v = 0.0;
+            if (r == lane) {
+                v = rinv;
+            } else if (r < lane) {
+                double t = 0.0;
+                for (int p = r + 1; p <= lane; p++) t = fma(A[r * k + p], Ri[p * k + lane], t);
+                v = -t * rr;
+            }
+            Ri[r * k + lane] = v;
         }
+        __syncwarp();
     }
     return true;
 }
@@ -156,40 +172,54 @@ __global__ void __launch_bounds__(kBlkThreads) k_block_pi(BlockArgs a, GridSync 
     };
     publish(0);
     if (!grid_sync(&s_bar)) return;
+    const double inv_g = 1.0 / a.g, inv_n = 1.0 / (double)n;
 
     for (int t = 0;; t++) {
-        // ---- sums of Y_t over all CTAs (same order in every CTA)
+        // ---- sums of Y_t over all CTAs (same order in every CTA): a group of 8
+        // lanes per sum, each lane every 8th CTA with four loads in flight, then
+        // the lanes' tree (one thread per sum added up to 152 values one by one)
         const double *src = a.part + (size_t)(t & 1) * gridDim.x * P;
-        for (int p = tid; p < P; p += kBlkThreads) {
+        for (int p0 = 0; p0 < P; p0 += kBlkThreads / 8) {
+            const int p = p0 + (tid >> 3), g = tid & 7;
             double s = 0.0;
-            for (int b = 0; b < (int)gridDim.x; b++) s += __ldcg(src + (size_t)b * P + p);
-            s_sum[p] = s;
+            if (p < P)
+                for (int b = g; b < (int)gridDim.x; b += 32) {
+                    double v[4];
+#pragma unroll
+                    for (int u = 0; u < 4; u++)
+                        v[u] = b + 8 * u < (int)gridDim.x ? __ldcg(src + (size_t)(b + 8 * u) * P + p) : 0.0;
+                    s += (v[0] + v[1]) + (v[2] + v[3]);
+                }
+            s = group_sum<8>(s);
+            if (p < P && g == 0) s_sum[p] = s;
         }
         __syncthreads();
-        if (tid == 0) {
-            // mu, the mean-free Gram matrix, its Cholesky factor and inverse
-            for (int i = 0; i < k; i++) s_mu[i] = s_sum[i] / (double)n;
-            for (int i = 0; i < k; i++)
-                for (int j = 0; j < k; j++)
-                    s_A[i * k + j] = s_sum[k + i * k + j] - (double)n * s_mu[i] * s_mu[j];
-            const bool ok = chol_inv(k, s_A, s_Ri);
-            int stop = 0, capped = 0;
-            double cmin = 1.0;
-            if (ok && t >= 1) {
+        if (warp == 0) {
+            // mu, the mean-free Gram matrix, its Cholesky factor's inverse
+            if (lane < k) s_mu[lane] = s_sum[lane] * inv_n;
+            __syncwarp();
+            for (int q = lane; q < k * k; q += 32)
+                s_A[q] = fma(-s_sum[q / k], s_mu[q % k], s_sum[k + q]);
+            __syncwarp();
+            const bool ok = chol_inv(k, s_A, s_Ri, lane);
+            __syncwarp();
+            double c = 1.0;
+            if (ok && t >= 1 && lane < k) {
                 // cos_i = x_{t,i} . x_{t-1,i} = sum_{j <= i} Ri[j][i] C[j][i]
-                for (int i = 0; i < k; i++) {
-                    double c = 0.0;
-                    for (int j = 0; j <= i; j++) c += s_Ri[j * k + i] * s_sum[k + k * k + j * k + i];
-                    if (blockIdx.x == 0) a.cos_out[i] = c;
-                    cmin = fmin(cmin, c);
-                }
+                c = 0.0;
+                for (int j = 0; j <= lane; j++) c = fma(s_Ri[j * k + lane], s_sum[k + k * k + j * k + lane], c);
+                if (blockIdx.x == 0) a.cos_out[lane] = c;
             }
-            if (!ok) stop = 2;
-            else if (a.mode == 1) stop = t >= a.k_fixed;
-            else if (t >= 1 && cmin >= 1.0 - a.tol) stop = 1;
-            else if (t >= a.max_sweeps) stop = capped = 1;
-            s_flag[0] = stop;
-            s_flag[1] = capped;
+            const bool done = __all_sync(0xffffffffu, lane >= k || c >= 1.0 - a.tol);
+            if (lane == 0) {
+                int stop = 0, capped = 0;
+                if (!ok) stop = 2;
+                else if (a.mode == 1) stop = t >= a.k_fixed;
+                else if (t >= 1 && done) stop = 1;
+                else if (t >= a.max_sweeps) stop = capped = 1;
+                s_flag[0] = stop;
+                s_flag[1] = capped;
+            }
         }
         __syncthreads();
         const int stop = s_flag[0];
@@ -222,7 +252,6 @@ __global__ void __launch_bounds__(kBlkThreads) k_block_pi(BlockArgs a, GridSync 
         // ---- rows of Y_{t+1} = (B_g Y_t - g 1 mu_t^T) R_t^{-1} / g and their sums
 #pragma unroll
         for (int q = 0; q < PL; q++) acc[q] = 0.0;
-        const double inv_g = 1.0 / a.g;
         for (int base = r0 + warp * 32; base < r1; base += NW * 32) {
             const int r = base + lane;
             double z[KM], yn[KM], xcur[KM];
@@ -232,13 +261,31 @@ __global__ void __launch_bounds__(kBlkThreads) k_block_pi(BlockArgs a, GridSync 
                 // B_g y_r = (g - d_r) y_r + sum_e w_e y_col(e)
                 double d = 0.0;
                 const int e0 = a.rp[r], e1 = a.rp[r + 1];
-                for (int e = e0; e < e1; e++) {
-                    const double we = a.w[e];
-                    const double *yc = Yt + (size_t)a.col[e] * k;
-                    d += we;
+                // entries in groups: columns and weights, then the gathers, so
+                // that a row costs two trips to L2 per group, not per entry
+                constexpr int GE = KM <= 4 ? 4 : 2;
+                for (int e = e0; e < e1; e += GE) {
+                    double we[GE], yv[GE][KM];
+                    int ce[GE];
 #pragma unroll
-                    for (int i = 0; i < KM; i++)
-                        if (i < k) z[i] = fma(we, __ldcg(yc + i), z[i]);
+                    for (int u = 0; u < GE; u++) {
+                        const bool in = e + u < e1;
+                        we[u] = in ? a.w[e + u] : 0.0;
+                        ce[u] = in ? a.col[e + u] : r;
+                    }
+#pragma unroll
+                    for (int u = 0; u < GE; u++)
+#pragma unroll
+                        for (int i = 0; i < KM; i++)
+                            if (i < k && e + u < e1) yv[u][i] = __ldcg(Yt + (size_t)ce[u] * k + i);
+#pragma unroll
+                    for (int u = 0; u < GE; u++) {
+                        if (e + u >= e1) break;
+                        d += we[u];
+#pragma unroll
+                        for (int i = 0; i < KM; i++)
+                            if (i < k) z[i] = fma(we[u], yv[u][i], z[i]);
+                    }
                 }
                 const double gd = a.g - d;
 #pragma unroll
