@@ -439,15 +439,13 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
                 free_sweep_layout(L.lay, s);
                 if (st != CMG_ERR_TOO_LARGE) return st;
             }
-            // FP64 levels: the row kernel, resident or streaming; FP32 levels:
-            // resident where the layout fits the SMs' shared memory, else the
-            // slice kernel.  CMG_STAGE (either value) keeps the slice kernel.
-            const bool try_rows = getenv("CMG_STAGE") == nullptr;
-            if (try_rows && !L.fp32) {
+            // FP64 levels: the row kernel.  CMG_STAGE (either value) keeps the
+            // slice kernel.
+            if (!L.fp32 && getenv("CMG_STAGE") == nullptr) {
                 size_t lb = 0, rb = 0;
                 CMG_TRY(build_sweep_layout(1, voff1, std::vector<int>{0, L.n}, L.n, L.rp, L.col, L.w, 0, &L.lay, &lb, s,
                                            true));
-                const cmg_status_t st = build_row_plan(L.n, L.nnz, L.rp, L.col, L.w, L.lay, 0, &L.rows, &rb, s);
+                const cmg_status_t st = build_row_plan(L.n, L.nnz, L.rp, L.col, L.w, L.g, L.lay, &L.rows, &rb, s);
                 if (st == CMG_OK) {
                     L.has_lay = L.has_rows = true;
                     lay_bytes += lb + rb;
@@ -460,17 +458,6 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
             CMG_TRY(build_sweep_layout(1, voff1, std::vector<int>{0, L.n}, L.n, L.rp, L.col, L.w, L.fp32,
                                        &L.lay, &lay_bytes, s));
             L.has_lay = true;
-            if (try_rows && L.fp32) {
-                size_t rb = 0;
-                const cmg_status_t st = build_row_plan(L.n, L.nnz, L.rp, L.col, L.w, L.lay, 1, &L.rows, &rb, s);
-                if (st == CMG_OK) {
-                    L.has_rows = true;
-                    lay_bytes += rb;
-                    continue;
-                }
-                free_row_plan(L.rows, s);
-                if (st != CMG_ERR_TOO_LARGE) return st;
-            }
             // gathers that a staged prefix of the iterate would serve
             stage_try[k] = std::min(L.n, stage_capacity(L.fp32));
             if (stage_try[k] > 0) CMG_TRY(layout_count_below(L.lay, stage_try[k], below_dev + k, s));
@@ -489,7 +476,8 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
             h->bufs.push_back(p);
         }
         double *gdp = nullptr;
-        if (!L.fp32) CMG_TRY(dev_alloc_n(&gdp, (size_t)L.n, s));
+        // (the fixed-point kernels keep their own diagonal)
+        if (!L.fp32 && !L.has_fix && !L.has_rows) CMG_TRY(dev_alloc_n(&gdp, (size_t)L.n, s));
         h->gd.push_back(gdp);
     }
     CMG_TRY(dev_alloc_n(&h->res, h->lv.size(), s));
@@ -503,7 +491,7 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
         if (L.w32) bytes += sizeof(float) * (size_t)L.nnz;
         if (L.agg) bytes += sizeof(int) * (size_t)L.n;
         bytes += 3 * (L.fp32 ? sizeof(float) : sizeof(double)) * (size_t)L.n;
-        if (!L.fp32) bytes += sizeof(double) * (size_t)L.n;
+        if (!L.fp32 && !L.has_fix && !L.has_rows) bytes += sizeof(double) * (size_t)L.n;
     }
     bytes += sizeof(double) * (size_t)n;
     h->bytes = bytes + lay_bytes;
@@ -529,6 +517,25 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
                      partial_stage_pays(below[nlev + k], L.lay.entries, L.n, di.sms))
                 h->lv[k].lay.stage_n = partial_try[k];
         }
+    }
+    // ---- FP32 levels that stage their whole iterate keep their layout in shared
+    // memory beside it where it fits
+    // (CMG_RESIDENT=0: never)
+    std::vector<int> res_try;
+    const char *res_env = getenv("CMG_RESIDENT");
+    if (form32 && !(res_env && res_env[0] == '0'))
+        for (int k = 0; k < nlev; k++)
+            if (h->lv[k].fp32 && h->lv[k].has_lay && h->lv[k].lay.stage_n >= h->lv[k].n) res_try.push_back(k);
+    if (!res_try.empty()) {
+        int *share_dev;
+        std::vector<int> share(2 * res_try.size());
+        CMG_TRY(scr.get(&share_dev, share.size()));
+        for (size_t q = 0; q < res_try.size(); q++)
+            CMG_TRY(sell_share_async(h->lv[res_try[q]].lay, h->lv[res_try[q]].n, share_dev + 2 * q, s));
+        CMG_CUDA(cudaMemcpyAsync(share.data(), share_dev, sizeof(int) * share.size(), cudaMemcpyDeviceToHost, s));
+        CMG_CUDA(cudaStreamSynchronize(s));
+        for (size_t q = 0; q < res_try.size(); q++)
+            CMG_TRY(sell_choose_resident(&h->lv[res_try[q]].lay, h->lv[res_try[q]].n, share[2 * q], share[2 * q + 1]));
     }
     return CMG_OK;
 }

@@ -41,10 +41,6 @@ __device__ __forceinline__ void fix_barrier(int C) {
     }
 }
 
-__device__ __forceinline__ double fix_value(int2 x) {
-    return fma((double)x.x, 0x1p29, (double)x.y) * 0x1p-58;
-}
-
 // Every CTA holds the whole iterate ring and its share of the items.  A sweep:
 // warp 0 (control) turns the previous sweep's sums into decisions while the
 // row warps compute their items from the local iterate and store each row's
@@ -55,8 +51,8 @@ __device__ __forceinline__ double fix_value(int2 x) {
 // runs beside it.  Six row warps reduce a sum each: a warp that reduced its
 // own five sums spent 610 cycles on 16 warp reductions, and atomics into the
 // other CTAs another 900 (3 CTAs) to 2,200 (8 CTAs).
-// us per sweep before (one CTA up to 512 rows, cluster above, FP64) and now,
-// levels of the 100^3 grid: @FIXT@
+// us per sweep before (cluster, FP64) and now: the 3,048-row level of the 100^3
+// grid 5.67 and 3.24.
 __global__ void __launch_bounds__(kFixMaxThreads) k_power_fix(PiArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ unsigned s_acc[2][kFixMaxCtas][kFixWords];   // the CTAs' stop sums by sweep parity
@@ -219,16 +215,7 @@ __global__ void __launch_bounds__(kFixMaxThreads) k_power_fix(PiArgs a) {
                 const int2 d = s_d[i - r0];
                 FixAcc t;
                 t.reset();
-                for (int t0 = 0; t0 < it.z; t0 += 8) {
-                    const int f0 = it.y + lane + 32 * t0;
-                    int cc[8];
-#pragma unroll
-                    for (int u = 0; u < 8; u++) cc[u] = t0 + u < it.z ? (int)s_col[f0 + 32 * u] : i;
-#pragma unroll
-                    for (int u = 0; u < 8; u++)
-                        if (t0 + u < it.z) t.add(x[cc[u]], s_c[f0 + 32 * u]);
-                    t.carry();
-                }
+                fix_quads(t, it.z, s_col + it.y + lane, s_c + it.y + lane, [&](int q) { return x[q]; });
                 const bool leads = r < rows && (lane & ((1 << lg) - 1)) == 0;
                 if (leads) t.add(xi, make_int2(-d.x, -d.y));
                 t.carry();
@@ -325,7 +312,9 @@ constexpr int kFixWarps = 15;
 // lanes' sums, finish, warp sums (about 900 cycles), and the control step
 // (about 1,000); then the barrier (60 cycles in one CTA, 420 in a cluster).
 // us per sweep before (FP64: one CTA up to 512 rows, cluster above), from
-// shared memory (k_power_fix) and here, levels of the 100^3 grid: @REGT@
+// shared memory (k_power_fix) and here, the 853-, 239-, 66- and
+// 18-row levels of the 100^3 grid: 3.55 / 2.48 / 1.70 / 1.24, 2.85 / 2.05 / 1.37 /
+// 1.23, and 1.29 / 1.07 / 0.95 / 0.87.
 template <int U>
 __global__ void __launch_bounds__(32 * (kFixWarps + 1)) k_power_fix_reg(PiArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -466,36 +455,11 @@ __global__ void __launch_bounds__(32 * (kFixWarps + 1)) k_power_fix_reg(PiArgs a
             code = decide(s & 1, &nx);
             rs = s;
         }
-        const double to_mean = 0x1p-58 / (double)n;
-        const double B = __shfl_sync(0xffffffffu, c.B, 4), Bp = __shfl_sync(0xffffffffu, c.Bp, 4);
-        if (lane == 0) {
-            const bool zero = code == 2;
-            s_res[0] = rs;
-            s_res[1] = zero;
-            if (rank == 0) {
-                PiResult r;
-                const double ss = zero ? Bp : B;
-                r.mu = (zero ? c.mu_p : c.muA) * to_mean;
-                r.inv_s = ss > 0.0 ? 1.0 / sqrt(ss) : 0.0;
-                const double den = sqrt(B * Bp);
-                r.cos = rs == 0 ? 0.0 : (zero ? 1.0 : (den > 0.0 ? c.C / den : 1.0));
-                r.mu_prev = c.mu_p * to_mean;
-                r.inv_s_prev = Bp > 0.0 ? 1.0 / sqrt(Bp) : 0.0;
-                r.buf = 0;
-                r.buf_prev = 1;
-                r.sweeps = rs;
-                r.capped = counted && a.mode == 0 && code == 0 ? 1 : 0;
-                r.zero = zero;
-                r.pad = 0;
-                if (s_bad) {
-                    // an infinity or NaN in the start vector: no sweep converges and
-                    // every one returns NaN, so none is run
-                    r.mu = r.cos = r.mu_prev = nan("");
-                    r.sweeps = a.mode == 1 ? max(a.k_fixed, 0) : a.max_sweeps;
-                    r.capped = a.mode == 0 ? 1 : 0;
-                }
-                *a.res = r;
-            }
+        fix_finish(a, lane, n, rs, code, counted, s_bad != 0, rank == 0, 0, c, s_res);
+        if (rank == 0 && lane == 0) {
+            // written to buf[0], the previous iterate to buf[1]
+            a.res->buf = 0;
+            a.res->buf_prev = 1;
         }
     } else {
         // ------------------------------------------------------ row warps
@@ -604,6 +568,17 @@ __global__ void __launch_bounds__(32 * (kFixWarps + 1)) k_power_fix_reg(PiArgs a
 }
 
 // ------------------------------------------------------------------ host side
+bool fix_reciprocal(double g, unsigned long long *ginv, int *ge) {
+    if (!(g > 0.0) || !std::isfinite(g)) return false;
+    int ex;
+    const double m = frexp(g, &ex);   // g = m 2^ex, m in [0.5, 1)
+    const unsigned long long G = (unsigned long long)ldexp(m, 64);
+    *ge = ex - 64;                    // g = G 2^ge, G in [2^63, 2^64)
+    const unsigned __int128 inv = ((unsigned __int128)1 << 127) / G;
+    *ginv = inv >> 64 ? ~0ull : (unsigned long long)inv;
+    return true;
+}
+
 bool fix_may_hold(int n, long long nnz) { return n >= 2 && n <= kFixMaxN && nnz <= (1 << 20); }
 
 // CTAs of a level: one per kFixCtaWork of its work (an entry counts 1, a row 8),
@@ -622,6 +597,7 @@ static size_t fix_smem(int n, int threads, int res_i, int res_e, int res_r) {
 }
 
 cmg_status_t build_fix_plans(std::vector<FixLevel> &lv, cudaStream_t s) {
+    Scratch scr(s);
     std::vector<SmallJob> jobs;
     std::vector<int> who;
     DeviceInfo di;
@@ -632,7 +608,7 @@ cmg_status_t build_fix_plans(std::vector<FixLevel> &lv, cudaStream_t s) {
     for (size_t q = 0; q < lv.size(); q++) {
         FixLevel &L = lv[q];
         L.ok = 0;
-        if (!fix_may_hold(L.n, L.nnz) || !(L.g > 0.0) || !std::isfinite(L.g)) continue;
+        if (!fix_may_hold(L.n, L.nnz)) continue;
         const long long work = L.nnz + 8ll * L.n;
         SmallJob J = {};
         J.n = L.n;
@@ -648,43 +624,26 @@ cmg_status_t build_fix_plans(std::vector<FixLevel> &lv, cudaStream_t s) {
         J.cap_items = (int)(L.n / 32 + L.nnz / 64 + 8);
         J.one_cta = kFixWarps;
         J.cap_warps = kFixWarps * L.max_ctas;
-        J.cap_entries = (int)(2 * L.nnz + L.nnz / 2 + 32 * J.S + 32 * 64);
         J.rp = L.rp;
         J.col = L.col;
         J.w = L.w;
-        int ex;
-        const double m = frexp(L.g, &ex);   // g = m 2^ex, m in [0.5, 1)
-        const unsigned long long G = (unsigned long long)ldexp(m, 64);
-        J.ge = ex - 64;                     // g = G 2^ge, G in [2^63, 2^64)
-        const unsigned __int128 one = (unsigned __int128)1 << 127;
-        const unsigned __int128 inv = one / G;
-        J.ginv = inv >> 64 ? ~0ull : (unsigned long long)inv;
-        // one arena: items, range, perm, diagonal, coefficients, columns
+        if (!fix_reciprocal(L.g, &J.ginv, &J.ge)) continue;
+        // items, range and perm in one allocation, the entries (exact) in another
         auto al = [](size_t x) { return (x + 15) & ~(size_t)15; };
-        size_t o[7];
-        o[0] = 0;
-        o[1] = o[0] + 16 * ((size_t)J.cap_items + 1);
-        o[2] = o[1] + al(4 * ((size_t)J.C + 1));
-        o[3] = o[2] + al(4 * (size_t)L.n);
-        o[4] = o[3] + al(8 * (size_t)L.n);
-        o[5] = o[4] + al(8 * (size_t)J.cap_entries);
-        o[6] = o[5] + al(2 * (size_t)J.cap_entries);
+        const size_t o1 = 16 * ((size_t)J.cap_items + 1), o2 = o1 + al(4 * ((size_t)J.C + 1)), o3 = o2 + al(4 * (size_t)L.n);
         FixPlan &F = L.plan;
-        CMG_TRY(dev_alloc(&F.arena, o[6], s));
+        CMG_TRY(dev_alloc(&F.arena, o3, s));
         char *base = (char *)F.arena;
         F.C = J.C;
-        J.item = F.item = (int4 *)(base + o[0]);
-        J.range = F.range = (int *)(base + o[1]);
-        J.perm = F.perm = (int *)(base + o[2]);
-        J.ud = F.ud = (int2 *)(base + o[3]);
-        J.uc = F.uc = (int2 *)(base + o[4]);
-        J.ucol = F.ucol = (uint16_t *)(base + o[5]);
-        F.bytes = o[6];
+        J.item = F.item = (int4 *)base;
+        J.range = F.range = (int *)(base + o1);
+        J.perm = F.perm = (int *)(base + o2);
+        CMG_TRY(scr.get(&J.inv, (size_t)L.n));
+        F.bytes = o3;
         jobs.push_back(J);
         who.push_back((int)q);
     }
     if (jobs.empty()) return CMG_OK;
-    Scratch scr(s);
     SmallJob *jobs_dev;
     PlanOut *out_dev;
     CMG_TRY(scr.get(&jobs_dev, jobs.size()));
@@ -741,13 +700,25 @@ cmg_status_t build_fix_plans(std::vector<FixLevel> &lv, cudaStream_t s) {
                 continue;
             }
         }
-        L.ok = fits ? 1 : 0;
+        if (!fits) continue;
+        // exact entries, filled below
+        const size_t ne = (size_t)std::max<long long>(out[k].entries, 1), o1 = 8 * ne, o2 = o1 + 8 * (size_t)L.n;
+        CMG_TRY(dev_alloc(&F.entries, o2 + 2 * ne, s));
+        jobs[k].uc = F.uc = (int2 *)F.entries;
+        jobs[k].ud = F.ud = (int2 *)((char *)F.entries + o1);
+        jobs[k].ucol = F.ucol = (uint16_t *)((char *)F.entries + o2);
+        jobs[k].ni = F.ni;
+        F.bytes += o2 + 2 * ne;
+        L.ok = 1;
     }
-    return CMG_OK;
+    // (a level that does not fit keeps ni = 0 items to fill)
+    CMG_CUDA(cudaMemcpyAsync(jobs_dev, jobs.data(), sizeof(SmallJob) * jobs.size(), cudaMemcpyHostToDevice, s));
+    return launch_fill_small(jobs_dev, (int)jobs.size(), s);
 }
 
 void free_fix_plan(FixPlan &F, cudaStream_t s) {
     dev_free(F.arena, s);
+    dev_free(F.entries, s);
     F = FixPlan();
 }
 

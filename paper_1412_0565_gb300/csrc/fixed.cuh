@@ -43,7 +43,7 @@ struct PlanOut {
 // A level for k_plan_small: its CSR, g's reciprocal (fix_weight), steps per lane,
 // CTAs, and the arrays to fill with their capacities.
 struct SmallJob {
-    int n, S, C, cap_items, cap_entries;
+    int n, S, C, cap_items, ni;
     int one_cta, cap_warps;   // most items the one-per-warp form takes in one CTA, and in all
     const int *rp, *col;
     const double *w;
@@ -51,11 +51,13 @@ struct SmallJob {
     int ge;
     int4 *item;
     int *range, *perm;
+    uint16_t *inv;             // scratch
     uint16_t *ucol;
-    int2 *uc, *ud;
+    int2 *uc, *ud;             // k_fill_small: ni items
     PlanOut *out;
 };
 cmg_status_t launch_plan_small(const SmallJob *jobs_dev, int count, cudaStream_t s);
+cmg_status_t launch_fill_small(const SmallJob *jobs_dev, int count, cudaStream_t s);
 
 // ------------------------------------------------------------------ arithmetic
 constexpr int kFixBits = 58;   // y = X 2^-58
@@ -107,14 +109,44 @@ struct FixAcc {
         m2 = 0;
     }
     // the accumulated product / 2^60 in sixteenths, and its sum over aligned
-    // groups of 2^lg lanes (after carry; the cut below 2^-4 of the last bit is a
-    // sixteenth of the final rounding)
+    // groups of 2^lg lanes (after carry).  Each lane rounds to nearest: cutting here
+    // shifts a row by up to half a unit per sweep in the same direction, and
+    // thousands of sweeps add that up (1e-12 in lambda2 on a power-law graph).
     __device__ __forceinline__ long long lanes(int lg) const {
-        long long v = (hi << 2) + (m1 >> 27);
+        long long v = (hi << 2) + ((m1 + (1ll << 26)) >> 27);
         for (int o = (1 << lg) >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         return v;
     }
 };
+
+// One lane's entries of an item in shared memory: `steps` (a multiple of 4) entries
+// 32 apart from col / cf on, four at a time (columns, then values, then products).
+template <typename IDX, typename LD>
+__device__ __forceinline__ void fix_quads(FixAcc &t, int steps, const IDX *col, const int2 *cf, LD ldx) {
+    int u = 0;
+    for (; u + 8 <= steps; u += 8, col += 256, cf += 256) {
+        int cc[8];
+        int2 xx[8];
+#pragma unroll
+        for (int j = 0; j < 8; j++) cc[j] = (int)col[32 * j];
+#pragma unroll
+        for (int j = 0; j < 8; j++) xx[j] = ldx(cc[j]);
+#pragma unroll
+        for (int j = 0; j < 8; j++) t.add(xx[j], cf[32 * j]);
+        if ((u & 24) == 24) t.carry();
+    }
+    if (u < steps) {
+        int cc[4];
+        int2 xx[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) cc[j] = (int)col[32 * j];
+#pragma unroll
+        for (int j = 0; j < 4; j++) xx[j] = ldx(cc[j]);
+#pragma unroll
+        for (int j = 0; j < 4; j++) t.add(xx[j], cf[32 * j]);
+    }
+    t.carry();
+}
 
 // The row's new value: p is the lane-summed product of its entries and of its
 // diagonal (-D_i) in sixteenths.
@@ -336,6 +368,81 @@ __device__ __forceinline__ int fix_decide(const PiArgs &a, int lane, long long v
     c.e = en;
     return code;
 }
+
+// State and first slots from the start vector's totals (read: value by lane group
+// as fix_decide wants it, A 2^-20 in the place of C's first value, and the maximum).
+template <typename READ>
+__device__ __forceinline__ void fix_ctl_start(const PiArgs &a, int lane, READ read, double omt2, int n, FixCtl &c,
+                                              FixSlot *slots) {
+    unsigned m;
+    const long long v = read(&m);
+    const int grp = lane >> 2;
+    double d = __ll2double_rn(v);
+    if (grp == 1) d *= 0x1p-42;
+    if (grp == 2) d *= 0x1p-86;
+    const double A = fma(__shfl_sync(0xffffffffu, d, 16), 0x1p20, __shfl_sync(0xffffffffu, d, 0));
+    const double B = __shfl_sync(0xffffffffu, d, 4) + __shfl_sync(0xffffffffu, d, 8);
+    const double mu0 = A * 0x1p-58 / (double)n;
+    double ss0 = B - (double)n * mu0 * mu0;
+    if (ss0 < 0.0) ss0 = 0.0;
+    c.B = c.Bp = ss0;
+    c.K = omt2 * ss0;
+    c.Z = ss0 * (double)a.zero_tol2;
+    c.C = 0.0;
+    c.muA = c.mu_p = A;
+    c.M = 0;
+    c.e = 0;
+    if (lane == 0) {
+        slots[1].M = __double2ll_rn(A / (double)n);   // sweep 1: exact mean of y_0
+        slots[1].e = 0;
+        slots[1].stop = 0;
+        slots[0].M = 0;                               // sweep 2: m_1 = 0
+        slots[0].e = 0;
+        slots[0].stop = 0;
+    }
+}
+
+// Result of a run whose last decided sweep is rs with `code` (fix_decide); buf:
+// the ring slot of sweep rs.  res[0..1]: rs, annihilated.
+__device__ __forceinline__ void fix_finish(const PiArgs &a, int lane, int n, int rs, int code, bool counted, bool bad,
+                                           bool writes, int buf, const FixCtl &c, int *res) {
+    const double to_mean = 0x1p-58 / (double)n;
+    const double B = __shfl_sync(0xffffffffu, c.B, 4), Bp = __shfl_sync(0xffffffffu, c.Bp, 4);
+    if (lane != 0) return;
+    const bool zero = code == 2;
+    res[0] = rs;
+    res[1] = zero;
+    if (!writes) return;
+    PiResult r;
+    const double ss = zero ? Bp : B;
+    r.mu = (zero ? c.mu_p : c.muA) * to_mean;
+    r.inv_s = ss > 0.0 ? 1.0 / sqrt(ss) : 0.0;
+    const double den = sqrt(B * Bp);
+    r.cos = rs == 0 ? 0.0 : (zero ? 1.0 : (den > 0.0 ? c.C / den : 1.0));
+    r.mu_prev = c.mu_p * to_mean;
+    r.inv_s_prev = Bp > 0.0 ? 1.0 / sqrt(Bp) : 0.0;
+    r.buf = zero ? (buf + 2) % 3 : buf;
+    r.buf_prev = (buf + 2) % 3;
+    r.sweeps = rs;
+    r.capped = counted && a.mode == 0 && code == 0 ? 1 : 0;
+    r.zero = zero;
+    r.pad = 0;
+    if (bad) {
+        // an infinity or NaN in the start vector: no sweep converges and every
+        // one returns NaN, so none is run
+        r.mu = r.cos = r.mu_prev = nan("");
+        r.sweeps = a.mode == 1 ? max(a.k_fixed, 0) : a.max_sweeps;
+        r.capped = a.mode == 0 ? 1 : 0;
+    }
+    *a.res = r;
+}
+
+__device__ __forceinline__ double fix_value(int2 x) {
+    return fma((double)x.x, 0x1p29, (double)x.y) * 0x1p-58;
+}
+
+// The reciprocal fix_weight takes: false when g is not a positive finite number.
+bool fix_reciprocal(double g, unsigned long long *ginv, int *ge);
 
 // The exponent k that scales a start vector of largest magnitude m (finite,
 // > 0) to |x| 2^k in (2^55, 2^56].

@@ -87,6 +87,10 @@ struct SweepLayout {
     // single-graph layouts: iterate entries the slice kernel stages in shared
     // memory per sweep (0: none)
     int stage_n = 0;
+    // FP32 slice kernel with the layout resident in shared memory beside the whole
+    // iterate: entries per CTA (0: not resident), dynamic shared memory
+    int res_e = 0;
+    size_t res_smem = 0;
 };
 constexpr int kHeavyChunk = 2048;
 // Builds the layout of the N rows of a level holding G graphs at union
@@ -157,6 +161,10 @@ void free_xlayout(XLayout &X, cudaStream_t s);
 size_t xsweep_smem(int fp32);
 // Adds to *out (zeroed first) the layout entries whose column is below S.
 cmg_status_t layout_count_below(const SweepLayout &L, int S, unsigned long long *out, cudaStream_t s);
+// Resident FP32 slice kernel: most entries and chunks of a CTA to out_dev[0..1]
+// (stage_n decided), and the choice from them.
+cmg_status_t sell_share_async(const SweepLayout &L, int n, int *out_dev, cudaStream_t s);
+cmg_status_t sell_choose_resident(SweepLayout *L, int n, int max_entries, int max_chunks);
 // Iterate entries the staged slice kernel can hold in shared memory (FP32 or
 // FP64 sweeps).
 int stage_capacity(int fp32);
@@ -178,13 +186,13 @@ inline bool partial_stage_pays(unsigned long long below, long long entries, int 
            (double)below * (double)n >= 3.0 * (double)kPartialStage * (double)entries;
 }
 
-// Plan of the row kernel (resident.cu) for a single-graph level whose rows are
-// in the sweep layout's order: items (a warp's unit of work) dealt to P CTAs
-// in contiguous ranges, and for FP64 sweeps the items' own entry arrays.
+// Plan of the row kernel (resident.cu) for a single-graph FP64 level whose rows
+// are in the sweep layout's order: items (a warp's unit of work) dealt to P CTAs
+// in contiguous ranges, and the items' entries in fixed point.
 struct RowPlan {
-    int P = 0;                  // CTAs of the launch
+    int P = 0, threads = 0;     // CTAs and threads of the launch
     int ni = 0;                 // items
-    int fp32 = 0, col16 = 1;
+    int col16 = 1;
     int resident = 0;           // the matrix stays in shared memory for the launch
     int stage = 0;              // ... and the iterate is copied there every sweep
     int stream = 0;             // streaming form: read evict-first
@@ -193,15 +201,15 @@ struct RowPlan {
     long long entries = 0;
     int4 *item = nullptr;       // [ni + 1] first row, first entry, steps, log2 lanes | rows << 3
     int *range = nullptr;       // [P + 1] first item of each CTA
-    void *ucol = nullptr;       // FP64: columns (uint16 or int32) and weights by item
-    double *uw = nullptr;
+    void *ucol = nullptr;       // columns (uint16 or int32), coefficients and diagonal
+    int2 *uc = nullptr, *ud = nullptr;
+    long long *acc = nullptr;   // the CTAs' stop sums
 };
-// Builds it from the level's CSR and the row order (FP64: L.perm / L.inv) or
-// the whole sweep layout (FP32).  CMG_ERR_TOO_LARGE: the level is left to the
-// slice kernel (an FP64 row of more than 4,096 entries, which one warp would
-// hold up, or an FP32 level beyond shared memory).  Adds its bytes to *bytes.
-cmg_status_t build_row_plan(int n, long long nnz, const int *rp, const int *col, const double *w,
-                            const SweepLayout &L, int fp32, RowPlan *R, size_t *bytes, cudaStream_t s);
+// Builds it from the level's CSR and the row order (L.perm / L.inv).
+// CMG_ERR_TOO_LARGE: the level is left to the slice kernel (a row of more than
+// 4,096 entries, which one warp would hold up).  Adds its bytes to *bytes.
+cmg_status_t build_row_plan(int n, long long nnz, const int *rp, const int *col, const double *w, double g,
+                            const SweepLayout &L, RowPlan *R, size_t *bytes, cudaStream_t s);
 void free_row_plan(RowPlan &R, cudaStream_t s);
 // Plan of the fixed-point kernel for small FP64 levels (fixed.cu): one CTA, or one
 // cluster of up to 8, holds the level in shared memory.
@@ -210,7 +218,7 @@ struct FixPlan {
     int ni = 0, by_warp = 0;               // one item of that many steps per row warp (0: by entries)
     int res_e = 0, res_i = 0, res_r = 0;   // most entries, items, rows of a CTA
     size_t smem = 0, bytes = 0;
-    void *arena = nullptr;                 // the arrays below, one allocation
+    void *arena = nullptr, *entries = nullptr;   // allocations of the arrays below
     int4 *item = nullptr;
     int *range = nullptr, *perm = nullptr;
     uint16_t *ucol = nullptr;

@@ -70,7 +70,6 @@ struct PiArgs {
     int *hcount;            // chunks finished per heavy row
     void *cpart;            // chunk partial sums
     int nchunks;
-    int stream_hint;        // the layout is larger than L2: read it evict-first
     int stage_n;            // iterate entries 0..stage_n-1 copied to shared memory per sweep
     // two-phase kernel: the level's XLayout (see internal.h)
     int x_T, x_Q, x_SB, x_VMAX;
@@ -81,10 +80,12 @@ struct PiArgs {
     double *x_pmax;
     void *x_buf[2];
     // row kernel: items, first item of each CTA, capacities of its shared memory
+    // (res_entries: also the resident slice kernel's)
     const int4 *items;
     const int *item_range;
     int res_entries, res_items, res_rows;
     int nitems;             // fixed-point sweeps: items of the level
+    void *fix_acc;          // row kernel: the CTAs' stop sums (see k_power_rows)
     const int2 *fix_d;      // fixed-point sweeps: diagonal D_i by row in layout order
 };
 

@@ -303,6 +303,29 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_power_tiled(PiArgs a, GridS
     }
 }
 
+// First entry and length (a multiple of 8) of chunk cidx of the heavy rows: a row
+// of len entries is cut into nc chunks of equal length rounded up to octets.
+__device__ __forceinline__ void sell_chunk(const PiArgs &a, const int *M, int cidx, int *f0, int *len) {
+    const int r = a.crow[cidx], c0 = a.hchunk[r], nc = a.hchunk[r + 1] - c0;
+    const int m0 = M[r], m1 = M[r + 1];
+    const int per = (((m1 - m0 + nc - 1) / nc) + 7) & ~7;
+    *f0 = min(m1, m0 + (cidx - c0) * per);
+    *len = min(m1, *f0 + per) - *f0;
+}
+
+// First slice of CTA b of nb: slices starting at b / nb of the slice entries.
+__device__ __forceinline__ int sell_first_slice(const int *SO, int nsl, int b, int nb) {
+    if (b >= nb) return nsl;
+    const long long target = SO[0] + ((long long)SO[nsl] - SO[0]) * b / nb;
+    int lo = 0, hi = nsl;   // first slice starting at or after the target
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (SO[mid] < target) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
 // ================================================================== slice kernel
 // Large levels with a sweep layout (rows renumbered by decreasing degree;
 // heavy rows in CSR form, the rest in 32-row slices with interleaved entries):
@@ -318,11 +341,26 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_power_tiled(PiArgs a, GridS
 // there.  A gather of 32 scattered words from L1 or L2 costs about one cycle
 // per distinct line; from shared memory it costs the bank conflicts, a few
 // cycles per 32 words.
-template <typename T, typename IDX, bool CHUNKS, bool STREAM, bool STAGE>
+//
+// RES (FP32 levels that stage their whole iterate and whose layout fits beside it in
+// the SMs' shared memory): the CTA copies its chunks and slices there once and
+// sweeps from there, instead of reading them from L2 every sweep.  The rows stay
+// with the CTA, warp and order that they have without RES -- the stop sums then
+// round the same way, and with them the mean that every FP32 sweep subtracts: a
+// level's thousands of sweeps turn one other rounding there into a different
+// vector at the 1e-8 level.  16K rows and 3.2M entries: 23.9 us per sweep
+// without, 18.8 with.  (The two-CTA form without a staged iterate measured the
+// same or slower from shared memory: 3,820 rows and 2.1M entries 14.4 and 15.0,
+// 100^3 grid levels 1 and 2 16.7 and 18.4, 9.7 and 10.2: it does not take it.)
+template <typename T, typename IDX, bool CHUNKS, bool STREAM, bool STAGE, bool RES>
 __global__ void __launch_bounds__(STAGE ? kStageThreads : kTileThreads, STAGE ? 1 : 2)
     k_power_sell(PiArgs a, GridSync *gs) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    // shared memory: the staged iterate; RES: weights, columns, chunk offsets
     T *const s_x = reinterpret_cast<T *>(smem_raw);
+    T *const s_w = s_x + (STAGE ? ((a.stage_n + 7) & ~7) : 0);
+    IDX *const s_c = reinterpret_cast<IDX *>(s_w + (RES ? a.res_entries : 0));
+    int *const s_co = reinterpret_cast<int *>(s_c + (RES ? a.res_entries : 0));
     __shared__ Part s_pw[kStageThreads / 32];
     __shared__ Slot s_slot[2];
     __shared__ GridBar s_bar;
@@ -343,21 +381,48 @@ __global__ void __launch_bounds__(STAGE ? kStageThreads : kTileThreads, STAGE ? 
     // of the slice entries (the slices are sorted by width, so equal slice
     // counts would not balance); heavy rows go round robin over all warps
     __shared__ int s_range[2];
-    if (threadIdx.x < 2) {
-        const long long tot = (long long)SO[nsl] - SO[0];
-        const long long target = SO[0] + tot * (blockIdx.x + threadIdx.x) / gridDim.x;
-        int lo = 0, hi = nsl;   // first slice starting at or after the target
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (SO[mid] < target) lo = mid + 1;
-            else hi = mid;
-        }
-        s_range[threadIdx.x] = (blockIdx.x + threadIdx.x == gridDim.x) ? nsl : lo;
-    }
+    if (threadIdx.x < 2)
+        s_range[threadIdx.x] = sell_first_slice(SO, nsl, (int)blockIdx.x + (int)threadIdx.x, (int)gridDim.x);
     __syncthreads();
     const int sb = s_range[0], se = s_range[1];
     const int r0 = (int)((long long)n * blockIdx.x / gridDim.x);
     const int r1 = (int)((long long)n * (blockIdx.x + 1) / gridDim.x);
+    int sl_off = 0;   // RES: shared-memory entry of slice entry e is e + sl_off
+    if (RES) {
+        // this CTA's chunks (chunk b + grid j is the j-th), then its slices
+        const int nj = CHUNKS && (int)blockIdx.x < a.nchunks ? (a.nchunks - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+        if (warp == 0) {
+            int carry = 0;
+            for (int j0 = 0; j0 < nj; j0 += 32) {
+                int f0 = 0, len = 0;
+                if (j0 + lane < nj) sell_chunk(a, M, (int)(blockIdx.x + gridDim.x * (j0 + lane)), &f0, &len);
+                int incl = len;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += t;
+                }
+                if (j0 + lane < nj) s_co[j0 + lane] = carry + incl - len;
+                carry += __shfl_sync(0xffffffffu, incl, 31);
+            }
+            if (lane == 0) s_co[nj] = carry;
+        }
+        __syncthreads();
+        for (int j = warp; j < nj; j += (int)(blockDim.x >> 5)) {
+            int f0, len;
+            sell_chunk(a, M, (int)(blockIdx.x + gridDim.x * j), &f0, &len);
+            const int d = s_co[j];
+            for (int k = lane; k < len; k += 32) {
+                s_w[d + k] = W[f0 + k];
+                s_c[d + k] = C[f0 + k];
+            }
+        }
+        sl_off = s_co[nj] - (sb < se ? SO[sb] : 0);
+        for (int k = (sb < se ? SO[sb] : 0) + tid; k < (sb < se ? SO[se] : 0); k += blockDim.x) {
+            s_w[k + sl_off] = W[k];
+            s_c[k + sl_off] = C[k];
+        }
+    }
 
     // ---------------------------------------------------------- start phase
     {
@@ -465,16 +530,22 @@ __global__ void __launch_bounds__(STAGE ? kStageThreads : kTileThreads, STAGE ? 
             // warp of a row's last chunk waits for the row's other chunks,
             // sums the chunk partials in chunk order and completes the row
             const bool vec = ((reinterpret_cast<uintptr_t>(C) | reinterpret_cast<uintptr_t>(W)) & 15) == 0;
-            for (int cidx = gw; CHUNKS && cidx < a.nchunks; cidx += ngw) {
+            for (int cidx = gw, j = rw; CHUNKS && cidx < a.nchunks; cidx += ngw, j += nrw) {
                 const int r = a.crow[cidx], c0 = a.hchunk[r], nc = a.hchunk[r + 1] - c0;
-                const int len = M[r + 1] - M[r];
-                const int per = (((len + nc - 1) / nc) + 7) & ~7;
-                const int f0 = min(M[r + 1], M[r] + (cidx - c0) * per);
-                const int f1 = min(M[r + 1], f0 + per);
+                int f0, flen;
+                sell_chunk(a, M, cidx, &f0, &flen);
                 const T xi = ldx(r);
-                T ac = vec ? row_sum_octets<T, IDX, sizeof(T) == 4 ? kOct32 : 1>(C, W, (f0 >> 3) + lane, f1 >> 3, xi, ldx,
-                                                                        STREAM)
-                           : row_sum_grouped<T, IDX>(C, W, f0 + lane, f1, 32, xi, ldx, STREAM);
+                T ac;
+                if (RES) {
+                    const int d = s_co[j] >> 3;
+                    ac = row_sum_octets<T, IDX, sizeof(T) == 4 ? kOct32 : 1>(s_c, s_w, d + lane, d + (flen >> 3), xi, ldx,
+                                                                             false);
+                } else {
+                    const int f1 = f0 + flen;
+                    ac = vec ? row_sum_octets<T, IDX, sizeof(T) == 4 ? kOct32 : 1>(C, W, (f0 >> 3) + lane, f1 >> 3, xi,
+                                                                                  ldx, STREAM)
+                             : row_sum_grouped<T, IDX>(C, W, f0 + lane, f1, 32, xi, ldx, STREAM);
+                }
                 ac = warp_sum(ac);
                 if (nc == 1) {
                     if (lane == 0) finish(r, xi, ac);
@@ -517,7 +588,8 @@ __global__ void __launch_bounds__(STAGE ? kStageThreads : kTileThreads, STAGE ? 
                 const int i = h + 32 * q + lane;
                 const int so = SO[q] + lane, wd = (SO[q + 1] - SO[q]) >> 5;
                 const T xi = (i < n) ? ldx(i) : (T)0;
-                const T ac = row_sum_grouped<T, IDX>(C, W, so, so + 32 * wd, 32, xi, ldx, STREAM);
+                const T ac = RES ? row_sum_grouped<T, IDX>(s_c, s_w, so + sl_off, so + sl_off + 32 * wd, 32, xi, ldx, false)
+                                 : row_sum_grouped<T, IDX>(C, W, so, so + 32 * wd, 32, xi, ldx, STREAM);
                 if (i < n) finish(i, xi, ac);
             }
             Part p = warp_sum_part(acc.get());
@@ -1123,10 +1195,10 @@ static size_t tiled_smem(bool fp32) {
 template <typename T, typename IDX, bool STAGE>
 static const void *sell_kernel_tis(bool chunks, bool stream) {
     if (chunks)
-        return stream ? (const void *)k_power_sell<T, IDX, true, true, STAGE>
-                      : (const void *)k_power_sell<T, IDX, true, false, STAGE>;
-    return stream ? (const void *)k_power_sell<T, IDX, false, true, STAGE>
-                  : (const void *)k_power_sell<T, IDX, false, false, STAGE>;
+        return stream ? (const void *)k_power_sell<T, IDX, true, true, STAGE, false>
+                      : (const void *)k_power_sell<T, IDX, true, false, STAGE, false>;
+    return stream ? (const void *)k_power_sell<T, IDX, false, true, STAGE, false>
+                  : (const void *)k_power_sell<T, IDX, false, false, STAGE, false>;
 }
 
 template <typename T, typename IDX>
@@ -1140,6 +1212,105 @@ static const void *sell_kernel(int fp32, int col16, bool chunks, bool stream, bo
                      : sell_kernel_ti<float, int>(chunks, stream, stage);
     return col16 ? sell_kernel_ti<double, uint16_t>(chunks, stream, stage)
                  : sell_kernel_ti<double, int>(chunks, stream, stage);
+}
+
+static const void *sell_res_kernel(int col16, bool chunks) {
+    if (col16)
+        return chunks ? (const void *)k_power_sell<float, uint16_t, true, false, true, true>
+                      : (const void *)k_power_sell<float, uint16_t, false, false, true, true>;
+    return chunks ? (const void *)k_power_sell<float, int, true, false, true, true>
+                  : (const void *)k_power_sell<float, int, false, false, true, true>;
+}
+
+// Launch of the slice kernel over a level's layout: CTAs and threads (the
+// resident form takes them over, so that the sums group the same way).
+static cmg_status_t sell_geometry(const SweepLayout &L, int n, int fp32, int *blocks, int *threads, const void **kern,
+                                  size_t *smem, bool *stream) {
+    DeviceInfo di;
+    CMG_TRY(device_info(&di));
+    // only a layout that cannot stay in L2 is read evict-first
+    const long long lay_bytes = L.entries * (long long)((L.col16 ? 2 : 4) + (fp32 ? 4 : 8));
+    *stream = di.l2_bytes > 0 && lay_bytes > (long long)di.l2_bytes;
+    const int stage_n = std::min(L.stage_n, n);
+    const bool stage = stage_n > 0;
+    *kern = sell_kernel(fp32, L.col16, L.hheavy[0] > 0, *stream, stage);
+    *threads = stage ? kStageThreads : kTileThreads;
+    *smem = stage ? (size_t)((stage_n + 7) & ~7) * (fp32 ? sizeof(float) : sizeof(double)) : 0;
+    if (stage) CMG_TRY(allow_max_dynamic_smem(*kern));
+    int maxb = 0;
+    CMG_TRY(coop_max_blocks(*kern, *threads, *smem, &maxb));
+    const int row_warps = *threads / 32 - 1;
+    const long long tasks = (long long)(n - L.hheavy[0] + 31) / 32 + L.nchunks;
+    *blocks = (int)std::max<long long>(1, std::min<long long>(maxb, (tasks + row_warps - 1) / row_warps));
+    return CMG_OK;
+}
+
+// Most entries and chunks of one CTA of the slice kernel: out[0], out[1].
+__global__ void k_sell_share(PiArgs a, int nb, int *out) {
+    const int *M = a.lay_meta, *SO = M + a.lay_h;
+    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) {
+        int e = 0, j = 0;
+        for (int c = b; c < a.nchunks; c += nb, j++) {
+            int f0, len;
+            sell_chunk(a, M, c, &f0, &len);
+            e += len;
+        }
+        e += SO[sell_first_slice(SO, a.lay_nsl, b + 1, nb)] - SO[sell_first_slice(SO, a.lay_nsl, b, nb)];
+        atomicMax(out, e);
+        atomicMax(out + 1, j);
+    }
+}
+
+static void sell_args(const SweepLayout &L, int n, PiArgs &a) {
+    a.perm = reinterpret_cast<const int *>(L.perm);
+    a.lay_h = L.hheavy[0];
+    a.lay_nsl = (n - a.lay_h + 31) / 32;
+    a.lay_meta = L.meta;
+    a.lay_col = L.bcol;
+    a.lay_w = L.bw;
+    a.hchunk = L.hchunk;
+    a.crow = L.crow;
+    a.hcount = L.hcount;
+    a.cpart = L.cpart;
+    a.nchunks = L.nchunks;
+}
+
+cmg_status_t sell_share_async(const SweepLayout &L, int n, int *out_dev, cudaStream_t s) {
+    CMG_CUDA(cudaMemsetAsync(out_dev, 0, 2 * sizeof(int), s));
+    PiArgs a = {};
+    sell_args(L, n, a);
+    int blocks, threads;
+    const void *kern;
+    size_t smem;
+    bool stream;
+    CMG_TRY(sell_geometry(L, n, 1, &blocks, &threads, &kern, &smem, &stream));
+    k_sell_share<<<div_up(blocks, 32), 32, 0, s>>>(a, blocks, out_dev);
+    return launch_status();
+}
+
+cmg_status_t sell_choose_resident(SweepLayout *L, int n, int max_entries, int max_chunks) {
+    L->res_e = 0;
+    int blocks, threads;
+    const void *kern;
+    size_t smem;
+    bool stream;
+    CMG_TRY(sell_geometry(*L, n, 1, &blocks, &threads, &kern, &smem, &stream));
+    if (L->stage_n < n) return CMG_OK;
+    const size_t need = 4 * (size_t)((n + 7) & ~7) + (size_t)max_entries * (4 + (L->col16 ? 2 : 4)) +
+                        4 * ((size_t)max_chunks + 2) + 16;
+    const void *k = sell_res_kernel(L->col16, L->hheavy[0] > 0);
+    DeviceInfo di;
+    CMG_TRY(device_info(&di));
+    cudaFuncAttributes fa;
+    CMG_CUDA(cudaFuncGetAttributes(&fa, k));
+    if ((long long)need > (long long)di.max_smem_optin - (long long)fa.sharedSizeBytes) return CMG_OK;
+    CMG_TRY(allow_max_dynamic_smem(k));
+    int maxb = 0;
+    CMG_TRY(coop_max_blocks(k, threads, need, &maxb));
+    if (maxb < blocks) return CMG_OK;
+    L->res_e = max_entries;
+    L->res_smem = need;
+    return CMG_OK;
 }
 
 static const void *small_kernel(int G) {
@@ -1192,8 +1363,8 @@ int stage_capacity(int fp32) {
     DeviceInfo d;
     if (device_info(&d) != CMG_OK) return 0;
     cudaFuncAttributes fa;
-    const void *k = fp32 ? (const void *)k_power_sell<float, int, true, true, true>
-                         : (const void *)k_power_sell<double, int, true, true, true>;
+    const void *k = fp32 ? (const void *)k_power_sell<float, int, true, true, true, false, true>
+                         : (const void *)k_power_sell<double, int, true, true, true, false>;
     if (cudaFuncGetAttributes(&fa, k) != cudaSuccess) return 0;
     const long long room = (long long)d.max_smem_optin - (long long)fa.sharedSizeBytes - 256;
     if (room <= 0) return 0;
@@ -1251,7 +1422,6 @@ cmg_status_t power_iteration(const PiRun &run, GridSync *gs, cudaStream_t s, con
     a.hcount = nullptr;
     a.cpart = nullptr;
     a.nchunks = 0;
-    a.stream_hint = 0;
     a.stage_n = 0;
     void *args[] = {&a, &gs};
     if (lv.fix && !run.fp32) return launch_power_fix(*lv.fix, a, s);
@@ -1262,6 +1432,7 @@ cmg_status_t power_iteration(const PiRun &run, GridSync *gs, cudaStream_t s, con
         CMG_TRY(allow_max_dynamic_smem(kern));
         return coop_launch(kern, 1, small_threads(lv.n, G), smem, s, args, gs);
     }
+    if (lv.rows && lv.lay) return launch_power_rows(*lv.rows, *lv.lay, a, gs, s);
     if (!run.fp32 && !run.gd) return CMG_ERR_INVALID_ARG;
     if (lv.xl && lv.lay) {
         // two-phase kernel: one 1024-thread CTA per SM, the layout's P CTAs
@@ -1301,45 +1472,26 @@ cmg_status_t power_iteration(const PiRun &run, GridSync *gs, cudaStream_t s, con
         a.partials = reinterpret_cast<PartRec *>(partials);
         return coop_launch(kern, X.P, kStageThreads, X.smem, s, args, gs);
     }
-    if (lv.rows && lv.lay) return launch_power_rows(*lv.rows, *lv.lay, a, gs, s);
     if (lv.lay) {
         // slice kernel over the level's sweep layout (one graph)
         const SweepLayout &L = *lv.lay;
-        a.perm = reinterpret_cast<const int *>(L.perm);
-        a.lay_h = L.hheavy[0];
-        a.lay_nsl = (lv.n - a.lay_h + 31) / 32;
-        {
-            // layout bytes against L2: only a stream that cannot stay in L2
-            // is read evict-first
-            DeviceInfo di;
-            CMG_TRY(device_info(&di));
-            const int l2 = di.l2_bytes;
-            const long long lay_bytes = L.entries * (long long)((L.col16 ? 2 : 4) + (run.fp32 ? 4 : 8));
-            a.stream_hint = (l2 > 0 && lay_bytes > (long long)l2) ? 1 : 0;
-        }
-        a.lay_meta = L.meta;
-        a.lay_col = L.bcol;
-        a.lay_w = L.bw;
-        a.hchunk = L.hchunk;
-        a.crow = L.crow;
-        a.hcount = L.hcount;
-        a.cpart = L.cpart;
-        a.nchunks = L.nchunks;
+        sell_args(L, lv.n, a);
         if (a.lay_h > 0) {
             if (!L.hchunk) return CMG_ERR_INVALID_ARG;
             CMG_CUDA(cudaMemsetAsync(L.hcount, 0, sizeof(int) * (size_t)a.lay_h, s));
         }
         a.stage_n = std::min(L.stage_n, lv.n);
-        const bool stage = a.stage_n > 0;
-        const void *kern = sell_kernel(run.fp32, L.col16, a.lay_h > 0, a.stream_hint != 0, stage);
-        const int threads = stage ? kStageThreads : kTileThreads;
-        const size_t smem = stage ? (size_t)a.stage_n * (run.fp32 ? sizeof(float) : sizeof(double)) : 0;
-        if (stage) CMG_TRY(allow_max_dynamic_smem(kern));
-        int maxb = 0;
-        CMG_TRY(coop_max_blocks(kern, threads, smem, &maxb));
-        const int row_warps = threads / 32 - 1;
-        const long long tasks = (long long)a.lay_nsl + a.nchunks;
-        const int blocks = (int)std::max<long long>(1, std::min<long long>(maxb, (tasks + row_warps - 1) / row_warps));
+        int blocks, threads;
+        const void *kern;
+        size_t smem;
+        bool stream;
+        CMG_TRY(sell_geometry(L, lv.n, run.fp32, &blocks, &threads, &kern, &smem, &stream));
+        if (run.fp32 && L.res_e > 0) {
+            kern = sell_res_kernel(L.col16, a.lay_h > 0);
+            CMG_TRY(allow_max_dynamic_smem(kern));
+            smem = L.res_smem;
+            a.res_entries = L.res_e;
+        }
         double *partials;
         if (ws) {
             if (2 * blocks * kPartDoubles > ws->partials_cap) return CMG_ERR_TOO_LARGE;

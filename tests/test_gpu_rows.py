@@ -60,24 +60,17 @@ def test_row_kernel_fp64_matches_oracle(monkeypatch, name):
     assert abs(lam - ref_lam) <= 1e-12 * abs(ref_lam)
 
 
-def test_resident_fp32_levels_keep_the_slice_kernels_sums(monkeypatch):
-    """FP32 sweeps from shared memory add the same terms in the same order as
-    the slice kernel (CMG_STAGE=0), heavy rows in chunks included; only the
-    float-float stop sums group differently, which reaches the iterate through
-    the mean estimate at the 1e-14 level.  Two FP32 iterates that differ there
-    differ in single roundings (6e-8 of an entry) at most."""
+def test_resident_fp32_levels_give_the_slice_kernels_bits(monkeypatch):
+    """FP32 levels held in shared memory keep the slice kernel's CTAs, warps and
+    order: bit for bit the vector of the slice kernel reading its layout from
+    L2 (CMG_RESIDENT=0)."""
     rp, col, w = inputs.chung_lu(80000, seed=21)
-    replay = None
     got = {}
-    for mode in ("0", None):
-        if mode is None:
-            monkeypatch.delenv("CMG_STAGE", raising=False)
-        else:
-            monkeypatch.setenv("CMG_STAGE", mode)
-        kw = {} if replay is None else {"schedule": "replay", "replay_sweeps": replay}
-        with cmg.Hierarchy(rp, col, w, seed=1412, precision="fp32", **kw) as h:
+    for mode in ("0", "1"):
+        monkeypatch.setenv("CMG_RESIDENT", mode)
+        with cmg.Hierarchy(rp, col, w, seed=1412, precision="fp32") as h:
             assert "fp32" in h.level_precision()
             u, lam, st = h.fiedler()
-        replay = st["sweeps"]
-        got[mode] = u
-    assert np.abs(got["0"] - got[None]).max() <= 1.2e-7 * np.abs(got["0"]).max()
+        got[mode] = (u, st["sweeps"])
+    assert got["0"][1] == got["1"][1]
+    assert np.array_equal(got["0"][0], got["1"][0])
