@@ -1363,7 +1363,7 @@ int stage_capacity(int fp32) {
     DeviceInfo d;
     if (device_info(&d) != CMG_OK) return 0;
     cudaFuncAttributes fa;
-    const void *k = fp32 ? (const void *)k_power_sell<float, int, true, true, true, false, true>
+    const void *k = fp32 ? (const void *)k_power_sell<float, int, true, true, true, false>
                          : (const void *)k_power_sell<double, int, true, true, true, false>;
     if (cudaFuncGetAttributes(&fa, k) != cudaSuccess) return 0;
     const long long room = (long long)d.max_smem_optin - (long long)fa.sharedSizeBytes - 256;
