@@ -24,37 +24,95 @@ namespace cmg {
 // without host synchronisation; grids are sized by upper bounds (c <= n,
 // records <= nnz).
 
+// The row loops below take G lanes per row (lanes_for_avg), so that the longest row
+// does not set a kernel's time: with a thread per row a 2,000-entry row was 2,000
+// dependent trips to L2, about 1 ms per kernel and level on a 250K-vertex
+// Chung-Lu graph, whatever the other rows took.  All lanes of a warp iterate
+// together (the shuffles and ballots need them converged).
+template <int G>
 __global__ void k_count_cross(int n, const int *__restrict__ rp, const int *__restrict__ col,
                               const int *__restrict__ agg, int *__restrict__ cnt) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int a = agg[i];
+    const int lane = threadIdx.x & (G - 1);
+    const int groups = (gridDim.x * blockDim.x) / G;
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) / G;; i += groups) {
+        if (__shfl_sync(0xffffffffu, i, 0) >= n) break;
         int c = 0;
-        for (int e = __ldg(rp + i), e1 = __ldg(rp + i + 1); e < e1; e++) c += (a < agg[__ldg(col + e)]);
-        cnt[i] = c;
+        if (i < n) {
+            const int a = agg[i];
+            for (int e = __ldg(rp + i) + lane, e1 = __ldg(rp + i + 1); e < e1; e += G) c += (a < agg[__ldg(col + e)]);
+        }
+        c = group_sum<G>(c);
+        if (i < n && lane == 0) cnt[i] = c;
     }
 }
 
 // off[n] holds the cross-entry count; records (a, b) go to [0, ncross),
-// records (b, a) to [ncross, 2 ncross).
+// records (b, a) to [ncross, 2 ncross), a row's in entry order.
+template <int G>
 __global__ void k_emit(int n, const int *__restrict__ rp, const int *__restrict__ col,
                        const int *__restrict__ agg, const int *__restrict__ off, int bb,
                        uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
                        LevelCounts *__restrict__ cnt) {
     const long long ncross = off[n];
     if (blockIdx.x == 0 && threadIdx.x == 0) cnt->m = (int)(2 * ncross);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const uint64_t a = (uint64_t)agg[i];
-        long long k = off[i];
-        for (int e = __ldg(rp + i), e1 = __ldg(rp + i + 1); e < e1; e++) {
-            const uint64_t b = (uint64_t)agg[__ldg(col + e)];
-            if (a < b) {
-                keys[k] = (a << bb) | b;
-                vals[k] = (uint32_t)e;
-                keys[ncross + k] = (b << bb) | a;
-                vals[ncross + k] = (uint32_t)e;
-                k++;
+    const int lane = threadIdx.x & (G - 1), shift = (threadIdx.x & 31) & ~(G - 1);
+    const unsigned gmask = (G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u)) << shift;
+    const unsigned below = gmask & ((1u << (threadIdx.x & 31)) - 1u);
+    const int groups = (gridDim.x * blockDim.x) / G;
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) / G;; i += groups) {
+        if (__shfl_sync(0xffffffffu, i, 0) >= n) break;
+        const bool row = i < n;
+        const uint64_t a = row ? (uint64_t)agg[i] : 0;
+        long long k = row ? off[i] : 0;
+        int e = row ? __ldg(rp + i) + lane : 0;
+        const int e1 = row ? __ldg(rp + i + 1) : 0;
+        while (__any_sync(0xffffffffu, e < e1)) {
+            const uint64_t b = e < e1 ? (uint64_t)agg[__ldg(col + e)] : 0;
+            const bool cross = e < e1 && a < b;
+            const unsigned m = __ballot_sync(0xffffffffu, cross) & gmask;
+            if (cross) {
+                const long long q = k + __popc(m & below);
+                keys[q] = (a << bb) | b;
+                vals[q] = (uint32_t)e;
+                keys[ncross + q] = (b << bb) | a;
+                vals[ncross + q] = (uint32_t)e;
             }
+            k += __popc(m);
+            e += G;
         }
+    }
+}
+
+template <int G>
+static cmg_status_t launch_count_g(int n, const int *rp, const int *col, const int *agg, int *cnt, cudaStream_t s) {
+    k_count_cross<G><<<grid_for((long long)n * G, 256), 256, 0, s>>>(n, rp, col, agg, cnt);
+    return launch_status();
+}
+static cmg_status_t launch_count(int n, double avg, const int *rp, const int *col, const int *agg, int *cnt,
+                                 cudaStream_t s) {
+    switch (lanes_for_avg(avg)) {
+        case 2: return launch_count_g<2>(n, rp, col, agg, cnt, s);
+        case 4: return launch_count_g<4>(n, rp, col, agg, cnt, s);
+        case 8: return launch_count_g<8>(n, rp, col, agg, cnt, s);
+        case 16: return launch_count_g<16>(n, rp, col, agg, cnt, s);
+        default: return launch_count_g<32>(n, rp, col, agg, cnt, s);
+    }
+}
+
+template <int G>
+static cmg_status_t launch_emit_g(int n, const int *rp, const int *col, const int *agg, const int *off, int bb,
+                                  uint64_t *keys, uint32_t *vals, LevelCounts *cnt, cudaStream_t s) {
+    k_emit<G><<<grid_for((long long)n * G, 256), 256, 0, s>>>(n, rp, col, agg, off, bb, keys, vals, cnt);
+    return launch_status();
+}
+static cmg_status_t launch_emit(int n, double avg, const int *rp, const int *col, const int *agg, const int *off, int bb,
+                                uint64_t *keys, uint32_t *vals, LevelCounts *cnt, cudaStream_t s) {
+    switch (lanes_for_avg(avg)) {
+        case 2: return launch_emit_g<2>(n, rp, col, agg, off, bb, keys, vals, cnt, s);
+        case 4: return launch_emit_g<4>(n, rp, col, agg, off, bb, keys, vals, cnt, s);
+        case 8: return launch_emit_g<8>(n, rp, col, agg, off, bb, keys, vals, cnt, s);
+        case 16: return launch_emit_g<16>(n, rp, col, agg, off, bb, keys, vals, cnt, s);
+        default: return launch_emit_g<32>(n, rp, col, agg, off, bb, keys, vals, cnt, s);
     }
 }
 
@@ -144,8 +202,8 @@ cmg_status_t galerkin_async(int n, long long nnz, const int *rp, const int *col,
     int *ccount, *off;
     CMG_TRY(scr.get(&ccount, n));
     CMG_TRY(scr.get(&off, (size_t)n + 1));
-    k_count_cross<<<grid_for(n, threads), threads, 0, s>>>(n, rp, col, agg, ccount);
-    CMG_TRY(launch_status());
+    const double avg = (double)nnz / (double)std::max(1, n);
+    CMG_TRY(launch_count(n, avg, rp, col, agg, ccount, s));
     CMG_TRY(exclusive_scan(ccount, off, n, scr, s));
     uint64_t *ka, *kb;
     uint32_t *va, *vb;
@@ -153,8 +211,7 @@ cmg_status_t galerkin_async(int n, long long nnz, const int *rp, const int *col,
     CMG_TRY(scr.get(&kb, (size_t)cap));
     CMG_TRY(scr.get(&va, (size_t)cap));
     CMG_TRY(scr.get(&vb, (size_t)cap));
-    k_emit<<<grid_for(n, threads), threads, 0, s>>>(n, rp, col, agg, off, key_bits, ka, va, cnt);
-    CMG_TRY(launch_status());
+    CMG_TRY(launch_emit(n, avg, rp, col, agg, off, key_bits, ka, va, cnt, s));
     CMG_TRY(radix_sort_pairs(&ka, &va, kb, vb, (int)cap, &cnt->m, 2 * key_bits, scr, s));
     int *head, *segid, *row_of;
     CMG_TRY(scr.get(&head, (size_t)cap));
