@@ -92,6 +92,15 @@ static cmg_status_t launch_check(int n, double avg, const int *rp, const int *co
     }
 }
 
+// Without input checks: whether every weight is finite and positive, which the
+// fixed-point sweeps rely on.
+__global__ void k_check_weights(long long m, const double *__restrict__ w, unsigned *__restrict__ flags) {
+    unsigned f = 0;
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < m; k += (long long)gridDim.x * blockDim.x)
+        if (!(w[k] > 0.0) || isinf(w[k])) f = kBadWeight;
+    if (f) atomicOr(flags, f);
+}
+
 __global__ void k_to_float(long long m, const double *__restrict__ w, float *__restrict__ w32) {
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < m;
          k += (long long)gridDim.x * blockDim.x)
@@ -301,12 +310,23 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
     LevelData &Z = h->lv.back();
     CMG_TRY(load_level0(n, row_ptr, col, w, mem, o.validate, &Z.rp, &Z.col, &Z.w, &Z.nnz, s));
     Scratch scr(s);
+    bool fixed_ok = true;   // weights the fixed-point sweeps take
     {
         double *gd;
         CMG_TRY(scr.get(&gd, 1));
         CMG_TRY(launch_gershgorin((int)n, Z.rp, Z.w, gd, s));
         CMG_CUDA(cudaMemcpyAsync(&Z.g, gd, sizeof(double), cudaMemcpyDeviceToHost, s));
+        unsigned hf = 0;
+        if (!o.validate && Z.nnz > 0) {
+            unsigned *flags;
+            CMG_TRY(scr.get(&flags, 1));
+            CMG_CUDA(cudaMemsetAsync(flags, 0, sizeof(unsigned), s));
+            k_check_weights<<<grid_for(Z.nnz, 256), 256, 0, s>>>(Z.nnz, Z.w, flags);
+            CMG_TRY(launch_status());
+            CMG_CUDA(cudaMemcpyAsync(&hf, flags, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+        }
         CMG_CUDA(cudaStreamSynchronize(s));
+        fixed_ok = hf == 0;
     }
     // ---- Alg. 1 Step 1: coarsen while n_i > coarse_size.  Each level runs
     // HEC, the Galerkin product and the SELL-32 sizing on the device into
@@ -401,7 +421,7 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
         std::vector<int> who;
         for (int k = 0; k < nlev; k++) {
             const LevelData &L = h->lv[k];
-            if (L.fp32 || !fix_may_hold(L.n, L.nnz)) continue;
+            if (!fixed_ok || L.fp32 || !fix_may_hold(L.n, L.nnz)) continue;
             FixLevel f = {};
             f.n = L.n;
             f.nnz = L.nnz;
@@ -460,7 +480,7 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
             }
             // FP64 levels: the row kernel.  CMG_STAGE (either value) keeps the
             // slice kernel.
-            if (!L.fp32 && getenv("CMG_STAGE") == nullptr) {
+            if (fixed_ok && !L.fp32 && getenv("CMG_STAGE") == nullptr) {
                 size_t lb = 0, rb = 0;
                 CMG_TRY(build_sweep_layout(1, voff1, std::vector<int>{0, L.n}, L.n, L.rp, L.col, L.w, 0, &L.lay, &lb, s,
                                            true));

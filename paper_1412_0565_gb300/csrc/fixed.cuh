@@ -87,6 +87,7 @@ __device__ __forceinline__ long long fix_weight(double w, unsigned long long gin
     const unsigned long long h = __umul64hi(m, ginv);  // w / g = h 2^(we - ge - 63)
     const int sh = 3 - (we - ge);                     // times 2^60: h >> sh
     if (sh >= 64) return 0;
+    if (sh < 1) return 1ll << 59;   // w > g / 2: not a weight of this level
     return (long long)((h >> sh) + ((h >> (sh - 1)) & 1ull));
 }
 

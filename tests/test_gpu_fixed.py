@@ -122,3 +122,23 @@ def test_no_sweeps_returns_the_projected_start():
     ref = x0 - x0.mean()
     assert st["sweeps"][0] == 0
     assert aligned_err(u, ref / np.linalg.norm(ref)) <= 1e-12
+
+
+def test_unchecked_weights_outside_the_contract_keep_fp64_sweeps():
+    """validate=0 takes weights that are not positive; the fixed-point sweeps rely
+    on positive ones, so such a graph keeps the FP64 kernels: the signed operator
+    is iterated as it is (one sweep against plain numpy)."""
+    rp, col, w = inputs.grid2d(12, 11, "uniform", seed=2)
+    rows = np.repeat(np.arange(132), np.diff(rp))
+    w = np.where((rows + col) % 7 == 3, -0.1 * w, w)
+    x0 = np.random.default_rng(3).standard_normal(132)
+    with cmg.Hierarchy(rp, col, w, seed=1412, validate=0, max_levels=1, schedule="replay", replay_sweeps=[1]) as h:
+        g = h.level_csr(0)[3]
+        u, lam, st = h.fiedler(x0=x0)
+    x = x0 - x0.mean()
+    d = np.zeros(132)
+    np.add.at(d, rows, w)
+    y = (g - d) * x
+    np.add.at(y, rows, w * x[col])
+    y -= y.mean()
+    assert aligned_err(u, y / np.linalg.norm(y)) <= 1e-12
