@@ -480,7 +480,7 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
             }
             // FP64 levels: the row kernel.  CMG_STAGE (either value) keeps the
             // slice kernel.
-            if (fixed_ok && !L.fp32 && getenv("CMG_STAGE") == nullptr) {
+            if (fixed_ok && !L.fp32 && rows_may_hold(L.n, L.nnz) && getenv("CMG_STAGE") == nullptr) {
                 size_t lb = 0, rb = 0;
                 CMG_TRY(build_sweep_layout(1, voff1, std::vector<int>{0, L.n}, L.n, L.rp, L.col, L.w, 0, &L.lay, &lb, s,
                                            true));

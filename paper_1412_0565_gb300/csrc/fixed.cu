@@ -11,7 +11,6 @@ namespace cmg {
 
 constexpr int kFixMaxThreads = 1024;
 constexpr int kFixMaxCtas = 8;
-constexpr int kFixSums = 6;   // A, Bh, Bm, Ch, Cm and the maximum
 
 __device__ __forceinline__ unsigned fix_rank() {
     unsigned r;
@@ -41,6 +40,18 @@ __device__ __forceinline__ void fix_barrier(int C) {
     }
 }
 
+// Result -> buf[0], previous iterate -> buf[1], in row order (res: fix_finish).
+__device__ __forceinline__ void fix_write(const PiArgs &a, const int2 *ring, int nr, const int *res) {
+    const int rs = res[0];
+    const int2 *rr = ring + (size_t)(res[1] ? (rs + 2) % 3 : rs % 3) * nr, *rp = ring + (size_t)((rs + 2) % 3) * nr;
+    double *o0 = (double *)a.buf[0], *o1 = (double *)a.buf[1];
+    for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
+        const int v = a.perm[i];
+        o0[v] = fix_value(rr[i]);
+        o1[v] = rs > 0 ? fix_value(rp[i]) : 0.0;
+    }
+}
+
 // Every CTA holds the whole iterate ring and its share of the items.  A sweep:
 // warp 0 (control) turns the previous sweep's sums into decisions while the
 // row warps compute their items from the local iterate and store each row's
@@ -51,15 +62,16 @@ __device__ __forceinline__ void fix_barrier(int C) {
 // runs beside it.  Six row warps reduce a sum each: a warp that reduced its
 // own five sums spent 610 cycles on 16 warp reductions, and atomics into the
 // other CTAs another 900 (3 CTAs) to 2,200 (8 CTAs).
-// us per sweep before (cluster, FP64) and now: the 3,048-row level of the 100^3
-// grid 5.67 and 3.24.
+// us per sweep in FP64 (one cluster) and here: the 3,048-row level of the 100^3
+// grid 5.67 and 3.18.
 __global__ void __launch_bounds__(kFixMaxThreads) k_power_fix(PiArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ unsigned s_acc[2][kFixMaxCtas][kFixWords];   // the CTAs' stop sums by sweep parity
+    __shared__ __align__(16) long long s_acc[2][kFixMaxCtas][kFixSums];   // the CTAs' stop sums by sweep parity
+    __shared__ __align__(16) long long s_rec[32][kFixSums];               // the start's sums by warp
     __shared__ FixSlot s_slot[2];
-    __shared__ Ctl c;
     __shared__ double s_mx[32];
     __shared__ int s_bad;
+    __shared__ int s_res[2];       // sweeps of the result, annihilated
     const int n = a.n, nr = (n + 1) & ~1;
     const int C = (int)fix_ctas();
     const unsigned rank = fix_rank();
@@ -88,123 +100,65 @@ __global__ void __launch_bounds__(kFixMaxThreads) k_power_fix(PiArgs a) {
             s_item[k] = it;
         }
     }
-    for (int k = tid; k < 2 * kFixMaxCtas * kFixWords; k += blockDim.x) (&s_acc[0][0][0])[k] = 0;
-    if (tid == 0) s_bad = 0;
-    __syncthreads();
-    // ---- start vector, the same in every CTA: values as doubles in ring slot 0,
-    // their largest magnitude, then fixed point
-    {
-        const void *cb = nullptr;
-        double cmu = 0.0, cinv = 0.0;
-        if (a.start == 1) {
-            cb = a.cbuf[a.cres->buf];
-            cmu = a.cres->mu;
-            cinv = a.cres->inv_s;
-        }
-        double mx = 0.0;
-        int bad = 0;
-        for (int i = tid; i < n; i += blockDim.x) {
-            const double v = start_value(a, a.perm[i], cb, cmu, cinv);
-            reinterpret_cast<double *>(ring)[i] = v;
-            if (isfinite(v)) mx = fmax(mx, fabs(v));
-            else bad = 1;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        if (lane == 0) s_mx[warp] = mx;
-        if (bad) s_bad = 1;
-    }
-    __syncthreads();
-    double mx = 0.0;
-    for (int w = 0; w < nw; w++) mx = fmax(mx, s_mx[w]);
-    {
-        const int k = mx > 0.0 ? fix_start_exponent(mx) : 0;
-        FixSum f;
-        f.reset();
-        for (int i = tid; i < n; i += blockDim.x) {
-            const double v = reinterpret_cast<double *>(ring)[i];
-            const long long X = s_bad ? 0 : __double2ll_rn(ldexp(v, k));
-            const int2 x = fix_split(X);
-            f.add(X, x, x);
-            ring[i] = x;
-        }
-        unsigned w[3];
-        const long long v[3] = {f.A, f.Bh, f.Bm};
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-            fix_warp_words(v[j], w);
-            if (lane < 3) atomicAdd(&s_acc[0][0][3 * j + lane], lane == 0 ? w[0] : (lane == 1 ? w[1] : w[2]));
-        }
-    }
-    __syncthreads();
+    fix_start(a, ring, s_mx, s_rec, &s_bad);
+
+    const int limit = s_bad ? 0 : (a.mode == 1 ? max(a.k_fixed, 0) : a.max_sweeps);
     if (warp == 0) {
+        // ------------------------------------------------------ control warp
+        const double omt = 1.0 - a.tol, omt2 = omt * omt;
+        const float inv_n = 1.0f / (float)n;
+        FixCtl c;
         unsigned m;
-        const Part P = fix_part(lane < kFixWords ? s_acc[0][0][lane] : 0u, lane, &m);
-        if (lane == 0) {
-            const double mu0 = to_d(P.A) / (double)n;
-            double ss0 = to_d(P.B) - (double)n * mu0 * mu0;
-            if (ss0 < 0.0) ss0 = 0.0;
-            ctl_init(c, a, mu0, ss0, 0);
-            if (s_bad) {
-                // an infinity or NaN in the start vector: the sums never converge
-                // and every sweep returns NaN, so no sweep is run
-                c.mu_res = c.ss_res = c.cos_res = c.mu_res_prev = c.ss_res_prev = nan("");
-                c.res_sweep = a.mode == 1 ? max(a.k_fixed, 0) : a.max_sweeps;
-                c.capped = a.mode == 0 ? 1 : 0;
+        const long long v0 = fix_sum_records(&s_rec[0][0], nw, lane, &m);
+        fix_ctl_start(a, lane, v0, omt2, n, c, s_slot);
+        fix_barrier(C);   // every CTA is set up before another stores into it
+        int s = 0, rs = 0, code = 0;
+        bool counted = false;
+        FixSlot nx;
+        for (;; s++) {
+            if (s_slot[(s + 1) & 1].stop) break;
+            if (s >= limit) {
+                counted = true;
+                break;
             }
-            s_slot[1].M = fix_mean(ff_from_double(mu0));   // sweep 1: exact mean of y_0
-            s_slot[1].e = 0;
-            s_slot[1].stop = 0;
-            s_slot[0].M = 0;                               // sweep 2: m_1 = 0
-            s_slot[0].e = 0;
-            s_slot[0].stop = 0;
-        }
-    }
-    __syncthreads();
-    fix_barrier(C);   // every CTA is set up before another stores into it
-
-    // the C CTAs' words of sweep parity par, summed (word l in lane l)
-    auto total_word = [&](int par) -> unsigned {
-        unsigned w = 0;
-        if (lane < kFixWords)
-            for (int p = 0; p < C; p++) {
-                const unsigned v = s_acc[par][p][lane];
-                w = lane == 15 ? max(w, v) : w + v;
-            }
-        return w;
-    };
-    // shared-memory windows of the other CTAs, as offsets from this one's
-    unsigned win[kFixMaxCtas - 1];
-#pragma unroll
-    for (int p = 0; p < kFixMaxCtas - 1; p++)
-        win[p] = p < C - 1 ? fix_peer(smem_raw, p < (int)rank ? p : p + 1) - (unsigned)__cvta_generic_to_shared(smem_raw)
-                           : 0u;
-    const int nrw = nw - 1, rt = tid - 32, nrt = (int)blockDim.x - 32;
-
-    const bool no_sweeps = (a.mode == 1 && a.k_fixed <= 0) || s_bad;
-    int s = 0;
-    int exit_kind = no_sweeps ? 2 : 0;
-    int k0 = 0, k1 = 1;   // s, s + 1 modulo 3
-    while (!no_sweeps) {
-        const FixSlot sl = s_slot[(s + 1) & 1];
-        if (sl.stop) {
-            exit_kind = 1;
-            break;
-        }
-        if ((a.mode == 1 && s >= a.k_fixed) || (a.mode == 0 && s >= a.max_sweeps)) {
-            exit_kind = 2;
-            break;
-        }
-        const int2 *x = ring + (size_t)k0 * nr;
-        int2 *y = ring + (size_t)k1 * nr;
-        if (warp == 0) {
             if (s >= 1) {
-                unsigned m;
-                const Part P = fix_part(total_word(s & 1), lane, &m);
-                if (lane == 0) fix_ctrl(a, s, P, m, c, &s_slot[s & 1], false);
+                const long long v = fix_sum_records(&s_acc[s & 1][0][0], C, lane, &m);
+                code = fix_decide(a, lane, v, m, omt2, inv_n, c, &nx);
+                rs = s;
+                nx.stop = code == 2 || (code == 1 && a.mode == 0);
+                if (lane == 0) s_slot[s & 1] = nx;
                 __syncwarp();
             }
-        } else {
+            fix_barrier(C);
+        }
+        if (counted && limit > 0) {
+            const long long v = fix_sum_records(&s_acc[s & 1][0][0], C, lane, &m);
+            code = fix_decide(a, lane, v, m, omt2, inv_n, c, &nx);
+            rs = s;
+        }
+        fix_finish(a, lane, n, rs, code, counted, s_bad != 0, rank == 0, 0, c, s_res);
+        if (rank == 0 && lane == 0) {
+            // written to buf[0], the previous iterate to buf[1]
+            a.res->buf = 0;
+            a.res->buf_prev = 1;
+        }
+    } else {
+        // ------------------------------------------------------ row warps
+        // shared-memory windows of the other CTAs, as offsets from this one's
+        unsigned win[kFixMaxCtas - 1];
+#pragma unroll
+        for (int p = 0; p < kFixMaxCtas - 1; p++)
+            win[p] = p < C - 1
+                         ? fix_peer(smem_raw, p < (int)rank ? p : p + 1) - (unsigned)__cvta_generic_to_shared(smem_raw)
+                         : 0u;
+        const int nrw = nw - 1, rt = tid - 32, nrt = (int)blockDim.x - 32;
+        fix_barrier(C);
+        int k0 = 0, k1 = 1;   // s, s + 1 modulo 3
+        for (int s = 0;; s++) {
+            const FixSlot sl = s_slot[(s + 1) & 1];
+            if (sl.stop || s >= limit) break;
+            const int2 *x = ring + (size_t)k0 * nr;
+            int2 *y = ring + (size_t)k1 * nr;
             FixSum f;
             f.reset();
             for (int k = ib + warp - 1; k < ie; k += nrw) {
@@ -221,7 +175,7 @@ __global__ void __launch_bounds__(kFixMaxThreads) k_power_fix(PiArgs a) {
                 t.carry();
                 const long long pr = t.lanes(lg);
                 if (leads) {
-                    const long long Y = fix_row(xi, pr, sl.M, sl.e);
+                    const long long X = fix_join(xi), Y = fix_row(X, pr, sl.M, sl.e);
                     const int2 yv = fix_split(Y);
                     y[i] = yv;
                     const unsigned ya = (unsigned)__cvta_generic_to_shared(y + i);
@@ -230,72 +184,39 @@ __global__ void __launch_bounds__(kFixMaxThreads) k_power_fix(PiArgs a) {
                         if (p < C - 1)
                             asm volatile("st.shared::cluster.v2.s32 [%0], {%1, %2};" ::"r"(ya + win[p]), "r"(yv.x), "r"(yv.y)
                                          : "memory");
-                    f.add(Y, yv, xi);
+                    f.add(Y, yv, FixSum::narrow(Y), FixSum::narrow(X));
                 }
                 __syncwarp();
             }
-            s_lane[rt] = f.A;
-            s_lane[nrt + rt] = f.Bh;
-            s_lane[2 * nrt + rt] = f.Bm;
-            s_lane[3 * nrt + rt] = f.Ch;
-            s_lane[4 * nrt + rt] = f.Cm;
+            const FixVals fv = fix_vals(f, false);
+#pragma unroll
+            for (int v = 0; v < 5; v++) s_lane[v * nrt + rt] = fv.v[v];
             s_lane[5 * nrt + rt] = (long long)f.mx;
             bar_rows(nrt);
             for (int v = warp - 1; v < kFixSums; v += nrw) {
                 const long long *src = s_lane + v * nrt + lane;
-                unsigned w[3] = {0, 0, 0};
+                long long sum = 0;
                 if (v < 5) {
-                    long long sum = 0;
                     for (int k = 0; k < nrw; k++) sum += src[32 * k];
-                    fix_warp_words(sum, w);
+                    sum = warp_sum(sum);
                 } else {
                     unsigned m = 0;
                     for (int k = 0; k < nrw; k++) m = max(m, (unsigned)src[32 * k]);
-                    w[0] = __reduce_max_sync(0xffffffffu, m);
+                    sum = (long long)__reduce_max_sync(0xffffffffu, m);
                 }
-                // lane 3 p + j: word j of the sum into CTA p's slot of this rank
-                const int p = lane / 3, j = lane - 3 * p;
-                if (p < C && (v < 5 || j == 0)) {
-                    const unsigned word = j == 0 ? w[0] : (j == 1 ? w[1] : w[2]);
-                    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(fix_peer(&s_acc[(s + 1) & 1][rank][3 * v + j], p)),
-                                 "r"(word)
+                // lane p: the sum into CTA p's slot of this rank
+                if (lane < C)
+                    asm volatile("st.shared::cluster.s64 [%0], %1;" ::"r"(fix_peer(&s_acc[(s + 1) & 1][rank][v], lane)), "l"(sum)
                                  : "memory");
-                }
                 __syncwarp();
             }
-        }
-        fix_barrier(C);
-        s++;
-        k0 = k1;
-        k1 = k1 == 2 ? 0 : k1 + 1;
-    }
-    __shared__ int s_rb, s_rbp;
-    if (warp == 0) {
-        if (exit_kind == 2 && !no_sweeps) {
-            unsigned m;
-            const Part P = fix_part(total_word(s & 1), lane, &m);
-            if (lane == 0) fix_ctrl(a, s, P, m, c, nullptr, true);
-            __syncwarp();
-        }
-        if (lane == 0) {
-            const int rs = s_bad ? 0 : c.res_sweep;
-            s_rb = c.zero ? (rs + 2) % 3 : rs % 3;
-            s_rbp = (rs + 2) % 3;
-            if (rank == 0) write_result(a, c, 0, 1);
+            fix_barrier(C);
+            k0 = k1;
+            k1 = k1 == 2 ? 0 : k1 + 1;
         }
     }
     __syncthreads();
-    if (rank == 0) {
-        // result -> buf[0], previous iterate -> buf[1], in row order
-        double *o0 = (double *)a.buf[0], *o1 = (double *)a.buf[1];
-        const int2 *rr = ring + (size_t)s_rb * nr, *rp = ring + (size_t)s_rbp * nr;
-        const bool prev = c.res_sweep > 0 && !s_bad;
-        for (int i = tid; i < n; i += blockDim.x) {
-            const int v = a.perm[i];
-            o0[v] = fix_value(rr[i]);
-            o1[v] = prev ? fix_value(rp[i]) : 0.0;
-        }
-    }
+    if (rank == 0) fix_write(a, ring, nr, s_res);
 }
 
 // Row warps per CTA of the register form: 15 leave 128 registers a thread (with 31
@@ -305,24 +226,26 @@ constexpr int kFixWarps = 15;
 
 // The same sweeps with one item of at most U steps per row warp: a lane keeps its
 // entries (column offsets and coefficients) in registers for the whole launch,
-// so a sweep reads only the iterate; the warp reduces its own five sums and
-// stores them into every CTA's slots, where the control warps add them up.
+// so a sweep reads only the iterate; a leading lane keeps its row's value; the warp
+// reduces its own five sums and stores them into every CTA's slots, where the
+// control warps add them up.
 // Row warps and control warp run separate loops that meet at the barrier.  What
-// bounds a sweep is the longer of two chains: gathers, 24 multiply-adds, the
+// bounds a sweep is the longer of two chains: gathers, 32 multiply-adds, the
 // lanes' sums, finish, warp sums (about 900 cycles), and the control step
 // (about 1,000); then the barrier (60 cycles in one CTA, 420 in a cluster).
-// us per sweep before (FP64: one CTA up to 512 rows, cluster above), from
-// shared memory (k_power_fix) and here, the 853-, 239-, 66- and
+// us per sweep in FP64 (one CTA up to 512 rows, cluster above), from shared memory
+// (k_power_fix, with three of the four products) and here, the 853-, 239-, 66- and
 // 18-row levels of the 100^3 grid: 3.55 / 2.48 / 1.70 / 1.24, 2.85 / 2.05 / 1.37 /
-// 1.23, and 1.29 / 1.07 / 0.95 / 0.87.
+// 1.23, and 1.45 / 1.22 / 1.05 / 0.96 (1.29 / 1.07 / 0.95 / 0.87 with three products
+// and 57 bits: the fourth product and the wider sums are the price of the accuracy
+// stated in fixed.cuh).
 template <int U>
 __global__ void __launch_bounds__(32 * (kFixWarps + 1)) k_power_fix_reg(PiArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ __align__(16) long long s_rec[kFixWarps + 1][kFixSums];   // the start's sums by warp
     __shared__ FixSlot s_slot[2];
-    __shared__ double s_init[2];   // mean and squared norm of y_0
     __shared__ int s_res[2];       // sweeps of the result, annihilated
     __shared__ double s_mx[32];
-    __shared__ unsigned s_start[kFixWords];
     __shared__ int s_bad;
     const int n = a.n, nr = (n + 1) & ~1;
     const int C = (int)fix_ctas();
@@ -331,74 +254,8 @@ __global__ void __launch_bounds__(32 * (kFixWarps + 1)) k_power_fix_reg(PiArgs a
     const int nw = (int)(blockDim.x >> 5), nrw = nw - 1;
     int2 *ring = reinterpret_cast<int2 *>(smem_raw);                        // [3][nr]
     long long *s_acc = reinterpret_cast<long long *>(ring + 3 * (size_t)nr);   // [2][C][nrw][kFixSums]
-    if (tid < kFixWords) s_start[tid] = 0;
     for (int k = tid; k < 2 * C * nrw * kFixSums; k += blockDim.x) s_acc[k] = 0;
-    if (tid == 0) s_bad = 0;
-    __syncthreads();
-    // ---- start vector, as in k_power_fix
-    {
-        const void *cb = nullptr;
-        double cmu = 0.0, cinv = 0.0;
-        if (a.start == 1) {
-            cb = a.cbuf[a.cres->buf];
-            cmu = a.cres->mu;
-            cinv = a.cres->inv_s;
-        }
-        double mx = 0.0;
-        int bad = 0;
-        for (int i = tid; i < n; i += blockDim.x) {
-            const double v = start_value(a, a.perm[i], cb, cmu, cinv);
-            reinterpret_cast<double *>(ring)[i] = v;
-            if (isfinite(v)) mx = fmax(mx, fabs(v));
-            else bad = 1;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        if (lane == 0) s_mx[warp] = mx;
-        if (bad) s_bad = 1;
-    }
-    __syncthreads();
-    {
-        double mx = 0.0;
-        for (int w = 0; w < nw; w++) mx = fmax(mx, s_mx[w]);
-        const int k = mx > 0.0 ? fix_start_exponent(mx) : 0;
-        FixSum f;
-        f.reset();
-        for (int i = tid; i < n; i += blockDim.x) {
-            const double v = reinterpret_cast<double *>(ring)[i];
-            const long long X = s_bad ? 0 : __double2ll_rn(ldexp(v, k));
-            const int2 x = fix_split(X);
-            f.add(X, x, x);
-            ring[i] = x;
-        }
-        unsigned w[3];
-        const long long v[3] = {f.A, f.Bh, f.Bm};
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-            fix_warp_words(v[j], w);
-            if (lane < 3) atomicAdd(&s_start[3 * j + lane], lane == 0 ? w[0] : (lane == 1 ? w[1] : w[2]));
-        }
-    }
-    __syncthreads();
-    if (warp == 0) {
-        unsigned m;
-        const Part P = fix_part(lane < kFixWords ? s_start[lane] : 0u, lane, &m);
-        if (lane == 0) {
-            const double mu0 = to_d(P.A) / (double)n;
-            double ss0 = to_d(P.B) - (double)n * mu0 * mu0;
-            if (ss0 < 0.0) ss0 = 0.0;
-            s_init[0] = mu0;
-            s_init[1] = ss0;
-            s_slot[1].M = fix_mean(ff_from_double(mu0));
-            s_slot[1].e = 0;
-            s_slot[1].stop = 0;
-            s_slot[0].M = 0;
-            s_slot[0].e = 0;
-            s_slot[0].stop = 0;
-        }
-    }
-    __syncthreads();
-    fix_barrier(C);   // every CTA is set up before another stores into it
+    fix_start(a, ring, s_mx, s_rec, &s_bad);
 
     const int limit = s_bad ? 0 : (a.mode == 1 ? max(a.k_fixed, 0) : a.max_sweeps);
     if (warp == 0) {
@@ -407,31 +264,15 @@ __global__ void __launch_bounds__(32 * (kFixWarps + 1)) k_power_fix_reg(PiArgs a
         const float inv_n = 1.0f / (float)n;
         const int N = C * nrw;
         FixCtl c;
-        c.B = c.Bp = s_init[1];
-        c.K = omt2 * c.B;
-        c.Z = c.B * (double)a.zero_tol2;
-        c.C = 0.0;
-        c.muA = c.mu_p = s_init[0] * (double)n * 0x1p58;
-        c.M = 0;
-        c.e = 0;
+        unsigned m;
+        const long long v0 = fix_sum_records(&s_rec[0][0], nw, lane, &m);
+        fix_ctl_start(a, lane, v0, omt2, n, c, s_slot);
+        fix_barrier(C);   // every CTA is set up before another stores into it
         // totals of the sweep of parity par: a record per lane
         auto decide = [&](int par, FixSlot *next) -> int {
-            FixVals f;
-#pragma unroll
-            for (int j = 0; j < 5; j++) f.v[j] = 0;
-            unsigned m = 0;
-            for (int r = lane; r < N; r += 32) {
-                const longlong2 *src = reinterpret_cast<const longlong2 *>(s_acc + ((size_t)par * N + r) * kFixSums);
-                const longlong2 u0 = src[0], u1 = src[1], u2 = src[2];
-                f.v[0] += u0.x;
-                f.v[1] += u0.y;
-                f.v[2] += u1.x;
-                f.v[3] += u1.y;
-                f.v[4] += u2.x;
-                m = max(m, (unsigned)u2.y);
-            }
-            m = __reduce_max_sync(0xffffffffu, m);
-            return fix_decide(a, lane, fix_warp_vals(f, lane), m, omt2, inv_n, c, next);
+            unsigned mx;
+            const long long v = fix_sum_records(s_acc + (size_t)par * N * kFixSums, N, lane, &mx);
+            return fix_decide(a, lane, v, mx, omt2, inv_n, c, next);
         };
         int s = 0, rs = 0, code = 0;
         bool counted = false;
@@ -502,15 +343,19 @@ __global__ void __launch_bounds__(32 * (kFixWarps + 1)) k_power_fix_reg(PiArgs a
         long long *mine = s_acc + ((size_t)rank * nrw + warp - 1) * kFixSums + (sends ? vi : 0);
         const unsigned acc0 = sends && p0 < C ? fix_peer(mine, p0) : 0u, acc1 = sends && p1 < C ? fix_peer(mine, p1) : 0u;
         const unsigned pstep = (unsigned)(N * sizeof(long long));
+        // a leading lane keeps its row's value from sweep to sweep
+        int2 xi = ring[i];
+        long long X = fix_join(xi);
+        fix_barrier(C);
         int s = 0, b0 = 0, b1 = nr;   // ring slots of x and y
         for (;; s++) {
             const FixSlot sl = s_slot[(s + 1) & 1];
             if (sl.stop || s >= limit) break;
             if (have) {
                 const int2 *x = ring + b0;
-                const int2 xi = x[i];
                 FixAcc t;
                 t.reset();
+                t.add(xi, d);   // (while the gathers are in flight)
                 // groups of four entries: loads first
 #pragma unroll
                 for (int u0 = 0; u0 < U; u0 += 4) {
@@ -520,28 +365,32 @@ __global__ void __launch_bounds__(32 * (kFixWarps + 1)) k_power_fix_reg(PiArgs a
                     for (int u = 0; u < 4; u++) xv[u] = x[off[u0 + u]];
 #pragma unroll
                     for (int u = 0; u < 4; u++) t.add(xv[u], cf[u0 + u]);
+                    if (u0 == 4 && U > 8) t.fold();
                 }
-                t.add(xi, d);
                 t.carry();
                 const long long pr = t.lanes(lg);
-                FixSum f;
-                f.reset();
+                FixVals f;
+                unsigned mx = 0;
+#pragma unroll
+                for (int j = 0; j < 5; j++) f.v[j] = 0;
                 if (leads) {
-                    const long long Y = fix_row(xi, pr, sl.M, sl.e);
-                    const int2 yv = fix_split(Y);
+                    const int2 xp = xi;
+                    X = fix_row(X, pr, sl.M, sl.e);
+                    xi = fix_split(X);
                     int2 *yp = ring + b1 + i;
-                    *yp = yv;
+                    *yp = xi;
                     const unsigned ya = (unsigned)__cvta_generic_to_shared(yp);
 #pragma unroll
                     for (int p = 0; p < kFixMaxCtas - 1; p++)
                         if (p < C - 1)
-                            asm volatile("st.shared::cluster.v2.s32 [%0], {%1, %2};" ::"r"(ya + win[p]), "r"(yv.x), "r"(yv.y)
+                            asm volatile("st.shared::cluster.v2.s32 [%0], {%1, %2};" ::"r"(ya + win[p]), "r"(xi.x), "r"(xi.y)
                                          : "memory");
-                    f.add(Y, yv, xi);
+                    f = fix_vals_row(X, xi, xp);
+                    mx = (unsigned)abs(xi.x);
                 }
                 __syncwarp();
-                const unsigned mx = __reduce_max_sync(0xffffffffu, f.mx);
-                long long v = fix_warp_vals(fix_vals(f), lane);
+                mx = __reduce_max_sync(0xffffffffu, mx);
+                long long v = fix_warp_vals(f, lane);
                 if (grp == 6) v = (long long)mx;
                 const unsigned po = ((s + 1) & 1) ? pstep : 0u;
                 if (acc0) asm volatile("st.shared::cluster.s64 [%0], %1;" ::"r"(acc0 + po), "l"(v) : "memory");
@@ -554,17 +403,7 @@ __global__ void __launch_bounds__(32 * (kFixWarps + 1)) k_power_fix_reg(PiArgs a
         }
     }
     __syncthreads();
-    if (rank == 0) {
-        const int rs = s_res[0];
-        const int rb = s_res[1] ? (rs + 2) % 3 : rs % 3, rbp = (rs + 2) % 3;
-        double *o0 = (double *)a.buf[0], *o1 = (double *)a.buf[1];
-        const bool prev = rs > 0;
-        for (int i = tid; i < n; i += blockDim.x) {
-            const int v = a.perm[i];
-            o0[v] = fix_value(ring[(size_t)rb * nr + i]);
-            o1[v] = prev ? fix_value(ring[(size_t)rbp * nr + i]) : 0.0;
-        }
-    }
+    if (rank == 0) fix_write(a, ring, nr, s_res);
 }
 
 // ------------------------------------------------------------------ host side

@@ -5,22 +5,36 @@
 // multiply-add with a 64-bit result issues every 2 to 4).  B_g / g = I - L / g
 // has non-negative entries and row sums 1, so a sweep is an average: no entry
 // of the result exceeds the largest of the iterate, and a common power-of-two
-// scale serves the whole vector.  The FP64 form's sweeps are therefore run on
-// the integer pipe, in 60-bit fixed point:
-//   iterate   X = q 2^29 + r   (q, r: signed 32-bit, |r| <= 2^28, |X| < 2^59),
-//             y = X 2^-58, rescaled by powers of two so that max |X| stays near
-//             2^56 (the sweep's own maximum is reduced with its sums);
-//   entries   C_ij = round(w_ij / g 2^60) = c1 2^29 + c0, D_i = sum_j C_ij exactly
-//             (constant vectors are fixed points, as in exact arithmetic);
-//   row       X_i - D_i X_i + sum_j C_ij X_j with the products q c1 and
-//             q c0 + r c1 accumulated in two 64-bit sums (r c0, below 2^-4 units
-//             of the result's last bit, is dropped), rounded once.
-// A sweep's rounding error is half a unit of 2^-55 to 2^-56 relative to max |x|, where
-// FP64's three roundings of g u - L u are about 2^-53 of each entry and of g - d_i:
-// over the families and sizes of the tests, and the timed cases, the vector's
-// error against a 64-bit reference is no larger than the FP64 sweeps' was.
-// The stop sums (sum y, sum y^2, sum y y_prev) are integers as well: exact to
-// 2^-28 of the last bit's square, and the same in every order of addition.
+// scale serves the whole vector.  The FP64 form's sweeps of levels of up to
+// kFixRowsMax rows are therefore run on the integer pipe:
+//   iterate   X = q 2^32 + r   (q, r: signed 32-bit, |X| < 2^62), y = X 2^-64,
+//             rescaled by powers of two so that max |X| stays in [2^61, 2^62)
+//             (the sweep's own maximum is reduced with its sums);
+//   entries   C_ij = round(w_ij / g 2^60) = c1 2^29 + c0, D_i = sum_j C_ij exactly;
+//   row       X_i + round((sum_j C_ij X_j - D_i X_i) 2^-60), all four products
+//             exact in 64-bit sums, one rounding to nearest per row (the lanes of a
+//             row each cut 2^-24 units before it).  Rows of a constant vector
+//             give 0, so constant vectors are fixed points, and a mean that is
+//             rounded to a whole unit only moves the vector along 1, which the
+//             result's projection takes out.
+// What it costs in accuracy.  The only rounding of a sweep is half a unit of at
+// most 2^-61 max |x| per entry, 0.29 2^-61 sqrt(n) max |x| as a vector; FP64 rounds
+// its largest entry by 0.29 2^-53 to 0.29 2^-52 of it, several times a sweep (and
+// g - d_i, the same in every sweep, by as much).  With sqrt(n) <= 2^8 the noise of the whole vector is no
+// more than that of one FP64 rounding of its largest entry, however localised the
+// vector is: that is where kFixRowsMax lies, and larger levels keep the FP64
+// kernels.  A coefficient is off by 2^-61 g, FP64's diagonal g - d_i by 2^-54 g.
+// A CPU model of both forms against 64-bit mantissas, 300 / 2,000 sweeps from one
+// start, error of the vector: Barabasi-Albert graph of 20K vertices from a random
+// start 1.5e-14 / 6.4e-14 (FP64) and 1.6e-16 / 4.2e-16 (here); on a pendant path
+// of ten vertices 1.2e-14 / 3.8e-14 and 5e-17 / 7e-17; 65K vertices 1.8e-14 /
+// 6.6e-14 and 1.1e-16 / 1.5e-16; on one vertex behind an edge of weight 0.01, the
+// form's worst case, 6e-17 / 1.1e-16 and 9e-17 / 1.0e-16 (20K), 5e-17 / 1.1e-16 and
+// 2.0e-16 / 2.4e-16 (65K), where storing the result as doubles costs 1e-16 itself.
+// (With |X| < 2^57 and the products r c0 dropped, the last but one rows read
+// 7e-15 / 9e-15 and the 20K vertex 6e-15 / 6.5e-15: above FP64.)
+// The stop sums (sum y, sum y^2, sum y y_prev) are integers as well, taken from X
+// rounded to 60 bits, and the same in every order of addition.
 #pragma once
 
 #include "pi_kernels.cuh"
@@ -28,7 +42,8 @@
 namespace cmg {
 
 // ------------------------------------------------------------------ plan
-constexpr int kFixMaxN = 4096;   // rows of a level k_power_fix takes
+constexpr int kFixMaxN = 4096;        // rows of a level k_power_fix takes
+constexpr int kFixRowsMax = 65536;    // rows of a level any fixed-point kernel takes (see above)
 
 // What a plan kernel reports to the host.
 struct PlanOut {
@@ -60,7 +75,7 @@ cmg_status_t launch_plan_small(const SmallJob *jobs_dev, int count, cudaStream_t
 cmg_status_t launch_fill_small(const SmallJob *jobs_dev, int count, cudaStream_t s);
 
 // ------------------------------------------------------------------ arithmetic
-constexpr int kFixBits = 58;   // y = X 2^-58
+constexpr int kFixTop = 62;   // |X| < 2^62; y = X 2^-64
 
 __device__ __forceinline__ long long mad_s(int a, int b, long long c) {
     long long d;
@@ -68,9 +83,16 @@ __device__ __forceinline__ long long mad_s(int a, int b, long long c) {
     return d;
 }
 
+// X = q 2^32 + r
 __device__ __forceinline__ int2 fix_split(long long X) {
-    const int q = (int)((X + (1ll << 28)) >> 29);
-    return make_int2(q, (int)(X - ((long long)q << 29)));
+    return make_int2((int)((X + (1ll << 31)) >> 32), (int)(unsigned)X);
+}
+__device__ __forceinline__ long long fix_join(int2 x) { return (long long)((unsigned long long)x.x << 32) + x.y; }
+
+// C = c1 2^29 + c0 (|c0| <= 2^28, |c1| <= 2^30)
+__device__ __forceinline__ int2 fix_split_c(long long C) {
+    const int q = (int)((C + (1ll << 28)) >> 29);
+    return make_int2(q, (int)(C - ((long long)q << 29)));
 }
 
 // round(w / g 2^60) for 0 < w <= g / 2: w as a normalised 64-bit mantissa times
@@ -91,32 +113,42 @@ __device__ __forceinline__ long long fix_weight(double w, unsigned long long gin
     return (long long)((h >> sh) + ((h >> (sh - 1)) & 1ull));
 }
 
-// Accumulators of one lane's part of a row: hi in units of 2^58, m1 and m2 of 2^29
-// (of the product X C).  m1 takes at most 32 products q c0 (below 2^55 each)
-// between carries; three chains, since a multiply-add waits for its own.
+// Accumulators of one lane's part of a row: hi in units of 2^61, m1 of 2^32, m2 of
+// 2^29 and m0 of 1 (of the product X C).  The coefficients of a row and its diagonal
+// add up to at most 2^60, so |hi| < 2^61 and |m2| < 2^62 over any row; m0 takes 15
+// products (below 2^59 each) between folds, m1 30 (below 2^58) between carries.
 struct FixAcc {
-    long long hi, m1, m2;
-    __device__ __forceinline__ void reset() { hi = m1 = m2 = 0; }
+    long long hi, m1, m2, m0;
+    __device__ __forceinline__ void reset() { hi = m1 = m2 = m0 = 0; }
     __device__ __forceinline__ void add(int2 x, int2 c) {
         hi = mad_s(x.x, c.x, hi);
         m1 = mad_s(x.x, c.y, m1);
         m2 = mad_s(x.y, c.x, m2);
+        m0 = mad_s(x.y, c.y, m0);
     }
-    // after at most 32 entries
+    // after at most 15 entries
+    __device__ __forceinline__ void fold() {
+        m1 += m0 >> 32;
+        m0 &= 0xffffffffll;
+    }
+    // after at most 30 entries
     __device__ __forceinline__ void carry() {
-        m1 += m2;
+        fold();
         hi += m1 >> 29;
         m1 &= (1ll << 29) - 1;
-        m2 = 0;
     }
-    // the accumulated product / 2^60 in sixteenths, and its sum over aligned
-    // groups of 2^lg lanes (after carry).  Each lane rounds to nearest: cutting here
-    // shifts a row by up to half a unit per sweep in the same direction, and
-    // thousands of sweeps add that up (1e-12 in lambda2 on a power-law graph).
+    // round(product 2^-60) of the sum over aligned groups of 2^lg lanes (after carry):
+    // the lanes' parts below 2^61 travel in units of 2^36, so that a row of 32
+    // lanes is rounded once, like a row of one (cutting them at the result's unit
+    // would shift every row the same way, sweep after sweep).
     __device__ __forceinline__ long long lanes(int lg) const {
-        long long v = (hi << 2) + ((m1 + (1ll << 26)) >> 27);
-        for (int o = (1 << lg) >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        return v;
+        unsigned long long h = (unsigned long long)(hi + (m2 >> 32));
+        unsigned l = ((unsigned)m1 >> 4) + ((unsigned)m2 >> 7);   // < 2^26 (m0 is below its unit)
+        for (int o = (1 << lg) >> 1; o > 0; o >>= 1) {
+            h += __shfl_xor_sync(0xffffffffu, h, o);
+            l += __shfl_xor_sync(0xffffffffu, l, o);
+        }
+        return (long long)(2 * h) + (long long)((l + (1u << 23)) >> 24);
     }
 };
 
@@ -134,7 +166,8 @@ __device__ __forceinline__ void fix_quads(FixAcc &t, int steps, const IDX *col, 
         for (int j = 0; j < 8; j++) xx[j] = ldx(cc[j]);
 #pragma unroll
         for (int j = 0; j < 8; j++) t.add(xx[j], cf[32 * j]);
-        if ((u & 24) == 24) t.carry();
+        if (u & 8) t.carry();
+        else t.fold();
     }
     if (u < steps) {
         int cc[4];
@@ -149,63 +182,78 @@ __device__ __forceinline__ void fix_quads(FixAcc &t, int steps, const IDX *col, 
     t.carry();
 }
 
-// The row's new value: p is the lane-summed product of its entries and of its
-// diagonal (-D_i) in sixteenths.
-__device__ __forceinline__ long long fix_row(int2 xi, long long p, long long M, int e) {
-    const long long X = ((long long)xi.x << 29) + xi.y;
-    return (X + ((p + 8) >> 4) - M) << e;
+// The row's new value: p is the rounded product of its entries and of its diagonal
+// (-D_i).
+__device__ __forceinline__ long long fix_row(long long X, long long p, long long M, int e) {
+    return (long long)((unsigned long long)(X + p - M) << e);
 }
 
-// Stop sums of the rows a lane computed in one sweep.
+// Stop sums of the rows a lane computed in one sweep: A in units of X (modulo 2^64:
+// the total is a few units a row), the others of X' = X / 4 rounded, |X'| <= 2^60 =
+// q 2^32 + r: B = Bh 2^64 + Bm 2^37, C = Ch 2^64 + Cm 2^36.  Up to 64 rows fit
+// (q^2 <= 2^56).
 struct FixSum {
     long long A, Bh, Bm, Ch, Cm;
-    unsigned mx;
+    unsigned mx;   // max |q| of X
     __device__ __forceinline__ void reset() {
         A = Bh = Bm = Ch = Cm = 0;
         mx = 0;
     }
-    __device__ __forceinline__ void add(long long Y, int2 y, int2 x) {
-        A += Y;
+    static __device__ __forceinline__ int2 narrow(long long X) { return fix_split((X + 2) >> 2); }   // X'
+    __device__ __forceinline__ void square(int2 y, int2 q) {
         Bh = mad_s(y.x, y.x, Bh);
-        // X^2 = q^2 2^58 + (q r + r^2 / 2^30) 2^30, and likewise X P
-        Bm = mad_s(y.x, y.y, Bm) + (mad_s(y.y, y.y, 1ll << 29) >> 30);
+        // X'^2 = q^2 2^64 + (q r + r^2 / 2^33) 2^33
+        Bm += mad_s(y.x, y.y, mad_s(y.y, y.y, 0) >> 33) >> 4;
+        mx = max(mx, (unsigned)abs(q.x));
+    }
+    // a row whose value became Y = q; y, x: X' of the new and the old value
+    __device__ __forceinline__ void add(long long Y, int2 q, int2 y, int2 x) {
+        A += Y;
+        square(y, q);
         Ch = mad_s(y.x, x.x, Ch);
-        Cm = mad_s(y.x, x.y, mad_s(y.y, x.x, Cm)) + (mad_s(y.y, x.y, 1ll << 28) >> 29);
-        mx = max(mx, (unsigned)abs(y.x));
+        Cm += mad_s(y.x, x.y, mad_s(y.y, x.x, mad_s(y.y, x.y, 0) >> 32)) >> 4;
+    }
+    // an entry of the start vector, whose sum is far from 0: its low 20 bits to A,
+    // the others to Ch
+    __device__ __forceinline__ void add_start(long long X, int2 q) {
+        A += X & 0xfffff;
+        Ch += X >> 20;
+        square(narrow(X), q);
     }
 };
 
-// A sweep's sums as 16 words that add with 32-bit atomics in any order: three
-// words of 22 bits (the third signed) per sum, then max |q|.  Totals of up to
-// 2^14 rows fit.
-constexpr int kFixWords = 16;
+constexpr int kFixSums = 6;   // 64-bit words of a record of sums: five values and max |q|
 
-// The three words of a warp's 64-bit sum (carried, so that the words of up to
-// 1,023 warps add without overflow); every lane receives them.
-__device__ __forceinline__ void fix_warp_words(long long v, unsigned (&w)[3]) {
-    unsigned s0 = __reduce_add_sync(0xffffffffu, (unsigned)v & 0x3fffffu);
-    unsigned s1 = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 22) & 0x3fffffu);
-    unsigned s2 = __reduce_add_sync(0xffffffffu, (unsigned)(int)(v >> 44));
-    s1 += s0 >> 22;
-    w[0] = s0 & 0x3fffffu;
-    w[2] = s2 + (s1 >> 22);
-    w[1] = s1 & 0x3fffffu;
-}
-
-// A lane's sums in five 64-bit values whose totals over up to 4,096 rows fit: A (its
-// total is near 0: exact modulo 2^64), then B as U 2^74 + V 2^30 and C as
-// U 2^74 + V 2^29 (units of X^2).
+// A lane's sums in five 64-bit values whose totals fit: A, then B as U 2^80 + V 2^37 and
+// C as U 2^80 + V 2^36 (units of X'^2).  A row adds at most 2^40 to a U and a lane
+// 2^44 to a V: 2^22 rows and 2^18 lanes fit (kFixRowsMax rows take at most 2^17).
+// start: A's two parts and B.
 struct FixVals {
     long long v[5];
 };
-__device__ __forceinline__ FixVals fix_vals(const FixSum &f) {
+__device__ __forceinline__ FixVals fix_vals(const FixSum &f, bool start) {
     FixVals r;
-    const long long bh = f.Bh + (f.Bm >> 28), ch = f.Ch + (f.Cm >> 29);
+    const long long bh = f.Bh + (f.Bm >> 27), ch = f.Ch + (f.Cm >> 28);
     r.v[0] = f.A;
     r.v[1] = bh >> 16;
-    r.v[2] = ((bh & 0xffff) << 28) + (f.Bm & ((1ll << 28) - 1));
-    r.v[3] = ch >> 16;
-    r.v[4] = ((ch & 0xffff) << 29) + (f.Cm & ((1ll << 29) - 1));
+    r.v[2] = ((bh & 0xffff) << 27) + (f.Bm & ((1ll << 27) - 1));
+    r.v[3] = start ? f.Ch : ch >> 16;
+    r.v[4] = start ? 0 : ((ch & 0xffff) << 28) + (f.Cm & ((1ll << 28) - 1));
+    return r;
+}
+
+// The same values of a single row that went from x to Y = y, in fewer steps (one row
+// fits without the narrower X').
+__device__ __forceinline__ FixVals fix_vals_row(long long Y, int2 y, int2 x) {
+    FixVals r;
+    // X^2 = bh 2^64 + (bm mod 2^31) 2^33, X P = ch 2^64 + (cm mod 2^32) 2^32
+    const long long bm = mad_s(y.x, y.y, mad_s(y.y, y.y, 0) >> 33), bh = mad_s(y.x, y.x, bm >> 31);
+    const long long cm = mad_s(y.x, x.y, mad_s(y.y, x.x, mad_s(y.y, x.y, 0) >> 32)), ch = mad_s(y.x, x.x, cm >> 32);
+    r.v[0] = Y;
+    r.v[1] = bh >> 20;
+    r.v[2] = ((bh & 0xfffff) << 23) + (((unsigned)bm & 0x7fffffffu) >> 8);
+    r.v[3] = ch >> 20;
+    r.v[4] = ((ch & 0xfffff) << 24) + ((unsigned)cm >> 8);
     return r;
 }
 
@@ -228,52 +276,35 @@ __device__ __forceinline__ long long fix_warp_vals(const FixVals &f, int lane) {
     return e;
 }
 
-// Float-float of v 2^e by integer operations (a 64-bit conversion takes about 160
-// cycles): the leading 24 bits, then the next 24, truncated.  Exponents must stay
-// in the floats' range.
-__device__ __forceinline__ ff fix_ff(long long v, int e) {
-    const unsigned sign = v < 0 ? 0x80000000u : 0u;
-    unsigned long long m = v < 0 ? (unsigned long long)(-v) : (unsigned long long)v;
-    if (m == 0) return ff_zero();
-    const int lz = __clzll((long long)m);
-    m <<= lz;                                    // value = m 2^(e - lz)
-    const int x = 63 - lz + e;                   // exponent of the leading bit
-    const float h = __uint_as_float(sign | ((unsigned)(x + 127) << 23) | ((unsigned)(m >> 40) & 0x7fffffu));
-    const unsigned r = (unsigned)(m >> 16) & 0xffffffu;
-    const float l = __uint2float_rn(r) * __uint_as_float((unsigned)(x - 47 + 127) << 23);
-    return fast_two_sum(h, sign ? -l : l);
+// A warp's sums as a record of kFixSums words.
+__device__ __forceinline__ void fix_warp_record(const FixSum &f, bool start, int lane, long long *rec) {
+    const unsigned m = __reduce_max_sync(0xffffffffu, f.mx);
+    long long v = fix_warp_vals(fix_vals(f, start), lane);
+    const int grp = lane >> 2;
+    if (grp == 6) v = (long long)m;
+    if ((lane & 3) == 0 && grp != 3 && grp != 7) rec[grp < 3 ? grp : grp - 1] = v;
+    __syncwarp();
 }
 
-// Stop sums in units of y from the total words (lane l holds word l, l < 16);
-// every lane receives them, and max |q| through *mx.
-__device__ __forceinline__ Part fix_part(unsigned word, int lane, unsigned *mx) {
-    *mx = __shfl_sync(0xffffffffu, word, 15);
-    // lane k < 5: sum k = w0 + 2^22 w1 + 2^44 w2
-    const unsigned w0 = __shfl_sync(0xffffffffu, word, min(3 * lane, 31));
-    const unsigned w1 = __shfl_sync(0xffffffffu, word, min(3 * lane + 1, 31));
-    const int w2 = (int)__shfl_sync(0xffffffffu, word, min(3 * lane + 2, 31));
-    const long long top = ((long long)w2 << 22) + (long long)w1 + (long long)(w0 >> 22);   // units of 2^22
-    // the low 22 bits are below 2^-48 of any sum that matters beside them
-    ff s = fix_ff(top, 22);
-    s = ff_add_f(s, (float)(w0 & 0x3fffffu));
-    auto get = [&](int k) {
-        return ff_make(__shfl_sync(0xffffffffu, s.hi, k), __shfl_sync(0xffffffffu, s.lo, k));
-    };
-    auto scale = [](ff a, float p) { return ff_make(a.hi * p, a.lo * p); };
-    const ff A = get(0), Bh = get(1), Bm = get(2), Ch = get(3), Cm = get(4);
-    Part P;
-    P.A = scale(A, 0x1p-58f);
-    P.B = ff_add(scale(Bh, 0x1p-58f), scale(Bm, 0x1p-86f));
-    P.C = ff_add(scale(Ch, 0x1p-58f), scale(Cm, 0x1p-87f));
-    return P;
-}
-
-// round(m 2^58) for a float-float m in (-2, 2); beyond the first sweeps the mean is a
-// few units, and the 32-bit conversion is the fast one
-__device__ __forceinline__ long long fix_mean(ff m) {
-    const float h = m.hi * 0x1p58f;
-    if (fabsf(h) < 0x1p30f) return __float2int_rn(h) + __float2int_rn((h - rintf(h)) + m.lo * 0x1p58f);
-    return __float2ll_rn(m.hi * 0x1p58f) + __float2ll_rn(m.lo * 0x1p58f);
+// Sum of `count` records (16-byte aligned) by one warp: value by lane group as
+// fix_warp_vals leaves it, and max |q| of all.
+__device__ __forceinline__ long long fix_sum_records(const long long *rec, int count, int lane, unsigned *mx) {
+    FixVals f;
+    unsigned m = 0;
+#pragma unroll
+    for (int j = 0; j < 5; j++) f.v[j] = 0;
+    for (int r = lane; r < count; r += 32) {
+        const longlong2 *src = reinterpret_cast<const longlong2 *>(rec + (size_t)r * kFixSums);
+        const longlong2 u0 = src[0], u1 = src[1], u2 = src[2];
+        f.v[0] += u0.x;
+        f.v[1] += u0.y;
+        f.v[2] += u1.x;
+        f.v[3] += u1.y;
+        f.v[4] += u2.x;
+        m = max(m, (unsigned)u2.y);
+    }
+    *mx = __reduce_max_sync(0xffffffffu, m);
+    return fix_warp_vals(f, lane);
 }
 
 // Slot of a fixed-point sweep: mean to subtract, rescale, decisions.
@@ -282,43 +313,11 @@ struct FixSlot {
     int e, stop;
 };
 
-// The control step of sweep s >= 1 (ctrl_step's decisions, from the integer
-// sums): fills the slot of sweep s + 2.  mx: max |q| of sweep s.
-__device__ __forceinline__ void fix_ctrl(const PiArgs &a, int s, const Part &P, unsigned mx, Ctl &c, FixSlot *next,
-                                         bool count_exit) {
-    const float nf = (float)a.n;
-    const ff mu = ff_mul(P.A, c.inv_n);
-    const ff ss = ff_add_f(P.B, -nf * mu.hi * mu.hi);
-    const ff cs = ff_add_f(P.C, -nf * mu.hi * c.mu_prev.hi);
-    const bool zero = ss.hi <= a.zero_tol2 * (c.e_prev ? ldexpf(c.ss_prev.hi, 2 * c.e_prev) : c.ss_prev.hi);
-    const bool conv = cs.hi > 0.f && !ff_lt(ff_mul(cs, cs), ff_mul(ff_mul(ss, c.ss_prev), c.omt2));
-    bool stop = zero;
-    if (a.mode == 0) stop = stop || conv || count_exit;
-    else stop = stop || count_exit;
-    if (stop && !c.stopped) ctl_stop(a, s, mu, ss, cs, zero, conv, c);
-    const ff dm = ff_sub(mu, c.m_cur);
-    const ff m_next = c.e_cur ? ff_make(ldexpf(dm.hi, c.e_cur), ldexpf(dm.lo, c.e_cur)) : dm;
-    // |X_s| < 2^b, so |X_{s+1}| < 2^(b + e_s) (an average, less a mean of a few
-    // units): lift it to 2^56, so that 248 rows' q^2 add up below 2^63
-    const int b = 61 - __clz((int)mx) + c.e_cur;
-    const int e_next = min(24, max(0, 56 - b));
-    if (next) {
-        next->M = fix_mean(m_next);
-        next->e = e_next;
-        next->stop = stop ? 1 : 0;
-    }
-    c.mu_prev = mu;
-    c.ss_prev = ss;
-    c.m_cur = m_next;
-    c.e_prev = c.e_cur;
-    c.e_cur = e_next;
-}
-
-// State of the register form's control warp, by lane where noted (the warp runs
-// one chain per sweep whose length is instructions, fetched anew every sweep
-// behind the row warps' code: the decisions are taken with a few FP64
-// instructions on the totals, whose pipe the sweeps leave idle, where the
-// float-float form of fix_ctrl takes 300 FP32 instructions).
+// State of the control warp, by lane where noted (the warp runs one chain per sweep
+// whose length is instructions, fetched anew every sweep behind the row warps'
+// code: the decisions are taken with a few FP64 instructions on the totals, whose
+// pipe the sweeps leave idle, where ctrl_step's float-float form takes 300 FP32
+// instructions).
 struct FixCtl {
     double B, K, Z;    // lanes 4..7: ||y||^2 of the last sweep, times (1 - tol)^2,
                        // times the annihilation threshold of the next
@@ -329,15 +328,15 @@ struct FixCtl {
     int e;             // rescale of the next sweep
 };
 
-// One control step for sweep s >= 1 (fix_ctrl's decisions): v is the sweep's
+// One control step for sweep s >= 1 (ctrl_step's decisions): v is the sweep's
 // total of the lane's value (fix_warp_vals' placement), mx its max |q|.
 // Returns 0, 1 (converged) or 2 (annihilated); *next: M, e of sweep s + 2.
 __device__ __forceinline__ int fix_decide(const PiArgs &a, int lane, long long v, unsigned mx, double omt2, float inv_n,
                                           FixCtl &c, FixSlot *next) {
     const int grp = lane >> 2;
-    // value to double, in units of y y (2^116) or, for A, of X
+    // value to double, in units of y y (2^124 of X' X') or, for A, of X
     double d = __ll2double_rn(v);
-    const int sh = grp == 0 ? 0 : (grp == 1 || grp == 4 ? -42 : (grp == 2 ? -86 : -87));
+    const int sh = grp == 0 ? 0 : (grp == 1 || grp == 4 ? -44 : (grp == 2 ? -87 : -88));
     if (v != 0) d = __hiloint2double(__double2hiint(d) + (sh << 20), __double2loint(d));
     const double up = __shfl_down_sync(0xffffffffu, d, 4);
     const double t = d + up;                 // lanes 4..7: B, 16..19: C
@@ -359,8 +358,9 @@ __device__ __forceinline__ int fix_decide(const PiArgs &a, int lane, long long v
     // mean of the next sweep, predicted: 2^e (mean - M); a few units
     const float m = (float)A * inv_n - (float)c.M;
     const long long Mn = (long long)__float2int_rn(c.e ? ldexpf(m, c.e) : m);
-    // |X_s| < 2^b, so |X_{s+1}| < 2^(b + e_s): lift it to 2^56
-    const int en = min(24, max(0, 56 - (61 - __clz((int)mx) + c.e)));
+    // |X_s| < 2^b, so |X_{s+1}| < 2^(b + e_s) (an average, less a mean of a few
+    // units): lift it to 2^62
+    const int en = min(24, max(0, kFixTop - (64 - __clz((int)mx) + c.e)));
     c.K = omt2 * t;
     c.Z = t * (double)(c.e ? ldexpf(a.zero_tol2, 2 * c.e) : a.zero_tol2);
     next->M = Mn;
@@ -370,20 +370,18 @@ __device__ __forceinline__ int fix_decide(const PiArgs &a, int lane, long long v
     return code;
 }
 
-// State and first slots from the start vector's totals (read: value by lane group
-// as fix_decide wants it, A 2^-20 in the place of C's first value, and the maximum).
-template <typename READ>
-__device__ __forceinline__ void fix_ctl_start(const PiArgs &a, int lane, READ read, double omt2, int n, FixCtl &c,
+// State and first slots from the start vector's totals (value by lane group, as
+// fix_warp_vals leaves a start's).
+__device__ __forceinline__ void fix_ctl_start(const PiArgs &a, int lane, long long v, double omt2, int n, FixCtl &c,
                                               FixSlot *slots) {
-    unsigned m;
-    const long long v = read(&m);
     const int grp = lane >> 2;
     double d = __ll2double_rn(v);
-    if (grp == 1) d *= 0x1p-42;
-    if (grp == 2) d *= 0x1p-86;
-    const double A = fma(__shfl_sync(0xffffffffu, d, 16), 0x1p20, __shfl_sync(0xffffffffu, d, 0));
+    if (grp == 1) d *= 0x1p-44;
+    if (grp == 2) d *= 0x1p-87;
     const double B = __shfl_sync(0xffffffffu, d, 4) + __shfl_sync(0xffffffffu, d, 8);
-    const double mu0 = A * 0x1p-58 / (double)n;
+    const double A = fma(__shfl_sync(0xffffffffu, d, 16), 0x1p20, __shfl_sync(0xffffffffu, d, 0));
+    const long long lo = __shfl_sync(0xffffffffu, v, 0), hi = __shfl_sync(0xffffffffu, v, 16);
+    const double mu0 = A * 0x1p-64 / (double)n;
     double ss0 = B - (double)n * mu0 * mu0;
     if (ss0 < 0.0) ss0 = 0.0;
     c.B = c.Bp = ss0;
@@ -394,10 +392,12 @@ __device__ __forceinline__ void fix_ctl_start(const PiArgs &a, int lane, READ re
     c.M = 0;
     c.e = 0;
     if (lane == 0) {
-        slots[1].M = __double2ll_rn(A / (double)n);   // sweep 1: exact mean of y_0
+        // sweep 1: the mean of y_0 to a unit, from the integer sums
+        const long long m = hi / n;
+        slots[1].M = m * (1ll << 20) + ((hi - m * n) * (1ll << 20) + lo + n / 2) / n;
         slots[1].e = 0;
         slots[1].stop = 0;
-        slots[0].M = 0;                               // sweep 2: m_1 = 0
+        slots[0].M = 0;   // sweep 2: m_1 = 0
         slots[0].e = 0;
         slots[0].stop = 0;
     }
@@ -407,7 +407,7 @@ __device__ __forceinline__ void fix_ctl_start(const PiArgs &a, int lane, READ re
 // the ring slot of sweep rs.  res[0..1]: rs, annihilated.
 __device__ __forceinline__ void fix_finish(const PiArgs &a, int lane, int n, int rs, int code, bool counted, bool bad,
                                            bool writes, int buf, const FixCtl &c, int *res) {
-    const double to_mean = 0x1p-58 / (double)n;
+    const double to_mean = 0x1p-64 / (double)n;
     const double B = __shfl_sync(0xffffffffu, c.B, 4), Bp = __shfl_sync(0xffffffffu, c.Bp, 4);
     if (lane != 0) return;
     const bool zero = code == 2;
@@ -439,18 +439,63 @@ __device__ __forceinline__ void fix_finish(const PiArgs &a, int lane, int n, int
 }
 
 __device__ __forceinline__ double fix_value(int2 x) {
-    return fma((double)x.x, 0x1p29, (double)x.y) * 0x1p-58;
+    return fma((double)x.x, 0x1p32, (double)x.y) * 0x1p-64;
+}
+
+// The exponent k that scales a start vector of largest magnitude m (finite,
+// > 0) to |x| 2^k in [2^60, 2^61): the first sweep subtracts a mean of that size.
+__device__ __forceinline__ int fix_start_exponent(double m) {
+    int ex;
+    frexp(m, &ex);   // m = f 2^ex, f in [0.5, 1)
+    return kFixTop - 1 - ex;
+}
+
+// The start vector of a level held by one CTA or cluster, the same in every CTA:
+// values as doubles in ring slot 0, their largest magnitude, then fixed point; the
+// warps' sums to s_rec (fix_warp_record).  *s_bad: an entry is not finite (the
+// vector is then 0).  Every thread of the CTA calls it; ends with a CTA barrier.
+__device__ __forceinline__ void fix_start(const PiArgs &a, int2 *ring, double *s_mx, long long (*s_rec)[kFixSums],
+                                          int *s_bad) {
+    const int n = a.n, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const void *cb = nullptr;
+    double cmu = 0.0, cinv = 0.0;
+    if (a.start == 1) {
+        cb = a.cbuf[a.cres->buf];
+        cmu = a.cres->mu;
+        cinv = a.cres->inv_s;
+    }
+    if (tid == 0) *s_bad = 0;
+    __syncthreads();
+    double mx = 0.0;
+    int bad = 0;
+    for (int i = tid; i < n; i += blockDim.x) {
+        const double v = start_value(a, a.perm[i], cb, cmu, cinv);
+        reinterpret_cast<double *>(ring)[i] = v;
+        if (isfinite(v)) mx = fmax(mx, fabs(v));
+        else bad = 1;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) s_mx[warp] = mx;
+    if (bad) *s_bad = 1;
+    __syncthreads();
+    mx = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); w++) mx = fmax(mx, s_mx[w]);
+    const int k = mx > 0.0 ? fix_start_exponent(mx) : 0;
+    FixSum f;
+    f.reset();
+    for (int i = tid; i < n; i += blockDim.x) {
+        const double v = reinterpret_cast<double *>(ring)[i];
+        const long long X = *s_bad ? 0 : __double2ll_rn(ldexp(v, k));
+        const int2 x = fix_split(X);
+        f.add_start(X, x);
+        ring[i] = x;
+    }
+    fix_warp_record(f, true, lane, s_rec[warp]);
+    __syncthreads();
 }
 
 // The reciprocal fix_weight takes: false when g is not a positive finite number.
 bool fix_reciprocal(double g, unsigned long long *ginv, int *ge);
-
-// The exponent k that scales a start vector of largest magnitude m (finite,
-// > 0) to |x| 2^k in (2^55, 2^56].
-__device__ __forceinline__ int fix_start_exponent(double m) {
-    int ex;
-    frexp(m, &ex);   // m = f 2^ex, f in [0.5, 1)
-    return 56 - ex;
-}
 
 }  // namespace cmg

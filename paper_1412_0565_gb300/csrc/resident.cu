@@ -9,11 +9,11 @@
 namespace cmg {
 
 // ------------------------------------------------------------------ plan
-// Lanes per row by row length (FP64 items): steps of at most S entries per
-// lane while the row fits a warp, S = 8 on levels with at most kWideEntries
-// entries per SM (a sweep there is a chain of latencies: a row of 16 entries on
-// one lane is two rounds of gathers, on two lanes one) and 16 above, where the
-// FP64 pipe is the bound and every split row costs extra adds.
+// Lanes per row by row length: steps of at most S entries per lane while the row
+// fits a warp, S = 8 on levels with at most kWideEntries entries per SM (a sweep
+// there is a chain of latencies: a row of 16 entries on one lane is two rounds of
+// gathers, on two lanes one) and 16 above, where the instructions are the bound
+// and every split row costs extra sums.
 constexpr int kWideEntries = 8192;
 constexpr int kItemCost = 256;     // per item, in entries: the rows' finish and stop sums
 // Work of one CTA at least, in entries (an item counts kItemCost): below it more
@@ -22,7 +22,7 @@ constexpr int kItemCost = 256;     // per item, in entries: the rows' finish and
 constexpr int kCtaWork = 2048;
 constexpr int kPlanThreads = 1024;
 constexpr int kStreamThreads = 384;   // two CTAs per SM with 85 registers a thread
-constexpr int kRowsMaxRow = 4096;  // longest row the FP64 items take (one warp each)
+constexpr int kRowsMaxRow = 4096;  // longest row the items take (one warp each)
 
 __device__ __forceinline__ int plan_deg(const int *rp, const uint32_t *perm, int p) {
     const int v = (int)perm[p];
@@ -171,9 +171,9 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_units(int n, const int *_
 
 // Entries and diagonal of one item in fixed point (one warp); short rows and
 // missing rows are padded with coefficient 0 and a valid column.
-template <typename PERM, typename INV, typename IDX>
+template <typename PERM, typename INV>
 __device__ __forceinline__ void fill_item(int4 it, int lane, const int *rp, const int *col, const double *w,
-                                          unsigned long long ginv, int ge, const PERM *perm, const INV *inv, IDX *ucol,
+                                          unsigned long long ginv, int ge, const PERM *perm, const INV *inv, uint16_t *ucol,
                                           int2 *uc, int2 *ud) {
     const int lg = it.w & 7, rows = it.w >> 3, r = lane >> lg, g = lane & ((1 << lg) - 1);
     const int p = it.x + (r < rows ? r : 0);
@@ -193,12 +193,12 @@ __device__ __forceinline__ void fill_item(int4 it, int lane, const int *rp, cons
             Cij = fix_weight(w[e0 + k], ginv, ge);
             cl = (int)inv[col[e0 + k]];
         }
-        ucol[d] = (IDX)cl;
-        uc[d] = fix_split(Cij);
+        ucol[d] = (uint16_t)cl;
+        uc[d] = fix_split_c(Cij);
         sum += Cij;
     }
     for (int o = (1 << lg) >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (r < rows && g == 0) ud[p] = fix_split(sum);
+    if (r < rows && g == 0) ud[p] = fix_split_c(sum);
 }
 
 // The plan of levels of at most kFixMaxN rows, one CTA per level and one launch for
@@ -294,10 +294,9 @@ __global__ void k_fill_small(const SmallJob *__restrict__ jobs) {
         fill_item(J.item[u], lane, J.rp, J.col, J.w, J.ginv, J.ge, J.perm, J.inv, J.ucol, J.uc, J.ud);
 }
 
-template <typename IDX>
 __global__ void k_fill_units(int ni, const int4 *__restrict__ item, const int *__restrict__ rp,
                              const int *__restrict__ col, const double *__restrict__ w, unsigned long long ginv, int ge,
-                             const uint32_t *__restrict__ perm, const int *__restrict__ inv, IDX *__restrict__ ucol,
+                             const uint32_t *__restrict__ perm, const int *__restrict__ inv, uint16_t *__restrict__ ucol,
                              int2 *__restrict__ uc, int2 *__restrict__ ud) {
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
@@ -312,7 +311,7 @@ constexpr int kFixRec = 8;   // 64-bit words of one sweep's sums: 5 values, max 
 // vector's largest magnitude.
 constexpr int kFixAccWords = 3 * kFixRec + 8;
 
-// Sweeps of a level over all SMs (cooperative, warp 0 the control warp, one grid
+// Sweeps of a level of up to kFixRowsMax rows over all SMs (cooperative, warp 0 the control warp, one grid
 // barrier per sweep, iterates in degree order, deferred decisions as in
 // k_power_sell).  A row warp takes items: 32 lanes on 32 / G rows, entry t of
 // lane l at offset 32 t + l.  The CTAs add their integer stop sums to one record
@@ -327,19 +326,17 @@ constexpr int kFixAccWords = 3 * kFixRec + 8;
 // whole iterate copied to shared memory at the top of a sweep) one trip.
 // Otherwise two CTAs per SM stream the items, each with its columns,
 // coefficients and own row in flight together, the next item's descriptor too.
-// us per sweep: slice kernel in FP64, this kernel in FP64, in fixed point:
-// 215 rows and 17K entries 14.0, 4.4, -; 1,542 rows and 103K entries 17.3, 6.3,
-// 4.2; 5,688 rows and 129K entries 16.0, 6.6, 4.6; 20K rows and 160K entries 16.0,
-// 5.0, 4.1; 100^3 grid levels 0 to 4: 40.4 / 23.6 / 14.7 / 9.4 / 8.3, 38.0 / 22.5 /
-// 11.3 / 6.9 / 4.8, and 23.1 / 19.8 / 9.6 / 5.4 / 3.4.
-template <typename IDX, bool RES, bool STAGE, bool STREAM>
+// us per sweep: slice kernel in FP64, this kernel in FP64, in fixed point: 1,542 rows
+// and 103K entries 17.3, 6.3, 4.0; 5,688 rows and 129K entries 16.0, 6.6, 4.4; 20K
+// rows and 160K entries 16.0, 5.0, 4.4; the 100^3 grid's 35K- and 10K-row levels
+// 9.4 / 8.3, 6.9 / 4.8, and 5.5 / 3.5.
+template <bool RES, bool STAGE>
 __global__ void __launch_bounds__(RES ? 1024 : kStreamThreads, RES ? 1 : 2) k_power_rows(PiArgs a, GridSync *gs) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ __align__(16) long long s_pw[32][6];   // the warps' sums
+    __shared__ __align__(16) long long s_pw[32][kFixSums];   // the warps' sums
     __shared__ FixSlot s_slot[2];
     __shared__ GridBar s_bar;
     __shared__ int s_res[2];       // sweeps of the result, annihilated
-    __shared__ double s_mx[32];
     const int n = a.n;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nw = (int)(blockDim.x >> 5);
@@ -353,14 +350,14 @@ __global__ void __launch_bounds__(RES ? 1024 : kStreamThreads, RES ? 1 : 2) k_po
     int2 *s_w = reinterpret_cast<int2 *>(s_item + a.res_items);
     int2 *s_x = s_w + a.res_entries;
     int2 *s_d = s_x + (STAGE ? ((n + 1) & ~1) : 0);
-    IDX *s_c = reinterpret_cast<IDX *>(s_d + ((a.res_rows + 1) & ~1));
+    uint16_t *s_c = reinterpret_cast<uint16_t *>(s_d + ((a.res_rows + 1) & ~1));
     if (RES) {
         const int2 *gw = reinterpret_cast<const int2 *>(a.lay_w) + e_lo;
-        const IDX *gc = reinterpret_cast<const IDX *>(a.lay_col) + e_lo;
+        const uint16_t *gc = reinterpret_cast<const uint16_t *>(a.lay_col) + e_lo;
         const int ne = last.y - e_lo;   // a multiple of 32: 16-byte copies
         for (int k = tid; k < ne / 2; k += blockDim.x)
             reinterpret_cast<uint4 *>(s_w)[k] = __ldg(reinterpret_cast<const uint4 *>(gw) + k);
-        for (int k = tid; k < ne * (int)sizeof(IDX) / 16; k += blockDim.x)
+        for (int k = tid; k < ne / 8; k += blockDim.x)
             reinterpret_cast<uint4 *>(s_c)[k] = __ldg(reinterpret_cast<const uint4 *>(gc) + k);
         for (int k = tid; k < r1 - r0; k += blockDim.x) s_d[k] = __ldg(a.fix_d + r0 + k);
         for (int k = tid; k < ie - ib; k += blockDim.x) {
@@ -369,49 +366,19 @@ __global__ void __launch_bounds__(RES ? 1024 : kStreamThreads, RES ? 1 : 2) k_po
             s_item[k] = it;
         }
     }
-    const IDX *C = RES ? s_c : reinterpret_cast<const IDX *>(a.lay_col);
+    const uint16_t *C = RES ? s_c : reinterpret_cast<const uint16_t *>(a.lay_col);
     const int2 *W = RES ? s_w : reinterpret_cast<const int2 *>(a.lay_w);
     unsigned long long *const acc = reinterpret_cast<unsigned long long *>(a.fix_acc);
-    // the warps' sums of the row warps (first ... nw - 1), added to record k
+    // the records of the warps from `first_warp` on, added to record k
     auto publish = [&](int first_warp, int k) {
-        FixVals f;
-        unsigned m = 0;
-#pragma unroll
-        for (int j = 0; j < 5; j++) f.v[j] = 0;
-        if (lane >= first_warp && lane < nw) {
-            const longlong2 *src = reinterpret_cast<const longlong2 *>(s_pw[lane]);
-            const longlong2 u0 = src[0], u1 = src[1], u2 = src[2];
-            f.v[0] = u0.x;
-            f.v[1] = u0.y;
-            f.v[2] = u1.x;
-            f.v[3] = u1.y;
-            f.v[4] = u2.x;
-            m = (unsigned)u2.y;
-        }
-        m = __reduce_max_sync(0xffffffffu, m);
-        const long long v = fix_warp_vals(f, lane);
+        unsigned m;
+        const long long v = fix_sum_records(s_pw[first_warp], nw - first_warp, lane, &m);
         const int grp = lane >> 2;
         if ((lane & 3) == 0 && grp != 3 && grp != 7) {
             unsigned long long *dst = acc + kFixRec * k + (grp < 3 ? grp : grp - 1);
             if (grp == 6) atomicMax(dst, (unsigned long long)m);
             else atomicAdd(dst, (unsigned long long)v);
         }
-        __syncwarp();
-    };
-    // a warp's sums into its record; start: the start vector's, whose sum A is far
-    // from 0 (its total passes 64 bits) and travels in two parts, the high one in
-    // C's place
-    auto warp_sums = [&](const FixSum &f, bool start) {
-        const unsigned m = __reduce_max_sync(0xffffffffu, f.mx);
-        FixVals fv = fix_vals(f);
-        if (start) {
-            fv.v[3] = f.A >> 20;
-            fv.v[0] = f.A & 0xfffff;
-        }
-        long long v = fix_warp_vals(fv, lane);
-        const int grp = lane >> 2;
-        if (grp == 6) v = (long long)m;
-        if ((lane & 3) == 0 && grp != 3 && grp != 7) s_pw[warp][grp < 3 ? grp : grp - 1] = v;
         __syncwarp();
     };
     // record k as fix_decide wants it: value by lane group, and max |q|
@@ -456,10 +423,10 @@ __global__ void __launch_bounds__(RES ? 1024 : kStreamThreads, RES ? 1 : 2) k_po
             const double v = reinterpret_cast<double *>(ring0)[p];
             const long long X = bad ? 0 : __double2ll_rn(ldexp(v, k));
             const int2 x = fix_split(X);
-            f.add(X, x, x);
+            f.add_start(X, x);
             ring0[p] = x;
         }
-        warp_sums(f, true);
+        fix_warp_record(f, true, lane, s_pw[warp]);
         __syncthreads();
         if (warp == 0) publish(0, 0);
     }
@@ -470,7 +437,9 @@ __global__ void __launch_bounds__(RES ? 1024 : kStreamThreads, RES ? 1 : 2) k_po
         const double omt = 1.0 - a.tol, omt2 = omt * omt;
         const float inv_n = 1.0f / (float)n;
         FixCtl c;
-        fix_ctl_start(a, lane, [&](unsigned *m) { return read_acc(0, m); }, omt2, n, c, s_slot);
+        unsigned m0;
+        const long long v0 = read_acc(0, &m0);
+        fix_ctl_start(a, lane, v0, omt2, n, c, s_slot);
         __syncthreads();
         int s = 0, rs = 0, code = 0, k0 = 0;   // k0 = s modulo 3
         bool counted = false;
@@ -561,8 +530,8 @@ __global__ void __launch_bounds__(RES ? 1024 : kStreamThreads, RES ? 1 : 2) k_po
                             ww[u] = make_int2(0, 0);
                             if (t0 + u < it.z) {
                                 const int e = base + 32 * (t0 + u);
-                                cc[u] = (int)(STREAM ? __ldcs(C + e) : C[e]);
-                                ww[u] = STREAM ? __ldcs(W + e) : W[e];
+                                cc[u] = (int)C[e];
+                                ww[u] = W[e];
                             }
                         }
 #pragma unroll
@@ -578,14 +547,14 @@ __global__ void __launch_bounds__(RES ? 1024 : kStreamThreads, RES ? 1 : 2) k_po
                 }
                 const long long pr = t.lanes(lg);
                 if (leads) {
-                    const long long Y = fix_row(xi, pr, sl.M, sl.e);
+                    const long long X = fix_join(xi), Y = fix_row(X, pr, sl.M, sl.e);
                     const int2 yv = fix_split(Y);
                     y[i] = yv;
-                    f.add(Y, yv, xi);
+                    f.add(Y, yv, FixSum::narrow(Y), FixSum::narrow(X));
                 }
             }
             __syncwarp();
-            warp_sums(f, false);
+            fix_warp_record(f, false, lane, s_pw[warp]);
             __syncthreads();   // the warps' sums are complete
             __syncthreads();   // the grid barrier has passed
             if (!s_bar.ok) return;
@@ -605,17 +574,9 @@ __global__ void __launch_bounds__(RES ? 1024 : kStreamThreads, RES ? 1 : 2) k_po
     }
 }
 
-template <typename IDX>
-static const void *rows_kernel_t(const RowPlan &R) {
-    if (R.resident)
-        return R.stage ? (const void *)k_power_rows<IDX, true, true, false>
-                       : (const void *)k_power_rows<IDX, true, false, false>;
-    return R.stream ? (const void *)k_power_rows<IDX, false, false, true>
-                    : (const void *)k_power_rows<IDX, false, false, false>;
-}
-
 static const void *rows_kernel(const RowPlan &R) {
-    return R.col16 ? rows_kernel_t<uint16_t>(R) : rows_kernel_t<int>(R);
+    if (!R.resident) return (const void *)k_power_rows<false, false>;
+    return R.stage ? (const void *)k_power_rows<true, true> : (const void *)k_power_rows<true, false>;
 }
 
 cmg_status_t launch_fill_small(const SmallJob *jobs_dev, int count, cudaStream_t s) {
@@ -628,9 +589,8 @@ cmg_status_t launch_plan_small(const SmallJob *jobs_dev, int count, cudaStream_t
     return launch_status();
 }
 
-static size_t rows_smem(int n, int col16, int stage, const PlanOut &o) {
-    const size_t isz = col16 ? 2 : 4;
-    return 16 * (size_t)o.max_i + (8 + isz) * (size_t)o.max_e + (stage ? 8 * (size_t)((n + 1) & ~1) : 0) +
+static size_t rows_smem(int n, int stage, const PlanOut &o) {
+    return 16 * (size_t)o.max_i + 10 * (size_t)o.max_e + (stage ? 8 * (size_t)((n + 1) & ~1) : 0) +
            8 * (size_t)((o.max_r + 1) & ~1) + 16;
 }
 
@@ -652,17 +612,23 @@ static cmg_status_t rows_choose(int n, const PlanOut &o, RowPlan *R) {
     size_t room = 0;
     CMG_TRY(rows_room(*R, &room));
     R->resident = R->stage = 0;
-    if (rows_smem(n, R->col16, 0, o) > room) return CMG_OK;
+    if (rows_smem(n, 0, o) > room) return CMG_OK;
     R->resident = 1;
     // staging the iterate costs one trip to L2 and n / 8 cycles of copying per
     // SM; a scattered gather costs about 1.4 cycles more from L1 or L2 than from
     // shared memory
-    if (rows_smem(n, R->col16, 1, o) <= room && (long long)n / 8 + 800 < (long long)o.max_e) R->stage = 1;
+    if (rows_smem(n, 1, o) <= room && (long long)n / 8 + 800 < (long long)o.max_e) R->stage = 1;
     R->res_e = o.max_e;
     R->res_i = o.max_i;
     R->res_r = o.max_r;
-    R->smem = rows_smem(n, R->col16, R->stage, o);
+    R->smem = rows_smem(n, R->stage, o);
     return CMG_OK;
+}
+
+bool rows_may_hold(int n, long long nnz) {
+    DeviceInfo d;
+    if (device_info(&d) != CMG_OK) return false;
+    return n <= kFixRowsMax && (d.l2_bytes <= 0 || 10 * nnz <= (long long)d.l2_bytes);
 }
 
 cmg_status_t build_row_plan(int n, long long nnz, const int *rp, const int *col, const double *w, double g,
@@ -672,7 +638,6 @@ cmg_status_t build_row_plan(int n, long long nnz, const int *rp, const int *col,
     if (!fix_reciprocal(g, &ginv, &ge)) return CMG_ERR_TOO_LARGE;
     DeviceInfo di;
     CMG_TRY(device_info(&di));
-    R->col16 = n <= 65536 ? 1 : 0;
     Scratch scr(s);
     PlanOut *out_dev, o;
     CMG_TRY(scr.get(&out_dev, 1));
@@ -696,8 +661,6 @@ cmg_status_t build_row_plan(int n, long long nnz, const int *rp, const int *col,
     R->threads = std::max(R->stage ? 512 : 64, 32 * (1 + std::min(31, std::max(1, o.max_i))));
     if (!R->resident) {
         CMG_TRY(plan(2 * di.sms, 0));
-        const long long lay = o.entries * (long long)(R->col16 ? 2 + 8 : 4 + 8);
-        R->stream = di.l2_bytes > 0 && lay > (long long)di.l2_bytes;
         R->threads = kStreamThreads;
     }
     // a lane adds at most this many rows' sums
@@ -708,18 +671,14 @@ cmg_status_t build_row_plan(int n, long long nnz, const int *rp, const int *col,
     CMG_TRY(dev_alloc_n(&R->item, (size_t)o.ni + 1, s));
     CMG_CUDA(cudaMemcpyAsync(R->item, item, sizeof(int4) * ((size_t)o.ni + 1), cudaMemcpyDeviceToDevice, s));
     const size_t ne = (size_t)std::max<long long>(o.entries, 1);
-    CMG_TRY(dev_alloc(&R->ucol, ne * (R->col16 ? 2 : 4), s));
+    CMG_TRY(dev_alloc_n(&R->ucol, ne, s));
     CMG_TRY(dev_alloc_n(&R->uc, ne, s));
     CMG_TRY(dev_alloc_n(&R->ud, (size_t)n, s));
     CMG_TRY(dev_alloc_n(&R->acc, (size_t)kFixAccWords, s));
     const int fb = grid_for(32ll * o.ni, 256);
-    if (R->col16)
-        k_fill_units<<<fb, 256, 0, s>>>(o.ni, R->item, rp, col, w, ginv, ge, L.perm, L.inv, (uint16_t *)R->ucol, R->uc,
-                                        R->ud);
-    else
-        k_fill_units<<<fb, 256, 0, s>>>(o.ni, R->item, rp, col, w, ginv, ge, L.perm, L.inv, (int *)R->ucol, R->uc, R->ud);
+    k_fill_units<<<fb, 256, 0, s>>>(o.ni, R->item, rp, col, w, ginv, ge, L.perm, L.inv, R->ucol, R->uc, R->ud);
     CMG_TRY(launch_status());
-    *bytes += 16 * ((size_t)o.ni + 1) + 4 * ((size_t)2 * di.sms + 1) + ne * (size_t)((R->col16 ? 2 : 4) + 8) +
+    *bytes += 16 * ((size_t)o.ni + 1) + 4 * ((size_t)2 * di.sms + 1) + 10 * ne +
               8 * (size_t)n + 8 * kFixAccWords;
     return CMG_OK;
 }
