@@ -254,6 +254,16 @@ cmg_status_t cmg_hierarchy_info(cmg_hierarchy_t h, int32_t *levels, int64_t *n_p
  * Errors: INVALID_ARG if h is NULL. */
 cmg_status_t cmg_level_kernels(cmg_hierarchy_t h, int32_t *kind_out, int32_t *staged_out);
 
+/* The form of the sweep kernel that runs on each level, for tests and measurements
+ * (host arrays of length >= levels, nullable).  form_out[j]: fixed point: 0 = the
+ * shared memory of one CTA or cluster with the entries in registers, 1 = the same
+ * with the entries in shared memory, row kernel 2 = streamed, 3 = resident,
+ * 4 = resident with the iterate staged every sweep; floating point: 5 = one CTA,
+ * slice kernel 6 = unstaged, 7 = staged, 8 = staged with the layout resident,
+ * 9 = two-phase, 10 = row tiles.  ctas_out[j]: CTAs of forms 0 to 4, else 0.
+ * Errors: INVALID_ARG if h is NULL. */
+cmg_status_t cmg_level_forms(cmg_hierarchy_t h, int32_t *form_out, int32_t *ctas_out);
+
 /* Sweep precision of each level (host int32 array of length >= levels):
  * CMG_PRECISION_FP32_SWEEP or CMG_PRECISION_FP64 (see the precision enum).
  * Errors: INVALID_ARG if h or prec_out is NULL. */

@@ -33,7 +33,7 @@ STATUS = {
 # every symbol include/cmg.h declares
 EXPORTS = [
     "cmg_options_default", "cmg_status_string", "cmg_version", "cmg_setup", "cmg_fiedler",
-    "cmg_hierarchy_info", "cmg_level_kernels", "cmg_level_precision", "cmg_hierarchy_device_bytes", "cmg_estimate_device_bytes",
+    "cmg_hierarchy_info", "cmg_level_kernels", "cmg_level_forms", "cmg_level_precision", "cmg_hierarchy_device_bytes", "cmg_estimate_device_bytes",
     "cmg_get_aggregates", "cmg_get_level_csr", "cmg_free", "cmg_heaviest_neighbour",
     "cmg_visit_ranks", "cmg_hec_aggregate", "cmg_power_sweeps", "cmg_rayleigh_residual",
     "cmg_power_sweeps_noalloc", "cmg_kernel_launches", "cmg_debug_fail_alloc_after", "cmg_debug_stall_barrier",
@@ -150,6 +150,7 @@ def load(build_if_stale: bool = True):
             "cmg_fiedler": (I32, [V, V, I32, P(F64), P(Stats), V]),
             "cmg_hierarchy_info": (I32, [V, P(I32), V, V]),
             "cmg_level_kernels": (I32, [V, V, V]),
+            "cmg_level_forms": (I32, [V, V, V]),
             "cmg_hierarchy_device_bytes": (I32, [V, P(C.c_size_t)]),
             "cmg_estimate_device_bytes": (I32, [I64, I64, I32, P(C.c_size_t)]),
             "cmg_get_aggregates": (I32, [V, I32, V]),
@@ -334,6 +335,18 @@ class Hierarchy:
         _check(load().cmg_level_kernels(self._h, C.c_void_p(kind.ctypes.data),
                                         C.c_void_p(staged.ctypes.data)), "level_kernels")
         return kind.tolist(), staged.tolist()
+
+    FORMS = ("fix_registers", "fix_shared", "rows_streamed", "rows_resident", "rows_staged", "one_cta", "slice",
+             "slice_staged", "slice_resident", "two_phase", "tiles")
+
+    def level_forms(self):
+        """Per level: the name (FORMS) of the sweep kernel's form, and its CTAs
+        (fixed-point forms; else 0)."""
+        form = np.zeros(self.levels, dtype=np.int32)
+        ctas = np.zeros(self.levels, dtype=np.int32)
+        _check(load().cmg_level_forms(self._h, C.c_void_p(form.ctypes.data), C.c_void_p(ctas.ctypes.data)),
+               "level_forms")
+        return [self.FORMS[f] for f in form], ctas.tolist()
 
     def eigenpairs(self, k: int, *, seed=None, U_out=None, stream=None):
         """cmg_eigenpairs: k approximate eigenpairs by the cascade with block

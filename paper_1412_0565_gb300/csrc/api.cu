@@ -844,6 +844,31 @@ cmg_status_t cmg_level_kernels(cmg_hierarchy_t h, int32_t *kind_out, int32_t *st
     return CMG_OK;
 }
 
+cmg_status_t cmg_level_forms(cmg_hierarchy_t h, int32_t *form_out, int32_t *ctas_out) {
+    if (!h) return CMG_ERR_INVALID_ARG;
+    // in the order in which power_iteration() chooses
+    for (size_t j = 0; j < h->lv.size(); j++) {
+        const LevelData &L = h->lv[j];
+        int form = 10, ctas = 0;
+        if (L.has_fix) {
+            form = L.fix.by_warp ? 0 : 1;
+            ctas = L.fix.C;
+        } else if (small_level_fits(level_view(L), L.fp32)) {
+            form = 5;
+        } else if (L.has_rows) {
+            form = !L.rows.resident ? 2 : (L.rows.stage ? 4 : 3);
+            ctas = L.rows.P;
+        } else if (L.has_xl) {
+            form = 9;
+        } else if (L.has_lay) {
+            form = L.lay.stage_n <= 0 ? 6 : (L.fp32 && L.lay.res_e > 0 ? 8 : 7);
+        }
+        if (form_out) form_out[j] = form;
+        if (ctas_out) ctas_out[j] = ctas;
+    }
+    return CMG_OK;
+}
+
 cmg_status_t cmg_level_precision(cmg_hierarchy_t h, int32_t *prec_out) {
     if (!h || !prec_out) return CMG_ERR_INVALID_ARG;
     for (size_t j = 0; j < h->lv.size(); j++)
