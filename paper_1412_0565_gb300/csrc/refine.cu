@@ -1214,12 +1214,10 @@ static const void *sell_kernel(int fp32, int col16, bool chunks, bool stream, bo
                  : sell_kernel_ti<double, int>(chunks, stream, stage);
 }
 
-static const void *sell_res_kernel(int col16, bool chunks) {
-    if (col16)
-        return chunks ? (const void *)k_power_sell<float, uint16_t, true, false, true, true>
-                      : (const void *)k_power_sell<float, uint16_t, false, false, true, true>;
-    return chunks ? (const void *)k_power_sell<float, int, true, false, true, true>
-                  : (const void *)k_power_sell<float, int, false, false, true, true>;
+// (a level that stages its whole iterate has 16-bit columns)
+static const void *sell_res_kernel(bool chunks) {
+    return chunks ? (const void *)k_power_sell<float, uint16_t, true, false, true, true>
+                  : (const void *)k_power_sell<float, uint16_t, false, false, true, true>;
 }
 
 // Launch of the slice kernel over a level's layout: CTAs and threads (the
@@ -1295,10 +1293,10 @@ cmg_status_t sell_choose_resident(SweepLayout *L, int n, int max_entries, int ma
     size_t smem;
     bool stream;
     CMG_TRY(sell_geometry(*L, n, 1, &blocks, &threads, &kern, &smem, &stream));
-    if (L->stage_n < n) return CMG_OK;
-    const size_t need = 4 * (size_t)((n + 7) & ~7) + (size_t)max_entries * (4 + (L->col16 ? 2 : 4)) +
+    if (L->stage_n < n || !L->col16) return CMG_OK;
+    const size_t need = 4 * (size_t)((n + 7) & ~7) + (size_t)max_entries * (4 + 2) +
                         4 * ((size_t)max_chunks + 2) + 16;
-    const void *k = sell_res_kernel(L->col16, L->hheavy[0] > 0);
+    const void *k = sell_res_kernel(L->hheavy[0] > 0);
     DeviceInfo di;
     CMG_TRY(device_info(&di));
     cudaFuncAttributes fa;
@@ -1487,7 +1485,7 @@ cmg_status_t power_iteration(const PiRun &run, GridSync *gs, cudaStream_t s, con
         bool stream;
         CMG_TRY(sell_geometry(L, lv.n, run.fp32, &blocks, &threads, &kern, &smem, &stream));
         if (run.fp32 && L.res_e > 0) {
-            kern = sell_res_kernel(L.col16, a.lay_h > 0);
+            kern = sell_res_kernel(a.lay_h > 0);
             CMG_TRY(allow_max_dynamic_smem(kern));
             smem = L.res_smem;
             a.res_entries = L.res_e;
