@@ -92,15 +92,6 @@ static cmg_status_t launch_check(int n, double avg, const int *rp, const int *co
     }
 }
 
-// Without input checks: whether every weight is finite and positive, which the
-// fixed-point sweeps rely on.
-__global__ void k_check_weights(long long m, const double *__restrict__ w, unsigned *__restrict__ flags) {
-    unsigned f = 0;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < m; k += (long long)gridDim.x * blockDim.x)
-        if (!(w[k] > 0.0) || isinf(w[k])) f = kBadWeight;
-    if (f) atomicOr(flags, f);
-}
-
 __global__ void k_to_float(long long m, const double *__restrict__ w, float *__restrict__ w32) {
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < m;
          k += (long long)gridDim.x * blockDim.x)
@@ -201,7 +192,7 @@ static cmg_status_t map_flags(unsigned f) {
 
 cmg_status_t cmg::load_level0(int64_t n, const int64_t *row_ptr, const int32_t *col, const double *w,
                               int32_t mem, int validate, int **rp_out, int **col_out,
-                              double **w_out, long long *nnz_out, cudaStream_t s) {
+                              double **w_out, long long *nnz_out, cudaStream_t s, bool *in_contract) {
     // ---- nnz and size limits
     int64_t nnz = 0;
     if (mem == CMG_MEM_HOST) {
@@ -246,6 +237,14 @@ cmg_status_t cmg::load_level0(int64_t n, const int64_t *row_ptr, const int32_t *
         CMG_CUDA(cudaMemcpyAsync(&hf, flags, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
         CMG_CUDA(cudaStreamSynchronize(s));
         CMG_TRY(map_flags(hf));
+        if (in_contract) *in_contract = true;
+    } else if (in_contract) {
+        // the check reads nothing outside the arrays, whatever they hold
+        unsigned hf = 0;
+        CMG_TRY(launch_check((int)n, (double)nnz / (double)n, *rp_out, *col_out, *w_out, flags, s));
+        CMG_CUDA(cudaMemcpyAsync(&hf, flags, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+        CMG_CUDA(cudaStreamSynchronize(s));
+        *in_contract = hf == 0;
     }
     return CMG_OK;
 }
@@ -308,25 +307,18 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
     L0.n = (int)n;
     h->lv.push_back(L0);
     LevelData &Z = h->lv.back();
-    CMG_TRY(load_level0(n, row_ptr, col, w, mem, o.validate, &Z.rp, &Z.col, &Z.w, &Z.nnz, s));
+    // the fixed-point sweeps rely on the input contract (positive finite weights, the
+    // same in both directions: the mean they subtract and their sums assume that a
+    // sweep keeps the mean): an unchecked graph outside it keeps the FP64 sweeps
+    bool fixed_ok = true;
+    CMG_TRY(load_level0(n, row_ptr, col, w, mem, o.validate, &Z.rp, &Z.col, &Z.w, &Z.nnz, s, &fixed_ok));
     Scratch scr(s);
-    bool fixed_ok = true;   // weights the fixed-point sweeps take
     {
         double *gd;
         CMG_TRY(scr.get(&gd, 1));
         CMG_TRY(launch_gershgorin((int)n, Z.rp, Z.w, gd, s));
         CMG_CUDA(cudaMemcpyAsync(&Z.g, gd, sizeof(double), cudaMemcpyDeviceToHost, s));
-        unsigned hf = 0;
-        if (!o.validate && Z.nnz > 0) {
-            unsigned *flags;
-            CMG_TRY(scr.get(&flags, 1));
-            CMG_CUDA(cudaMemsetAsync(flags, 0, sizeof(unsigned), s));
-            k_check_weights<<<grid_for(Z.nnz, 256), 256, 0, s>>>(Z.nnz, Z.w, flags);
-            CMG_TRY(launch_status());
-            CMG_CUDA(cudaMemcpyAsync(&hf, flags, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-        }
         CMG_CUDA(cudaStreamSynchronize(s));
-        fixed_ok = hf == 0;
     }
     // ---- Alg. 1 Step 1: coarsen while n_i > coarse_size.  Each level runs
     // HEC, the Galerkin product and the SELL-32 sizing on the device into

@@ -44,10 +44,11 @@ cmg_status_t check_options(const cmg_options_t &o);
 // Level 0 of a hierarchy: copies the CSR (host or device, int64 row pointers)
 // into new device arrays (int32 row pointers) and, with `validate`, checks
 // the input contract of cmg_setup.  The arrays belong to the caller as soon
-// as they are allocated, also when an error is returned.
+// as they are allocated, also when an error is returned.  in_contract (nullable):
+// whether the input keeps the contract, also found out without `validate`.
 cmg_status_t load_level0(int64_t n, const int64_t *row_ptr, const int32_t *col, const double *w,
                          int32_t mem, int validate, int **rp_out, int **col_out, double **w_out,
-                         long long *nnz_out, cudaStream_t s);
+                         long long *nnz_out, cudaStream_t s, bool *in_contract = nullptr);
 // w32[k] = (float)w[k].
 cmg_status_t launch_to_float(long long m, const double *w, float *w32, cudaStream_t s);
 
