@@ -230,9 +230,10 @@ cmg_status_t cmg_hierarchy_info(cmg_hierarchy_t h, int32_t *levels, int64_t *n_p
 
 /* Sweep kernel that runs Alg. 3 on each level (host arrays of length >= levels,
  * nullable).  kind_out[j]: 0 = the level in the shared memory (and registers) of
- * one CTA, or of a small thread-block cluster for a level below 512 rows,
- * 1 = all SMs over the level's items or sweep layout, streamed or held in the
- * SMs' shared memory, 2 = the FP32 slice kernel (FP64 with CMG_STAGE=1) with the
+ * one CTA, or, where CMG_CLUSTER is not set, of a small thread-block cluster for a
+ * level below 512 rows,
+ * 1 = all SMs over the level's items (FP64 levels of up to 65,536 rows) or sweep
+ * layout, streamed or held in the SMs' shared memory, 2 = the slice kernel with the
  * iterate's first staged_out[j] entries (its highest-degree rows) copied to
  * shared memory every sweep, 3 = row-tile kernel, 4 = two-phase kernel (a
  * sweep in passes: the columns' values are first copied, block by block
@@ -240,15 +241,19 @@ cmg_status_t cmg_hierarchy_info(cmg_hierarchy_t h, int32_t *levels, int64_t *n_p
  * then every row sums a contiguous stream in 64-bit fixed point; taken only
  * when the environment variable CMG_2P=1 is set at cmg_setup, for every
  * level beyond the shared-memory kernels), 5 = cluster kernel (FP64 sweeps of a
- * level of 512 to a few thousand rows spread over one thread-block cluster of
+ * level of up to a few thousand rows spread over one thread-block cluster of
  * 2 to 8 CTAs: every CTA holds the iterate, computes its share of the rows and
- * stores them into the others' shared memory; CMG_CLUSTER=0 keeps such levels
- * off clusters, CMG_CLUSTER=<rows> moves the 512).  FP64 sweeps of kinds 0, 1 and
- * 5 run in 60-bit fixed point, whose rounding is below FP64's.  Staging is
- * chosen at setup where the gathers
+ * stores them into the others' shared memory).  CMG_CLUSTER, read by cmg_setup:
+ * 0 keeps every level off clusters, <rows> (at least 128) the levels of fewer rows.
+ * cmg_level_forms tells the kernels' forms apart.
+ * FP64 levels of up to 65,536 rows sweep in 62-bit fixed point (a graph that is not
+ * checked, validate = 0, only if it keeps the input contract): its noise over the
+ * whole vector is below one FP64 rounding of the largest entry.  Larger FP64 levels,
+ * levels with a row of more than 4,096 entries and levels whose layout is larger
+ * than L2 sweep in FP64.  Staging is chosen at setup where the gathers
  * it serves are several per staged entry and SM; CMG_STAGE=0 (never) or
  * CMG_STAGE=1 (every slice level), read by cmg_setup, overrides that rule and
- * keeps FP64 levels on the slice kernel.
+ * keeps FP64 levels beyond the shared-memory kernels on the slice kernel.
  * Results do not depend on the kernel beyond rounding; every kernel sums in
  * a fixed order (or exactly), so repeated solves are bit-identical.
  * Errors: INVALID_ARG if h is NULL. */

@@ -404,10 +404,11 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
     }
     // ---- FP64 levels of up to a few thousand rows: fixed-point sweeps in the
     // shared memory of one CTA or one thread-block cluster (CMG_CLUSTER=0: one
-    // CTA only; CMG_CLUSTER=<rows>: what cmg_level_kernels calls a cluster level)
+    // CTA only; CMG_CLUSTER=<rows>: levels of fewer rows keep to one CTA)
     size_t lay_bytes = 0;
     const char *cl_env = getenv("CMG_CLUSTER");
-    h->cluster_min = cl_env ? std::max(128, atoi(cl_env)) : 512;
+    const int cl_min = !cl_env ? 0 : (cl_env[0] == '0' ? 0x7fffffff : std::max(128, atoi(cl_env)));
+    h->cluster_min = cl_env ? cl_min : 512;
     {
         std::vector<FixLevel> small;
         std::vector<int> who;
@@ -421,7 +422,7 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
             f.col = L.col;
             f.w = L.w;
             f.g = L.g;
-            f.max_ctas = cl_env && cl_env[0] == '0' ? 1 : 8;
+            f.max_ctas = L.n < cl_min ? 1 : 8;
             small.push_back(f);
             who.push_back(k);
         }

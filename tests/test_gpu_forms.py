@@ -96,3 +96,25 @@ def test_resident_fp32_layout_gives_the_streamed_bits(monkeypatch, name):
             assert h.level_forms()[0] == [form]
             got[mode] = h.fiedler(x0=x0)
     assert np.array_equal(got["0"][0], got["1"][0]) and got["0"][1] == got["1"][1]
+
+
+@pytest.mark.parametrize("switch", ["0", "128", "1000", "2000", "9000"])
+def test_cluster_switch_keeps_smaller_levels_on_one_cta(monkeypatch, switch):
+    """CMG_CLUSTER=<rows>: no level of fewer rows takes a cluster, whatever the plan
+    would have given it; larger levels take the plan's."""
+    rp, col, w = inputs.grid2d(64, 64, "uniform", seed=3)
+    with cmg.Hierarchy(rp, col, w, seed=1412) as h:
+        free = h.level_forms()[1]
+        u0 = h.fiedler()[0]
+    monkeypatch.setenv("CMG_CLUSTER", switch)
+    with cmg.Hierarchy(rp, col, w, seed=1412) as h:
+        forms, ctas = h.level_forms()
+        kinds, n = h.level_kernels()[0], h.sizes()[0]
+        u = h.fiedler()[0]
+    least = int(switch) if int(switch) else 1 << 30
+    assert any(c > 1 and rows < 512 for c, rows in zip(free, n))
+    for f, c, k, rows, plan in zip(forms, ctas, kinds, n, free):
+        if f.startswith("fix"):
+            assert c == (plan if rows >= least else 1)
+            assert k == (5 if c > 1 else 0)
+    assert np.linalg.norm(u - u0) <= 1e-10
