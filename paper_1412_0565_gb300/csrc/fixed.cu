@@ -437,7 +437,7 @@ static size_t fix_smem(int n, int threads, int res_i, int res_e, int res_r) {
 
 cmg_status_t build_fix_plans(std::vector<FixLevel> &lv, cudaStream_t s) {
     Scratch scr(s);
-    std::vector<SmallJob> jobs;
+    SmallJobs jobs = {};
     std::vector<int> who;
     DeviceInfo di;
     CMG_TRY(device_info(&di));
@@ -447,7 +447,7 @@ cmg_status_t build_fix_plans(std::vector<FixLevel> &lv, cudaStream_t s) {
     for (size_t q = 0; q < lv.size(); q++) {
         FixLevel &L = lv[q];
         L.ok = 0;
-        if (!fix_may_hold(L.n, L.nnz)) continue;
+        if (!fix_may_hold(L.n, L.nnz) || who.size() == kSmallJobs) continue;
         const long long work = L.nnz + 8ll * L.n;
         SmallJob J = {};
         J.n = L.n;
@@ -479,21 +479,19 @@ cmg_status_t build_fix_plans(std::vector<FixLevel> &lv, cudaStream_t s) {
         J.perm = F.perm = (int *)(base + o2);
         CMG_TRY(scr.get(&J.inv, (size_t)L.n));
         F.bytes = o3;
-        jobs.push_back(J);
+        jobs.j[who.size()] = J;
         who.push_back((int)q);
     }
-    if (jobs.empty()) return CMG_OK;
-    SmallJob *jobs_dev;
+    const int count = (int)who.size();
+    if (count == 0) return CMG_OK;
     PlanOut *out_dev;
-    CMG_TRY(scr.get(&jobs_dev, jobs.size()));
-    CMG_TRY(scr.get(&out_dev, jobs.size()));
-    for (size_t k = 0; k < jobs.size(); k++) jobs[k].out = out_dev + k;
-    std::vector<PlanOut> out(jobs.size());
-    CMG_CUDA(cudaMemcpyAsync(jobs_dev, jobs.data(), sizeof(SmallJob) * jobs.size(), cudaMemcpyHostToDevice, s));
-    CMG_TRY(launch_plan_small(jobs_dev, (int)jobs.size(), s));
-    CMG_CUDA(cudaMemcpyAsync(out.data(), out_dev, sizeof(PlanOut) * jobs.size(), cudaMemcpyDeviceToHost, s));
+    CMG_TRY(scr.get(&out_dev, (size_t)count));
+    for (int k = 0; k < count; k++) jobs.j[k].out = out_dev + k;
+    std::vector<PlanOut> out(count);
+    CMG_TRY(launch_plan_small(jobs, count, s));
+    CMG_CUDA(cudaMemcpyAsync(out.data(), out_dev, sizeof(PlanOut) * (size_t)count, cudaMemcpyDeviceToHost, s));
     CMG_CUDA(cudaStreamSynchronize(s));
-    for (size_t k = 0; k < jobs.size(); k++) {
+    for (int k = 0; k < count; k++) {
         FixLevel &L = lv[who[k]];
         FixPlan &F = L.plan;
         F.res_e = out[k].max_e;
@@ -543,16 +541,15 @@ cmg_status_t build_fix_plans(std::vector<FixLevel> &lv, cudaStream_t s) {
         // exact entries, filled below
         const size_t ne = (size_t)std::max<long long>(out[k].entries, 1), o1 = 8 * ne, o2 = o1 + 8 * (size_t)L.n;
         CMG_TRY(dev_alloc(&F.entries, o2 + 2 * ne, s));
-        jobs[k].uc = F.uc = (int2 *)F.entries;
-        jobs[k].ud = F.ud = (int2 *)((char *)F.entries + o1);
-        jobs[k].ucol = F.ucol = (uint16_t *)((char *)F.entries + o2);
-        jobs[k].ni = F.ni;
+        jobs.j[k].uc = F.uc = (int2 *)F.entries;
+        jobs.j[k].ud = F.ud = (int2 *)((char *)F.entries + o1);
+        jobs.j[k].ucol = F.ucol = (uint16_t *)((char *)F.entries + o2);
+        jobs.j[k].ni = F.ni;
         F.bytes += o2 + 2 * ne;
         L.ok = 1;
     }
     // (a level that does not fit keeps ni = 0 items to fill)
-    CMG_CUDA(cudaMemcpyAsync(jobs_dev, jobs.data(), sizeof(SmallJob) * jobs.size(), cudaMemcpyHostToDevice, s));
-    return launch_fill_small(jobs_dev, (int)jobs.size(), s);
+    return launch_fill_small(jobs, count, s);
 }
 
 void free_fix_plan(FixPlan &F, cudaStream_t s) {

@@ -71,8 +71,16 @@ struct SmallJob {
     int2 *uc, *ud;             // k_fill_small: ni items
     PlanOut *out;
 };
-cmg_status_t launch_plan_small(const SmallJob *jobs_dev, int count, cudaStream_t s);
-cmg_status_t launch_fill_small(const SmallJob *jobs_dev, int count, cudaStream_t s);
+// The levels of a hierarchy, by value: a launch holds its own copy, so the host's may
+// change or go.  (Coarsening at least halves the vertices that have an edge, so a
+// hierarchy has at most 13 such levels of up to kFixMaxN rows.)
+constexpr int kSmallJobs = 16;
+struct SmallJobs {
+    SmallJob j[kSmallJobs];
+};
+static_assert(sizeof(SmallJobs) <= 4000, "kernel parameters");
+cmg_status_t launch_plan_small(const SmallJobs &jobs, int count, cudaStream_t s);
+cmg_status_t launch_fill_small(const SmallJobs &jobs, int count, cudaStream_t s);
 
 // ------------------------------------------------------------------ arithmetic
 constexpr int kFixTop = 62;   // |X| < 2^62; y = X 2^-64

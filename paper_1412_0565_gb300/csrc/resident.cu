@@ -205,14 +205,14 @@ __device__ __forceinline__ void fill_item(int4 it, int lane, const int *rp, cons
 // all of them: degree order (a stable counting sort), items and ranges.  (The one-CTA and
 // cluster kernels sorted and laid out their level in the sweep launch itself,
 // and the cluster's plan read its row pointers back to the host.)
-__global__ void __launch_bounds__(kPlanThreads) k_plan_small(const SmallJob *__restrict__ jobs) {
+__global__ void __launch_bounds__(kPlanThreads) k_plan_small(const __grid_constant__ SmallJobs jobs) {
     __shared__ SmallJob J;
     __shared__ unsigned short s_perm[kFixMaxN], s_inv[kFixMaxN];
     __shared__ int s_hist[kFixMaxN + 1];
     __shared__ int s_md;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
-        J = jobs[blockIdx.x];
+        J = jobs.j[blockIdx.x];
         s_md = 0;
     }
     __syncthreads();
@@ -286,8 +286,8 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_small(const SmallJob *__r
 }
 
 // Entries and diagonal of the planned levels, a warp per item (blockIdx.y: level).
-__global__ void k_fill_small(const SmallJob *__restrict__ jobs) {
-    const SmallJob &J = jobs[blockIdx.y];
+__global__ void k_fill_small(const __grid_constant__ SmallJobs jobs) {
+    const SmallJob &J = jobs.j[blockIdx.y];
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
     for (int u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < J.ni; u += warps)
@@ -579,13 +579,13 @@ static const void *rows_kernel(const RowPlan &R) {
     return R.stage ? (const void *)k_power_rows<true, true> : (const void *)k_power_rows<true, false>;
 }
 
-cmg_status_t launch_fill_small(const SmallJob *jobs_dev, int count, cudaStream_t s) {
-    k_fill_small<<<dim3(64, count), 256, 0, s>>>(jobs_dev);
+cmg_status_t launch_fill_small(const SmallJobs &jobs, int count, cudaStream_t s) {
+    k_fill_small<<<dim3(64, count), 256, 0, s>>>(jobs);
     return launch_status();
 }
 
-cmg_status_t launch_plan_small(const SmallJob *jobs_dev, int count, cudaStream_t s) {
-    k_plan_small<<<count, kPlanThreads, 0, s>>>(jobs_dev);
+cmg_status_t launch_plan_small(const SmallJobs &jobs, int count, cudaStream_t s) {
+    k_plan_small<<<count, kPlanThreads, 0, s>>>(jobs);
     return launch_status();
 }
 
