@@ -10,7 +10,8 @@ headline is the FP64 form, the paper's arithmetic; the FP32-sweep form, the
 are reported under their own keys, each result's accuracy against the CPU
 oracle.
 
-Prints ONE JSON line (rank 0).  `--impl reference` times the CPU oracle (the
+Prints ONE JSON line (rank 0) of under 2,000 characters; the full record, every
+section with its notes, goes to --details FILE, or to stderr.  `--impl reference` times the CPU oracle (the
 plain sequential FP64 restatement of the method) on the same workload.
 With N > 1 ranks (torchrun), every rank solves its own replica of the
 workload (the method does not shard a single graph; replicas only).
@@ -533,10 +534,51 @@ def run_gpu(args):
             "gcmg": gcmg,
             "schedule_study": study,
         }
-        print(json.dumps(line), flush=True)
+        details = json.dumps(line)
+        if args.details:
+            with open(args.details, "w") as f:
+                f.write(details + "\n")
+        else:
+            print(details, file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)), flush=True)
     if world > 1:
         dist.barrier()
         dist.destroy_process_group()
+
+
+def headline(line):
+    """The printed line: the headline's own keys, and one figure of every other
+    section of the full record.  Under 2,000 characters, so that a reader who keeps
+    only the end of the output still has all of it."""
+    def short(v):
+        if isinstance(v, float):
+            return float(f"{v:.6g}")
+        return {k: short(x) for k, x in v.items()} if isinstance(v, dict) else v
+
+    def pick(section, *keys):
+        d = line.get(section)
+        return {k: d[k] for k in keys if k in d} if d else None
+
+    def dig(*path):
+        d = line
+        for k in path:
+            d = d.get(k) if isinstance(d, dict) else None
+        return d
+
+    out = {k: line[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+                                "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "config",
+                                "latency_ms", "split_ms", "lambda2")}
+    out["roofline"] = pick("roofline", "bound", "kernel", "achieved", "peak", "unit", "frac", "traffic")
+    out["cpu_baseline"] = pick("cpu_baseline", "value", "unit", "cores", "kind")
+    out["e2e"] = pick("e2e", "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")
+    out["gpu_launches"] = line["gpu_launches"]
+    out["clocks"] = pick("clocks", "sm_mhz", "sm_max_mhz", "reasons")
+    out["vec_err_vs_oracle"] = dig("accuracy_vs_oracle", "c2_fp64", "vec_rel_err")
+    out["others"] = {"fp32": dig("fp32", "value"), "grid_64x64": dig("c1", "value"),
+                     "batch_fp32": dig("batch", "fp32", "value"),
+                     "serving_fp32": dig("serving", "fp32", "saturation_solves_s"),
+                     "chung_lu_fp32": dig("chung_lu", "fp32", "value"), "unit": UNIT}
+    return short(out)
 
 
 def oracle_checks(args, c2_graph, r64, r32, batch, chung_lu, stream):
@@ -1164,6 +1206,7 @@ def main():
     ap.add_argument("--steps", type=int, default=20)
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", default="cuda", choices=["cuda", "reference"])
+    ap.add_argument("--details", help="write the full record here (default: stderr)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-fp32", action="store_true")
     ap.add_argument("--no-e2e", action="store_true")
