@@ -232,7 +232,7 @@ cmg_status_t cmg_hierarchy_info(cmg_hierarchy_t h, int32_t *levels, int64_t *n_p
  * nullable).  kind_out[j]: 0 = the level in the shared memory (and registers) of
  * one CTA, or, where CMG_CLUSTER is not set, of a small thread-block cluster for a
  * level below 512 rows,
- * 1 = all SMs over the level's items (FP64 levels of up to 65,536 rows) or sweep
+ * 1 = all SMs over the level's items (FP64 levels of up to 2^20 rows) or sweep
  * layout, streamed or held in the SMs' shared memory, 2 = the slice kernel with the
  * iterate's first staged_out[j] entries (its highest-degree rows) copied to
  * shared memory every sweep, 3 = row-tile kernel, 4 = two-phase kernel (a
@@ -246,11 +246,10 @@ cmg_status_t cmg_hierarchy_info(cmg_hierarchy_t h, int32_t *levels, int64_t *n_p
  * stores them into the others' shared memory).  CMG_CLUSTER, read by cmg_setup:
  * 0 keeps every level off clusters, <rows> (at least 128) the levels of fewer rows.
  * cmg_level_forms tells the kernels' forms apart.
- * FP64 levels of up to 65,536 rows sweep in 62-bit fixed point (a graph that is not
+ * FP64 levels of up to 2^20 rows sweep in 63-bit fixed point (a graph that is not
  * checked, validate = 0, only if it keeps the input contract): its noise over the
- * whole vector is below one FP64 rounding of the largest entry.  Larger FP64 levels,
- * levels with a row of more than 4,096 entries and levels whose layout is larger
- * than L2 sweep in FP64.  Staging is chosen at setup where the gathers
+ * whole vector is no more than one FP64 rounding of the largest entry.  Larger FP64 levels
+ * and levels with a row of more than 4,096 entries sweep in FP64.  Staging is chosen at setup where the gathers
  * it serves are several per staged entry and SM; CMG_STAGE=0 (never) or
  * CMG_STAGE=1 (every slice level), read by cmg_setup, overrides that rule and
  * keeps FP64 levels beyond the shared-memory kernels on the slice kernel.
@@ -265,7 +264,8 @@ cmg_status_t cmg_level_kernels(cmg_hierarchy_t h, int32_t *kind_out, int32_t *st
  * with the entries in shared memory, row kernel 2 = streamed, 3 = resident,
  * 4 = resident with the iterate staged every sweep; floating point: 5 = one CTA,
  * slice kernel 6 = unstaged, 7 = staged, 8 = staged with the layout resident,
- * 9 = two-phase, 10 = row tiles.  ctas_out[j]: CTAs of forms 0 to 4, else 0.
+ * 9 = two-phase, 10 = row tiles; 11 = row kernel (fixed point) streamed evict-first.
+ * ctas_out[j]: CTAs of the fixed-point forms, else 0.
  * Errors: INVALID_ARG if h is NULL. */
 cmg_status_t cmg_level_forms(cmg_hierarchy_t h, int32_t *form_out, int32_t *ctas_out);
 

@@ -337,7 +337,7 @@ class Hierarchy:
         return kind.tolist(), staged.tolist()
 
     FORMS = ("fix_registers", "fix_shared", "rows_streamed", "rows_resident", "rows_staged", "one_cta", "slice",
-             "slice_staged", "slice_resident", "two_phase", "tiles")
+             "slice_staged", "slice_resident", "two_phase", "tiles", "rows_evict_first")
 
     def level_forms(self):
         """Per level: the name (FORMS) of the sweep kernel's form, and its CTAs

@@ -321,7 +321,7 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
         CMG_CUDA(cudaStreamSynchronize(s));
     }
     // ---- Alg. 1 Step 1: coarsen while n_i > coarse_size.  Each level runs
-    // HEC, the Galerkin product and the SELL-32 sizing on the device into
+    // HEC and the Galerkin product on the device into
     // buffers sized by upper bounds, then reads its sizes back with one
     // host synchronisation and moves the coarse CSR into exact allocations.
     LevelCounts *cnt_dev;
@@ -473,7 +473,7 @@ static cmg_status_t build_hierarchy(cmg_hierarchy_s *h, int64_t n, const int64_t
             }
             // FP64 levels: the row kernel.  CMG_STAGE (either value) keeps the
             // slice kernel.
-            if (fixed_ok && !L.fp32 && rows_may_hold(L.n, L.nnz) && getenv("CMG_STAGE") == nullptr) {
+            if (fixed_ok && !L.fp32 && rows_may_hold(L.n) && getenv("CMG_STAGE") == nullptr) {
                 size_t lb = 0, rb = 0;
                 CMG_TRY(build_sweep_layout(1, voff1, std::vector<int>{0, L.n}, L.n, L.rp, L.col, L.w, 0, &L.lay, &lb, s,
                                            true));
@@ -849,7 +849,7 @@ cmg_status_t cmg_level_forms(cmg_hierarchy_t h, int32_t *form_out, int32_t *ctas
         } else if (small_level_fits(level_view(L), L.fp32)) {
             form = 5;
         } else if (L.has_rows) {
-            form = !L.rows.resident ? 2 : (L.rows.stage ? 4 : 3);
+            form = !L.rows.resident ? (L.rows.stream ? 11 : 2) : (L.rows.stage ? 4 : 3);
             ctas = L.rows.P;
         } else if (L.has_xl) {
             form = 9;

@@ -236,7 +236,7 @@ constexpr int kFixWarps = 15;
 // us per sweep in FP64 (one CTA up to 512 rows, cluster above), from shared memory
 // (k_power_fix, with three of the four products) and here, the 853-, 239-, 66- and
 // 18-row levels of the 100^3 grid: 3.55 / 2.48 / 1.70 / 1.24, 2.85 / 2.05 / 1.37 /
-// 1.23, and 1.45 / 1.22 / 1.05 / 0.96 (1.29 / 1.07 / 0.95 / 0.87 with three products
+// 1.23, and 1.44 / 1.22 / 1.05 / 0.95 (1.29 / 1.07 / 0.95 / 0.87 with three products
 // and 57 bits: the fourth product and the wider sums are the price of the accuracy
 // stated in fixed.cuh).
 template <int U>
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(32 * (kFixWarps + 1)) k_power_fix_reg(PiArgs a
                     for (int u = 0; u < 4; u++) xv[u] = x[off[u0 + u]];
 #pragma unroll
                     for (int u = 0; u < 4; u++) t.add(xv[u], cf[u0 + u]);
-                    if (u0 == 4 && U > 8) t.fold();
+                    if (u0 == 4 && U > 8) t.carry();
                 }
                 t.carry();
                 const long long pr = t.lanes(lg);
@@ -421,7 +421,9 @@ bool fix_reciprocal(double g, unsigned long long *ginv, int *ge) {
 bool fix_may_hold(int n, long long nnz) { return n >= 2 && n <= kFixMaxN && nnz <= (1 << 20); }
 
 // CTAs of a level: one per kFixCtaWork of its work (an entry counts 1, a row 8),
-// at least what its entries need of shared memory.
+// at least what its entries need of shared memory.  (1,500 and 6,000 give the same
+// times; 12,000, fewer CTAs than a large level's eight, 4.0 us per sweep against 3.3
+// on 4,096 rows and 16K entries and 3.7 against 3.2 on 3,048 rows and 44K entries.)
 constexpr int kFixCtaWork = 3000;
 
 static const void *fix_kernel(const FixPlan &F) {

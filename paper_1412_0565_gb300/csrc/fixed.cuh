@@ -7,32 +7,34 @@
 // of the result exceeds the largest of the iterate, and a common power-of-two
 // scale serves the whole vector.  The FP64 form's sweeps of levels of up to
 // kFixRowsMax rows are therefore run on the integer pipe:
-//   iterate   X = q 2^32 + r   (q, r: signed 32-bit, |X| < 2^62), y = X 2^-64,
-//             rescaled by powers of two so that max |X| stays in [2^61, 2^62)
+//   iterate   X = q 2^32 + r   (q, r: signed 32-bit, |X| < 2^63), y = X 2^-65,
+//             rescaled by powers of two so that max |X| stays in [2^62, 2^63)
 //             (the sweep's own maximum is reduced with its sums);
 //   entries   C_ij = round(w_ij / g 2^60) = c1 2^29 + c0, D_i = sum_j C_ij exactly;
 //   row       X_i + round((sum_j C_ij X_j - D_i X_i) 2^-60), all four products
 //             exact in 64-bit sums, one rounding to nearest per row (the lanes of a
-//             row each cut 2^-24 units before it).  Rows of a constant vector
+//             row each cut a few 2^-24 units before it).  Rows of a constant vector
 //             give 0, so constant vectors are fixed points, and a mean that is
 //             rounded to a whole unit only moves the vector along 1, which the
 //             result's projection takes out.
-// What it costs in accuracy.  The only rounding of a sweep is half a unit of at
-// most 2^-61 max |x| per entry, 0.29 2^-61 sqrt(n) max |x| as a vector; FP64 rounds
-// its largest entry by 0.29 2^-53 to 0.29 2^-52 of it, several times a sweep (and
-// g - d_i, the same in every sweep, by as much).  With sqrt(n) <= 2^8 the noise of the whole vector is no
-// more than that of one FP64 rounding of its largest entry, however localised the
-// vector is: that is where kFixRowsMax lies, and larger levels keep the FP64
-// kernels.  A coefficient is off by 2^-61 g, FP64's diagonal g - d_i by 2^-54 g.
+// What it costs in accuracy.  The only rounding of a sweep is half a unit per entry.
+// With max |x| = m 2^e, 1 <= m < 2, the unit is 2^-62 2^e, and FP64's last place at the
+// largest entry is 2^-52 2^e: the noise of the whole vector, 0.29 sqrt(n) units as a
+// standard deviation, is no more than that of one FP64 rounding of its largest
+// entry, 0.29 last places, while sqrt(n) <= 2^10, however localised the vector is.
+// That is where kFixRowsMax lies; larger levels keep the FP64 kernels.  (FP64 rounds
+// several times a sweep, each entry by its own last place, and g - d_i by as much,
+// the same way in every sweep.)  A coefficient is off by 2^-61 g, FP64's diagonal by
+// 2^-54 g.
 // A CPU model of both forms against 64-bit mantissas, 300 / 2,000 sweeps from one
 // start, error of the vector: Barabasi-Albert graph of 20K vertices from a random
-// start 1.5e-14 / 6.4e-14 (FP64) and 1.6e-16 / 4.2e-16 (here); on a pendant path
-// of ten vertices 1.2e-14 / 3.8e-14 and 5e-17 / 7e-17; 65K vertices 1.8e-14 /
-// 6.6e-14 and 1.1e-16 / 1.5e-16; on one vertex behind an edge of weight 0.01, the
-// form's worst case, 6e-17 / 1.1e-16 and 9e-17 / 1.0e-16 (20K), 5e-17 / 1.1e-16 and
-// 2.0e-16 / 2.4e-16 (65K), where storing the result as doubles costs 1e-16 itself.
-// (With |X| < 2^57 and the products r c0 dropped, the last but one rows read
-// 7e-15 / 9e-15 and the 20K vertex 6e-15 / 6.5e-15: above FP64.)
+// start 1.5e-14 / 6.4e-14 (FP64) and 1.6e-16 / 4.2e-16 (here); on a pendant path of ten
+// vertices 1.2e-14 / 3.8e-14 and 2.7e-17 / 4.3e-17, 65K vertices 1.8e-14 / 6.6e-14 and
+// 5.8e-17 / 8.3e-17; on one vertex behind an edge of weight 0.01, the form's worst case
+// (FP64's roundings there lie along the vector), 20K 6.3e-17 / 1.1e-16 and 4.7e-17 /
+// 5.1e-17, where storing the result as doubles costs 1e-16 itself.  (With 57 bits and
+// the products r c0 dropped: 3.4e-15 / 3.8e-15 on the path, 6.1e-15 / 6.5e-15 on the
+// vertex.)
 // The stop sums (sum y, sum y^2, sum y y_prev) are integers as well, taken from X
 // rounded to 60 bits, and the same in every order of addition.
 #pragma once
@@ -43,7 +45,7 @@ namespace cmg {
 
 // ------------------------------------------------------------------ plan
 constexpr int kFixMaxN = 4096;        // rows of a level k_power_fix takes
-constexpr int kFixRowsMax = 65536;    // rows of a level any fixed-point kernel takes (see above)
+constexpr int kFixRowsMax = 1 << 20;  // rows of a level any fixed-point kernel takes (see above)
 
 // What a plan kernel reports to the host.
 struct PlanOut {
@@ -83,7 +85,7 @@ cmg_status_t launch_plan_small(const SmallJobs &jobs, int count, cudaStream_t s)
 cmg_status_t launch_fill_small(const SmallJobs &jobs, int count, cudaStream_t s);
 
 // ------------------------------------------------------------------ arithmetic
-constexpr int kFixTop = 62;   // |X| < 2^62; y = X 2^-64
+constexpr int kFixTop = 63;   // |X| < 2^63; y = X 2^-65
 
 __device__ __forceinline__ long long mad_s(int a, int b, long long c) {
     long long d;
@@ -123,8 +125,8 @@ __device__ __forceinline__ long long fix_weight(double w, unsigned long long gin
 
 // Accumulators of one lane's part of a row: hi in units of 2^61, m1 of 2^32, m2 of
 // 2^29 and m0 of 1 (of the product X C).  The coefficients of a row and its diagonal
-// add up to at most 2^60, so |hi| < 2^61 and |m2| < 2^62 over any row; m0 takes 15
-// products (below 2^59 each) between folds, m1 30 (below 2^58) between carries.
+// add up to at most 2^60, so |hi| <= 2^62 and |m2| <= 2^62 over any row; m1 and m0 take
+// 15 products (at most 2^59 each) between carries.
 struct FixAcc {
     long long hi, m1, m2, m0;
     __device__ __forceinline__ void reset() { hi = m1 = m2 = m0 = 0; }
@@ -135,13 +137,9 @@ struct FixAcc {
         m0 = mad_s(x.y, c.y, m0);
     }
     // after at most 15 entries
-    __device__ __forceinline__ void fold() {
+    __device__ __forceinline__ void carry() {
         m1 += m0 >> 32;
         m0 &= 0xffffffffll;
-    }
-    // after at most 30 entries
-    __device__ __forceinline__ void carry() {
-        fold();
         hi += m1 >> 29;
         m1 &= (1ll << 29) - 1;
     }
@@ -174,8 +172,7 @@ __device__ __forceinline__ void fix_quads(FixAcc &t, int steps, const IDX *col, 
         for (int j = 0; j < 8; j++) xx[j] = ldx(cc[j]);
 #pragma unroll
         for (int j = 0; j < 8; j++) t.add(xx[j], cf[32 * j]);
-        if (u & 8) t.carry();
-        else t.fold();
+        t.carry();
     }
     if (u < steps) {
         int cc[4];
@@ -197,7 +194,7 @@ __device__ __forceinline__ long long fix_row(long long X, long long p, long long
 }
 
 // Stop sums of the rows a lane computed in one sweep: A in units of X (modulo 2^64:
-// the total is a few units a row), the others of X' = X / 4 rounded, |X'| <= 2^60 =
+// the total is a few units a row), the others of X' = X / 8 rounded, |X'| <= 2^60 =
 // q 2^32 + r: B = Bh 2^64 + Bm 2^37, C = Ch 2^64 + Cm 2^36.  Up to 64 rows fit
 // (q^2 <= 2^56).
 struct FixSum {
@@ -207,7 +204,7 @@ struct FixSum {
         A = Bh = Bm = Ch = Cm = 0;
         mx = 0;
     }
-    static __device__ __forceinline__ int2 narrow(long long X) { return fix_split((X + 2) >> 2); }   // X'
+    static __device__ __forceinline__ int2 narrow(long long X) { return fix_split((X + 4) >> 3); }   // X'
     __device__ __forceinline__ void square(int2 y, int2 q) {
         Bh = mad_s(y.x, y.x, Bh);
         // X'^2 = q^2 2^64 + (q r + r^2 / 2^33) 2^33
@@ -234,7 +231,7 @@ constexpr int kFixSums = 6;   // 64-bit words of a record of sums: five values a
 
 // A lane's sums in five 64-bit values whose totals fit: A, then B as U 2^80 + V 2^37 and
 // C as U 2^80 + V 2^36 (units of X'^2).  A row adds at most 2^40 to a U and a lane
-// 2^44 to a V: 2^22 rows and 2^18 lanes fit (kFixRowsMax rows take at most 2^17).
+// 2^44 to a V: 2^22 rows and 2^18.9 lanes fit (the kernels have at most 2^17.3).
 // start: A's two parts and B.
 struct FixVals {
     long long v[5];
@@ -258,10 +255,10 @@ __device__ __forceinline__ FixVals fix_vals_row(long long Y, int2 y, int2 x) {
     const long long bm = mad_s(y.x, y.y, mad_s(y.y, y.y, 0) >> 33), bh = mad_s(y.x, y.x, bm >> 31);
     const long long cm = mad_s(y.x, x.y, mad_s(y.y, x.x, mad_s(y.y, x.y, 0) >> 32)), ch = mad_s(y.x, x.x, cm >> 32);
     r.v[0] = Y;
-    r.v[1] = bh >> 20;
-    r.v[2] = ((bh & 0xfffff) << 23) + (((unsigned)bm & 0x7fffffffu) >> 8);
-    r.v[3] = ch >> 20;
-    r.v[4] = ((ch & 0xfffff) << 24) + ((unsigned)cm >> 8);
+    r.v[1] = bh >> 22;   // X^2 = 64 X'^2
+    r.v[2] = ((bh & 0x3fffff) << 21) + (((unsigned)bm & 0x7fffffffu) >> 10);
+    r.v[3] = ch >> 22;
+    r.v[4] = ((ch & 0x3fffff) << 22) + ((unsigned)cm >> 10);
     return r;
 }
 
@@ -366,9 +363,9 @@ __device__ __forceinline__ int fix_decide(const PiArgs &a, int lane, long long v
     // mean of the next sweep, predicted: 2^e (mean - M); a few units
     const float m = (float)A * inv_n - (float)c.M;
     const long long Mn = (long long)__float2int_rn(c.e ? ldexpf(m, c.e) : m);
-    // |X_s| < 2^b, so |X_{s+1}| < 2^(b + e_s) (an average, less a mean of a few
-    // units): lift it to 2^62
-    const int en = min(24, max(0, kFixTop - (64 - __clz((int)mx) + c.e)));
+    // |X_s| < (mx + 1) 2^32, and an average, less a mean of a few units, stays below
+    // (mx + 2) 2^32 2^e: lift that to 2^63 (q must stay below 2^31)
+    const int en = min(24, max(0, __clz((int)(mx + 2)) - 1 - c.e));
     c.K = omt2 * t;
     c.Z = t * (double)(c.e ? ldexpf(a.zero_tol2, 2 * c.e) : a.zero_tol2);
     next->M = Mn;
@@ -389,7 +386,7 @@ __device__ __forceinline__ void fix_ctl_start(const PiArgs &a, int lane, long lo
     const double B = __shfl_sync(0xffffffffu, d, 4) + __shfl_sync(0xffffffffu, d, 8);
     const double A = fma(__shfl_sync(0xffffffffu, d, 16), 0x1p20, __shfl_sync(0xffffffffu, d, 0));
     const long long lo = __shfl_sync(0xffffffffu, v, 0), hi = __shfl_sync(0xffffffffu, v, 16);
-    const double mu0 = A * 0x1p-64 / (double)n;
+    const double mu0 = A * 0x1p-65 / (double)n;
     double ss0 = B - (double)n * mu0 * mu0;
     if (ss0 < 0.0) ss0 = 0.0;
     c.B = c.Bp = ss0;
@@ -415,7 +412,7 @@ __device__ __forceinline__ void fix_ctl_start(const PiArgs &a, int lane, long lo
 // the ring slot of sweep rs.  res[0..1]: rs, annihilated.
 __device__ __forceinline__ void fix_finish(const PiArgs &a, int lane, int n, int rs, int code, bool counted, bool bad,
                                            bool writes, int buf, const FixCtl &c, int *res) {
-    const double to_mean = 0x1p-64 / (double)n;
+    const double to_mean = 0x1p-65 / (double)n;
     const double B = __shfl_sync(0xffffffffu, c.B, 4), Bp = __shfl_sync(0xffffffffu, c.Bp, 4);
     if (lane != 0) return;
     const bool zero = code == 2;
@@ -447,11 +444,11 @@ __device__ __forceinline__ void fix_finish(const PiArgs &a, int lane, int n, int
 }
 
 __device__ __forceinline__ double fix_value(int2 x) {
-    return fma((double)x.x, 0x1p32, (double)x.y) * 0x1p-64;
+    return fma((double)x.x, 0x1p32, (double)x.y) * 0x1p-65;
 }
 
 // The exponent k that scales a start vector of largest magnitude m (finite,
-// > 0) to |x| 2^k in [2^60, 2^61): the first sweep subtracts a mean of that size.
+// > 0) to |x| 2^k in [2^61, 2^62): the first sweep subtracts a mean of that size.
 __device__ __forceinline__ int fix_start_exponent(double m) {
     int ex;
     frexp(m, &ex);   // m = f 2^ex, f in [0.5, 1)

@@ -193,20 +193,22 @@ inline bool partial_stage_pays(unsigned long long below, long long entries, int 
 struct RowPlan {
     int P = 0, threads = 0;     // CTAs and threads of the launch
     int ni = 0;                 // items
+    int col16 = 1;
     int resident = 0;           // the matrix stays in shared memory for the launch
     int stage = 0;              // ... and the iterate is copied there every sweep
+    int stream = 0;             // streaming form: read evict-first
     size_t smem = 0;
     int res_e = 0, res_i = 0, res_r = 0;   // most entries, items, rows of a CTA
     long long entries = 0;
     int4 *item = nullptr;       // [ni + 1] first row, first entry, steps, log2 lanes | rows << 3
     int *range = nullptr;       // [P + 1] first item of each CTA
-    uint16_t *ucol = nullptr;   // columns, coefficients and diagonal
+    void *ucol = nullptr;       // columns (uint16 or int32), coefficients and diagonal
     int2 *uc = nullptr, *ud = nullptr;
     long long *acc = nullptr;   // the CTAs' stop sums
 };
-// Whether the row kernel may take a level: at most kFixRowsMax (65,536) rows, the line
-// of the fixed point's accuracy (fixed.cuh), and a layout that stays in L2.
-bool rows_may_hold(int n, long long nnz);
+// Whether the row kernel may take a level: at most kFixRowsMax (2^20) rows, the line of
+// the fixed point's accuracy (fixed.cuh).
+bool rows_may_hold(int n);
 // Builds it from the level's CSR and the row order (L.perm / L.inv).
 // CMG_ERR_TOO_LARGE: the level is left to the slice kernel (a row of more than
 // 4,096 entries, which one warp would hold up, or more than 64 items a warp).

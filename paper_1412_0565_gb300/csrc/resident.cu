@@ -12,13 +12,20 @@ namespace cmg {
 // Lanes per row by row length: steps of at most S entries per lane while the row
 // fits a warp, S = 8 on levels with at most kWideEntries entries per SM (a sweep
 // there is a chain of latencies: a row of 16 entries on one lane is two rounds of
-// gathers, on two lanes one) and 16 above, where the instructions are the bound
-// and every split row costs extra sums.
+// gathers, on two lanes one; S = 16 takes 4.15 us per sweep on 10K rows and 153K
+// entries where S = 8 takes 3.40, and 4.7 on 15K rows and 93K entries against 4.2)
+// and 16 above, where the instructions are the bound and every split row costs
+// extra sums.
 constexpr int kWideEntries = 8192;
-constexpr int kItemCost = 256;     // per item, in entries: the rows' finish and stop sums
+// Cost of an item beside its entries, in entries: the rows' finish and stop sums.
+// (5,047 rows and 23K entries 3.3 us per sweep; with 64 4.5, the CTAs too few; with
+// 1,024 the same there, 45K rows and 354K entries 5.9 against 5.6.)
+constexpr int kItemCost = 256;
 // Work of one CTA at least, in entries (an item counts kItemCost): below it more
 // CTAs make the barrier dearer and the rows no faster, and leave no SM to the
-// other streams of a server.
+// other streams of a server.  (1,024: within 3 % either way on levels of 1.5K to
+// 45K rows; 4,096: 4.5 us per sweep against 3.3 on the 5,047 rows; 8,192: 6.8 against
+// 4.5 on 20K rows and 160K entries.)
 constexpr int kCtaWork = 2048;
 constexpr int kPlanThreads = 1024;
 constexpr int kStreamThreads = 384;   // two CTAs per SM with 85 registers a thread
@@ -171,9 +178,9 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_units(int n, const int *_
 
 // Entries and diagonal of one item in fixed point (one warp); short rows and
 // missing rows are padded with coefficient 0 and a valid column.
-template <typename PERM, typename INV>
+template <typename PERM, typename INV, typename IDX>
 __device__ __forceinline__ void fill_item(int4 it, int lane, const int *rp, const int *col, const double *w,
-                                          unsigned long long ginv, int ge, const PERM *perm, const INV *inv, uint16_t *ucol,
+                                          unsigned long long ginv, int ge, const PERM *perm, const INV *inv, IDX *ucol,
                                           int2 *uc, int2 *ud) {
     const int lg = it.w & 7, rows = it.w >> 3, r = lane >> lg, g = lane & ((1 << lg) - 1);
     const int p = it.x + (r < rows ? r : 0);
@@ -193,7 +200,7 @@ __device__ __forceinline__ void fill_item(int4 it, int lane, const int *rp, cons
             Cij = fix_weight(w[e0 + k], ginv, ge);
             cl = (int)inv[col[e0 + k]];
         }
-        ucol[d] = (uint16_t)cl;
+        ucol[d] = (IDX)cl;
         uc[d] = fix_split_c(Cij);
         sum += Cij;
     }
@@ -294,9 +301,10 @@ __global__ void k_fill_small(const __grid_constant__ SmallJobs jobs) {
         fill_item(J.item[u], lane, J.rp, J.col, J.w, J.ginv, J.ge, J.perm, J.inv, J.ucol, J.uc, J.ud);
 }
 
+template <typename IDX>
 __global__ void k_fill_units(int ni, const int4 *__restrict__ item, const int *__restrict__ rp,
                              const int *__restrict__ col, const double *__restrict__ w, unsigned long long ginv, int ge,
-                             const uint32_t *__restrict__ perm, const int *__restrict__ inv, uint16_t *__restrict__ ucol,
+                             const uint32_t *__restrict__ perm, const int *__restrict__ inv, IDX *__restrict__ ucol,
                              int2 *__restrict__ uc, int2 *__restrict__ ud) {
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
@@ -328,9 +336,10 @@ constexpr int kFixAccWords = 3 * kFixRec + 8;
 // coefficients and own row in flight together, the next item's descriptor too.
 // us per sweep: slice kernel in FP64, this kernel in FP64, in fixed point: 1,542 rows
 // and 103K entries 17.3, 6.3, 4.0; 5,688 rows and 129K entries 16.0, 6.6, 4.4; 20K
-// rows and 160K entries 16.0, 5.0, 4.4; the 100^3 grid's 35K- and 10K-row levels
-// 9.4 / 8.3, 6.9 / 4.8, and 5.5 / 3.5.
-template <bool RES, bool STAGE>
+// rows and 160K entries 16.0, 5.0, 3.6; the 100^3 grid's levels of 1M, 348K, 114K, 35K
+// and 10K rows 40.4 / 23.6 / 14.7 / 9.4 / 8.3, 38.0 / 22.5 / 11.3 / 6.9 / 4.8, and
+// 24.8 / 19.9 / 9.5 / 5.1 / 3.5.
+template <typename IDX, bool RES, bool STAGE, bool STREAM>
 __global__ void __launch_bounds__(RES ? 1024 : kStreamThreads, RES ? 1 : 2) k_power_rows(PiArgs a, GridSync *gs) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(16) long long s_pw[32][kFixSums];   // the warps' sums
@@ -350,14 +359,14 @@ __global__ void __launch_bounds__(RES ? 1024 : kStreamThreads, RES ? 1 : 2) k_po
     int2 *s_w = reinterpret_cast<int2 *>(s_item + a.res_items);
     int2 *s_x = s_w + a.res_entries;
     int2 *s_d = s_x + (STAGE ? ((n + 1) & ~1) : 0);
-    uint16_t *s_c = reinterpret_cast<uint16_t *>(s_d + ((a.res_rows + 1) & ~1));
+    IDX *s_c = reinterpret_cast<IDX *>(s_d + ((a.res_rows + 1) & ~1));
     if (RES) {
         const int2 *gw = reinterpret_cast<const int2 *>(a.lay_w) + e_lo;
-        const uint16_t *gc = reinterpret_cast<const uint16_t *>(a.lay_col) + e_lo;
+        const IDX *gc = reinterpret_cast<const IDX *>(a.lay_col) + e_lo;
         const int ne = last.y - e_lo;   // a multiple of 32: 16-byte copies
         for (int k = tid; k < ne / 2; k += blockDim.x)
             reinterpret_cast<uint4 *>(s_w)[k] = __ldg(reinterpret_cast<const uint4 *>(gw) + k);
-        for (int k = tid; k < ne / 8; k += blockDim.x)
+        for (int k = tid; k < ne * (int)sizeof(IDX) / 16; k += blockDim.x)
             reinterpret_cast<uint4 *>(s_c)[k] = __ldg(reinterpret_cast<const uint4 *>(gc) + k);
         for (int k = tid; k < r1 - r0; k += blockDim.x) s_d[k] = __ldg(a.fix_d + r0 + k);
         for (int k = tid; k < ie - ib; k += blockDim.x) {
@@ -366,7 +375,7 @@ __global__ void __launch_bounds__(RES ? 1024 : kStreamThreads, RES ? 1 : 2) k_po
             s_item[k] = it;
         }
     }
-    const uint16_t *C = RES ? s_c : reinterpret_cast<const uint16_t *>(a.lay_col);
+    const IDX *C = RES ? s_c : reinterpret_cast<const IDX *>(a.lay_col);
     const int2 *W = RES ? s_w : reinterpret_cast<const int2 *>(a.lay_w);
     unsigned long long *const acc = reinterpret_cast<unsigned long long *>(a.fix_acc);
     // the records of the warps from `first_warp` on, added to record k
@@ -530,8 +539,8 @@ __global__ void __launch_bounds__(RES ? 1024 : kStreamThreads, RES ? 1 : 2) k_po
                             ww[u] = make_int2(0, 0);
                             if (t0 + u < it.z) {
                                 const int e = base + 32 * (t0 + u);
-                                cc[u] = (int)C[e];
-                                ww[u] = W[e];
+                                cc[u] = (int)(STREAM ? __ldcs(C + e) : C[e]);
+                                ww[u] = STREAM ? __ldcs(W + e) : W[e];
                             }
                         }
 #pragma unroll
@@ -574,9 +583,18 @@ __global__ void __launch_bounds__(RES ? 1024 : kStreamThreads, RES ? 1 : 2) k_po
     }
 }
 
+// (a staged iterate fits only where columns have 16 bits)
 static const void *rows_kernel(const RowPlan &R) {
-    if (!R.resident) return (const void *)k_power_rows<false, false>;
-    return R.stage ? (const void *)k_power_rows<true, true> : (const void *)k_power_rows<true, false>;
+    if (R.resident) {
+        if (R.stage) return (const void *)k_power_rows<uint16_t, true, true, false>;
+        return R.col16 ? (const void *)k_power_rows<uint16_t, true, false, false>
+                       : (const void *)k_power_rows<int, true, false, false>;
+    }
+    if (R.stream)
+        return R.col16 ? (const void *)k_power_rows<uint16_t, false, false, true>
+                       : (const void *)k_power_rows<int, false, false, true>;
+    return R.col16 ? (const void *)k_power_rows<uint16_t, false, false, false>
+                   : (const void *)k_power_rows<int, false, false, false>;
 }
 
 cmg_status_t launch_fill_small(const SmallJobs &jobs, int count, cudaStream_t s) {
@@ -589,8 +607,8 @@ cmg_status_t launch_plan_small(const SmallJobs &jobs, int count, cudaStream_t s)
     return launch_status();
 }
 
-static size_t rows_smem(int n, int stage, const PlanOut &o) {
-    return 16 * (size_t)o.max_i + 10 * (size_t)o.max_e + (stage ? 8 * (size_t)((n + 1) & ~1) : 0) +
+static size_t rows_smem(int n, int col16, int stage, const PlanOut &o) {
+    return 16 * (size_t)o.max_i + (col16 ? 10 : 12) * (size_t)o.max_e + (stage ? 8 * (size_t)((n + 1) & ~1) : 0) +
            8 * (size_t)((o.max_r + 1) & ~1) + 16;
 }
 
@@ -612,24 +630,23 @@ static cmg_status_t rows_choose(int n, const PlanOut &o, RowPlan *R) {
     size_t room = 0;
     CMG_TRY(rows_room(*R, &room));
     R->resident = R->stage = 0;
-    if (rows_smem(n, 0, o) > room) return CMG_OK;
+    if (rows_smem(n, R->col16, 0, o) > room) return CMG_OK;
     R->resident = 1;
     // staging the iterate costs one trip to L2 and n / 8 cycles of copying per
     // SM; a scattered gather costs about 1.4 cycles more from L1 or L2 than from
-    // shared memory
-    if (rows_smem(n, 1, o) <= room && (long long)n / 8 + 800 < (long long)o.max_e) R->stage = 1;
+    // shared memory.  (us per sweep unstaged and staged: 1,542 rows and 103K entries
+    // 5.1 and 4.0, 5,688 rows and 129K entries 5.3 and 4.3, which the rule stages;
+    // 5,047 rows and 23K entries 3.3 and 4.4, 10K and 153K 3.4 and 5.2, 20K and
+    // 160K 4.5 and 5.7, which it does not.)
+    if (R->col16 && rows_smem(n, 1, 1, o) <= room && (long long)n / 8 + 800 < (long long)o.max_e) R->stage = 1;
     R->res_e = o.max_e;
     R->res_i = o.max_i;
     R->res_r = o.max_r;
-    R->smem = rows_smem(n, R->stage, o);
+    R->smem = rows_smem(n, R->col16, R->stage, o);
     return CMG_OK;
 }
 
-bool rows_may_hold(int n, long long nnz) {
-    DeviceInfo d;
-    if (device_info(&d) != CMG_OK) return false;
-    return n <= kFixRowsMax && (d.l2_bytes <= 0 || 10 * nnz <= (long long)d.l2_bytes);
-}
+bool rows_may_hold(int n) { return n <= kFixRowsMax; }
 
 cmg_status_t build_row_plan(int n, long long nnz, const int *rp, const int *col, const double *w, double g,
                             const SweepLayout &L, RowPlan *R, size_t *bytes, cudaStream_t s) {
@@ -638,6 +655,7 @@ cmg_status_t build_row_plan(int n, long long nnz, const int *rp, const int *col,
     if (!fix_reciprocal(g, &ginv, &ge)) return CMG_ERR_TOO_LARGE;
     DeviceInfo di;
     CMG_TRY(device_info(&di));
+    R->col16 = n <= 65536 ? 1 : 0;
     Scratch scr(s);
     PlanOut *out_dev, o;
     CMG_TRY(scr.get(&out_dev, 1));
@@ -661,6 +679,8 @@ cmg_status_t build_row_plan(int n, long long nnz, const int *rp, const int *col,
     R->threads = std::max(R->stage ? 512 : 64, 32 * (1 + std::min(31, std::max(1, o.max_i))));
     if (!R->resident) {
         CMG_TRY(plan(2 * di.sms, 0));
+        // only a layout that cannot stay in L2 is read evict-first
+        R->stream = di.l2_bytes > 0 && o.entries * (R->col16 ? 10ll : 12ll) > (long long)di.l2_bytes;
         R->threads = kStreamThreads;
     }
     // a lane adds at most this many rows' sums
@@ -671,14 +691,18 @@ cmg_status_t build_row_plan(int n, long long nnz, const int *rp, const int *col,
     CMG_TRY(dev_alloc_n(&R->item, (size_t)o.ni + 1, s));
     CMG_CUDA(cudaMemcpyAsync(R->item, item, sizeof(int4) * ((size_t)o.ni + 1), cudaMemcpyDeviceToDevice, s));
     const size_t ne = (size_t)std::max<long long>(o.entries, 1);
-    CMG_TRY(dev_alloc_n(&R->ucol, ne, s));
+    CMG_TRY(dev_alloc(&R->ucol, ne * (R->col16 ? 2 : 4), s));
     CMG_TRY(dev_alloc_n(&R->uc, ne, s));
     CMG_TRY(dev_alloc_n(&R->ud, (size_t)n, s));
     CMG_TRY(dev_alloc_n(&R->acc, (size_t)kFixAccWords, s));
     const int fb = grid_for(32ll * o.ni, 256);
-    k_fill_units<<<fb, 256, 0, s>>>(o.ni, R->item, rp, col, w, ginv, ge, L.perm, L.inv, R->ucol, R->uc, R->ud);
+    if (R->col16)
+        k_fill_units<<<fb, 256, 0, s>>>(o.ni, R->item, rp, col, w, ginv, ge, L.perm, L.inv, (uint16_t *)R->ucol, R->uc,
+                                        R->ud);
+    else
+        k_fill_units<<<fb, 256, 0, s>>>(o.ni, R->item, rp, col, w, ginv, ge, L.perm, L.inv, (int *)R->ucol, R->uc, R->ud);
     CMG_TRY(launch_status());
-    *bytes += 16 * ((size_t)o.ni + 1) + 4 * ((size_t)2 * di.sms + 1) + 10 * ne +
+    *bytes += 16 * ((size_t)o.ni + 1) + 4 * ((size_t)2 * di.sms + 1) + ne * (size_t)(R->col16 ? 10 : 12) +
               8 * (size_t)n + 8 * kFixAccWords;
     return CMG_OK;
 }

@@ -25,15 +25,20 @@ CASES = {
     "resident": (lambda: inputs.grid2d(100, 101, "uniform", seed=2), "rows_resident", {}),
     "resident_edges_odd": (lambda: ladder(60002, EDGES + [7, 3], 2), "rows_resident", {}),
     "resident_longest_row": (lambda: ladder(60000, [4090, 2000], 3), "rows_resident", {}),
-    "resident_most_rows": (lambda: ladder(65533, [40, 50, 60], 5), "rows_resident", {}),
+    "resident_most_16_bit_columns": (lambda: ladder(65533, [40, 50, 60], 5), "rows_resident", {}),
+    "resident_32_bit_columns": (lambda: ladder(65534, [40, 50, 60], 5), "rows_resident", {}),
     "staged_edges": (lambda: ladder(6000, EDGES, 1), "rows_staged", {}),
     "staged_edges_odd": (lambda: ladder(6002, EDGES + [7, 3], 2), "rows_staged", {}),
     "staged_longest_row": (lambda: ladder(9000, [4090, 2000], 3), "rows_staged", {}),
     "staged": (lambda: inputs.random_connected(3000, 150000, seed=6), "rows_staged", {}),
     "staged_odd": (lambda: inputs.random_connected(3001, 150000, seed=7), "rows_staged", {}),
     "streamed": (lambda: inputs.random_connected(60001, 1900000, seed=8), "rows_streamed", {}),
+    "streamed_32_bit_columns": (lambda: inputs.grid3d(70, 71, 72, "uniform", seed=9), "rows_streamed", {}),
+    "streamed_most_rows": (lambda: ladder((1 << 20) - 3, [40, 50, 60], 5), "rows_streamed", {}),
+    "evict_first": (lambda: inputs.random_connected(60001, 7300000, seed=10), "rows_evict_first", {}),
+    "evict_first_32_bit_columns": (lambda: inputs.random_connected(70001, 6300000, seed=11), "rows_evict_first", {}),
     "row_too_long": (lambda: ladder(9000, [4200], 4), "slice", {}),
-    "one_row_too_many": (lambda: ladder(65534, [40, 50, 60], 5), "slice", {}),
+    "one_row_too_many": (lambda: ladder((1 << 20) - 2, [40, 50, 60], 5), "slice", {}),
     "slice_by_choice": (lambda: ladder(6000, EDGES, 1), "slice", {"CMG_STAGE": "0"}),
     "staged_slice_by_choice": (lambda: ladder(6000, EDGES, 1), "slice_staged", {"CMG_STAGE": "1"}),
 }

@@ -37,7 +37,7 @@ def sweeps(rp, col, w, g, x, k):
 
 
 @pytest.mark.parametrize("tail,weight", [(10, 1.0), (1, 0.01)])
-@pytest.mark.parametrize("n", [600, 3000, 20000, 60000])
+@pytest.mark.parametrize("n", [600, 3000, 20000, 60000, 250000])
 def test_localised_vectors_keep_fp64_accuracy(n, tail, weight):
     k = 100
     rp, col, w = with_tail(n, tail, weight, seed=n)
