@@ -135,14 +135,15 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
-PROFILES = {"fp64": os.path.join(ROOT, "profiles", "k_power_sell_f64_grid3d_100_level0.md"),
+PROFILES = {"fp64": os.path.join(ROOT, "profiles", "k_power_rows_grid3d_100_level0.md"),
             "fp32": os.path.join(ROOT, "profiles", "k_power_sell_f32_grid3d_100_level0.md")}
 NOMINAL_HBM_GBS = 7900.0   # GB300 HBM3e nominal bandwidth (context beside the measured copy peak)
 # FP64 pipe: 2 FMA per SM per clock (the nominal 1.25 TFLOP/s of a 152-SM GB300 at 2.07 GHz)
 FP64_FMA_PER_SM_CLK = 2
 SMS = 152
 PROFILED_SOURCES = [os.path.join(ROOT, "paper_1412_0565_gb300", "csrc", f)
-                    for f in ("refine.cu", "pi_common.cuh", "ffloat.cuh")]
+                    for f in ("refine.cu", "resident.cu", "fixed.cuh", "pi_kernels.cuh", "pi_common.cuh",
+                              "ffloat.cuh", "common.cuh")]
 
 
 def kernel_fingerprint():
@@ -400,10 +401,11 @@ def run_gpu(args):
         return ms0, by0, tot_b, tot_ms, st0
 
     def roofline(r, fp32):
-        """The dominant kernel: the level-0 power-iteration launch, against the
-        HBM copy peak.  FP64 sweeps run in fixed point on the integer pipe, so
-        the FP64 pipe does not bound them; their FP64-equivalent rate is given
-        beside it."""
+        """The dominant kernel of the level-0 power iteration, against the HBM copy
+        peak.  FP64 levels of up to 2^20 rows sweep in fixed point on the integer
+        pipe: neither memory nor a pipe is near its limit there, a warp waits for
+        two dependent trips to L2 per item ("latency"); their FP64-equivalent rate
+        is given beside it.  FP32 sweeps stream from L2."""
         ms0, by0, tot_b, tot_ms, st0 = level0(r, fp32)
         n0, nnz0, k0 = st0["n"][0], st0["nnz"][0], st0["sweeps"][0]
         gbs = by0 / (ms0 * 1e-3) / 1e9
@@ -424,7 +426,7 @@ def run_gpu(args):
         flops = k0 * sweep_flops_fp64(n0, nnz0)
         peak_tf = FP64_FMA_PER_SM_CLK * 2 * SMS * sm_mhz * 1e6 / 1e12
         tf = flops / (ms0 * 1e-3) / 1e12
-        return dict({"bound": "hbm", "kernel": "k_power_rows<int>, level-0 launch"}, **hbm,
+        return dict({"bound": "latency", "kernel": "k_power_rows<int> (fixed point), level-0 launch"}, **hbm,
                     fp64_equivalent={"achieved": tf, "fp64_pipe_peak": peak_tf, "unit": "TFLOP/s",
                                      "flops_per_launch": flops}, **common)
 
@@ -509,9 +511,9 @@ def run_gpu(args):
             "warmup": max(3, args.warmup), "ms_per_step": r64["ms_per_step"],
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
             "dtype": "f64",
-            "dtype_note": "f64 sweeps, f64 Rayleigh quotient and residual; the stop cosine, mean and norm "
-                          "sums in float-float (about 48 bits: the 1 - 1e-8 cosine test is resolved to "
-                          "about 1e-14)",
+            "dtype_note": "f64 form: sweeps in 63-bit fixed point on levels of up to 2^20 rows (f64 above), "
+                          "f64 Rayleigh quotient and residual; the stop cosine, mean and norm sums exact "
+                          "integers on the fixed-point levels, float-float elsewhere",
             "data": "synthetic",
             "config": config(world),
             "latency_ms": {"p50": r64["p50_ms"], "p99": r64["p99_ms"]},

@@ -422,7 +422,7 @@ bool fix_may_hold(int n, long long nnz) { return n >= 2 && n <= kFixMaxN && nnz 
 
 // CTAs of a level: one per kFixCtaWork of its work (an entry counts 1, a row 8),
 // at least what its entries need of shared memory.  (1,500 and 6,000 give the same
-// times; 12,000, fewer CTAs than a large level's eight, 4.0 us per sweep against 3.3
+// times; 12,000, fewer CTAs than a large level's eight, 3.9 us per sweep against 3.4
 // on 4,096 rows and 16K entries and 3.7 against 3.2 on 3,048 rows and 44K entries.)
 constexpr int kFixCtaWork = 3000;
 

@@ -30,9 +30,10 @@
 // start, error of the vector: Barabasi-Albert graph of 20K vertices from a random
 // start 1.5e-14 / 6.4e-14 (FP64) and 1.6e-16 / 4.2e-16 (here); on a pendant path of ten
 // vertices 1.2e-14 / 3.8e-14 and 2.7e-17 / 4.3e-17, 65K vertices 1.8e-14 / 6.6e-14 and
-// 5.8e-17 / 8.3e-17; on one vertex behind an edge of weight 0.01, the form's worst case
-// (FP64's roundings there lie along the vector), 20K 6.3e-17 / 1.1e-16 and 4.7e-17 /
-// 5.1e-17, where storing the result as doubles costs 1e-16 itself.  (With 57 bits and
+// 5.8e-17 / 8.3e-17; on one vertex behind an edge of weight 0.01, the one kind where
+// FP64 can be closer (its roundings there lie along the vector), 20K 6.3e-17 / 1.1e-16
+// and 4.7e-17 / 5.1e-17, 300 sweeps on 250K 3.1e-17 and 2.2e-16, on 1M 2.4e-17 and
+// 5.1e-16: no more than the roundings of the result itself.  (With 57 bits and
 // the products r c0 dropped: 3.4e-15 / 3.8e-15 on the path, 6.1e-15 / 6.5e-15 on the
 // vertex.)
 // The stop sums (sum y, sum y^2, sum y y_prev) are integers as well, taken from X

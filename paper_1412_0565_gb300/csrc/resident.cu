@@ -12,20 +12,18 @@ namespace cmg {
 // Lanes per row by row length: steps of at most S entries per lane while the row
 // fits a warp, S = 8 on levels with at most kWideEntries entries per SM (a sweep
 // there is a chain of latencies: a row of 16 entries on one lane is two rounds of
-// gathers, on two lanes one; S = 16 takes 4.15 us per sweep on 10K rows and 153K
-// entries where S = 8 takes 3.40, and 4.7 on 15K rows and 93K entries against 4.2)
-// and 16 above, where the instructions are the bound and every split row costs
-// extra sums.
+// gathers, on two lanes one) and 16 above, where the instructions are the bound and
+// every split row costs extra sums.  us per sweep, S = 8 and 16: 15K rows and 93K
+// entries 4.1 and 4.3, 10K and 153K 3.5 and 3.65; 114K and 1.5M 11.2 and 9.5.
 constexpr int kWideEntries = 8192;
 // Cost of an item beside its entries, in entries: the rows' finish and stop sums.
-// (5,047 rows and 23K entries 3.3 us per sweep; with 64 4.5, the CTAs too few; with
-// 1,024 the same there, 45K rows and 354K entries 5.9 against 5.6.)
+// (64: 4.4 us per sweep against 3.4 on 5,047 rows and 23K entries, the CTAs too few;
+// 1,024: 10.7 against 9.5 on 114K rows and 1.5M entries.)
 constexpr int kItemCost = 256;
 // Work of one CTA at least, in entries (an item counts kItemCost): below it more
 // CTAs make the barrier dearer and the rows no faster, and leave no SM to the
-// other streams of a server.  (1,024: within 3 % either way on levels of 1.5K to
-// 45K rows; 4,096: 4.5 us per sweep against 3.3 on the 5,047 rows; 8,192: 6.8 against
-// 4.5 on 20K rows and 160K entries.)
+// other streams of a server.  (1,024: the same times; 4,096: 4.4 us per sweep against
+// 3.4 on 5,047 rows and 23K entries; 8,192: 6.4 against 3.7 on 20K rows and 160K.)
 constexpr int kCtaWork = 2048;
 constexpr int kPlanThreads = 1024;
 constexpr int kStreamThreads = 384;   // two CTAs per SM with 85 registers a thread
@@ -635,9 +633,8 @@ static cmg_status_t rows_choose(int n, const PlanOut &o, RowPlan *R) {
     // staging the iterate costs one trip to L2 and n / 8 cycles of copying per
     // SM; a scattered gather costs about 1.4 cycles more from L1 or L2 than from
     // shared memory.  (us per sweep unstaged and staged: 1,542 rows and 103K entries
-    // 5.1 and 4.0, 5,688 rows and 129K entries 5.3 and 4.3, which the rule stages;
-    // 5,047 rows and 23K entries 3.3 and 4.4, 10K and 153K 3.4 and 5.2, 20K and
-    // 160K 4.5 and 5.7, which it does not.)
+    // 4.1 and 4.0, 5,688 and 129K 4.1 and 4.4, which the rule stages; 5,047 and 23K 3.4
+    // and 4.3, 10K and 153K 3.5 and 5.2, 20K and 160K 3.7 and 5.9, which it does not.)
     if (R->col16 && rows_smem(n, 1, 1, o) <= room && (long long)n / 8 + 800 < (long long)o.max_e) R->stage = 1;
     R->res_e = o.max_e;
     R->res_i = o.max_i;
