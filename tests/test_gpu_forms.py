@@ -4,7 +4,7 @@ the lines of their plans, the levels that leave them, and the FP32 slice kernel
 with its layout resident.
 
 Bars on the vector after k sweeps.  Fixed point: three FP64 roundings of the
-result's entries and two of its scale, and half a unit of 2^-61 of the largest entry per row and sweep (0.29 of
+result's entries and two of its scale, and half a unit of 2^-62 of the largest entry per row and sweep (0.29 of
 one as a standard deviation, times two).  FP64 kernels: 2^-52 of the vector for
 each of four roundings a sweep, and the same again for the rows' sums."""
 import numpy as np
@@ -68,7 +68,7 @@ def test_each_form_runs_where_it_is_named(monkeypatch, name):
     if form.startswith("slice"):
         bar = 8 * 2.0 ** -52 * K
     else:
-        bar = 5 * 2.0 ** -53 + 2 * 0.29 * 2.0 ** -61 * np.sqrt(K * n) * float(np.abs(ref).max()) * np.sqrt(K)
+        bar = 5 * 2.0 ** -53 + 2 * 0.29 * 2.0 ** -62 * np.sqrt(K * n) * float(np.abs(ref).max()) * np.sqrt(K)
     assert err <= bar
 
 

@@ -4,7 +4,7 @@ so this is where it can fall behind FP64, whose units follow each entry.
 
 Reference: the same sweeps in extended precision.  Bar on the vector: the
 result's own three FP64 roundings of its largest entry (the mean, the scale, the
-store), and the sweeps' roundings of half a unit of 2^-61 of the largest entry
+store), and the sweeps' roundings of half a unit of 2^-62 of the largest entry
 per row, 0.29 of one as a standard deviation, added up undamped over the sweeps
 with their standard deviation times two."""
 import numpy as np
@@ -53,4 +53,4 @@ def test_localised_vectors_keep_fp64_accuracy(n, tail, weight):
     if (u * ref).sum() < 0:
         u = -u
     err = float(np.sqrt(((u - ref) ** 2).sum()))
-    assert err <= 3 * 2.0 ** -53 + 2 * 0.29 * 2.0 ** -61 * np.sqrt(k * N)
+    assert err <= 3 * 2.0 ** -53 + 2 * 0.29 * 2.0 ** -62 * np.sqrt(k * N)
