@@ -231,8 +231,7 @@ cmg_status_t cmg_hierarchy_info(cmg_hierarchy_t h, int32_t *levels, int64_t *n_p
 /* Sweep kernel that runs Alg. 3 on each level (host arrays of length >= levels,
  * nullable).  kind_out[j]: 0 = the level in the shared memory (and registers) of
  * one CTA, or, where CMG_CLUSTER is not set, of a small thread-block cluster for a
- * level below 512 rows,
- * 1 = all SMs over the level's items (FP64 levels of up to 2^20 rows) or sweep
+ * level below 512 rows, 1 = all SMs over the level's items (FP64 levels of up to 2^20 rows) or sweep
  * layout, streamed or held in the SMs' shared memory, 2 = the slice kernel with the
  * iterate's first staged_out[j] entries (its highest-degree rows) copied to
  * shared memory every sweep, 3 = row-tile kernel, 4 = two-phase kernel (a
@@ -247,11 +246,11 @@ cmg_status_t cmg_hierarchy_info(cmg_hierarchy_t h, int32_t *levels, int64_t *n_p
  * 0 keeps every level off clusters, <rows> (at least 128) the levels of fewer rows.
  * cmg_level_forms tells the kernels' forms apart.
  * FP64 levels of up to 2^20 rows sweep in 63-bit fixed point (a graph that is not
- * checked, validate = 0, only if it keeps the input contract): its noise over the
- * whole vector is no more than one FP64 rounding of the largest entry.  Larger FP64 levels
- * and levels with a row of more than 4,096 entries sweep in FP64.  Staging is chosen at setup where the gathers
- * it serves are several per staged entry and SM; CMG_STAGE=0 (never) or
- * CMG_STAGE=1 (every slice level), read by cmg_setup, overrides that rule and
+ * checked, validate = 0, only if it keeps the input contract): a sweep's noise over
+ * the whole vector is no more than one FP64 rounding of the largest entry.  Larger
+ * FP64 levels and levels with a row of more than 4,096 entries sweep in FP64.
+ * Staging is chosen at setup where the gathers it serves are several per staged
+ * entry and SM; CMG_STAGE=0 (never) or CMG_STAGE=1 (every slice level), read by cmg_setup, overrides that rule and
  * keeps FP64 levels beyond the shared-memory kernels on the slice kernel.
  * Results do not depend on the kernel beyond rounding; every kernel sums in
  * a fixed order (or exactly), so repeated solves are bit-identical.

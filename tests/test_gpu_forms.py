@@ -4,8 +4,8 @@ the lines of their plans, the levels that leave them, and the FP32 slice kernel
 with its layout resident.
 
 Bars on the vector after k sweeps.  Fixed point: three FP64 roundings of the
-result's entries and two of its scale, and half a unit of 2^-62 of the largest entry per row and sweep (0.29 of
-one as a standard deviation, times two).  FP64 kernels: 2^-52 of the vector for
+result's entries and two of its scale, and half a unit of 2^-62 of the largest
+entry per row and sweep (0.29 of one as a standard deviation, times two).  FP64 kernels: 2^-52 of the vector for
 each of four roundings a sweep, and the same again for the rows' sums."""
 import numpy as np
 import pytest
